@@ -753,8 +753,8 @@ def main():
     if rank == 0 and not args.no_serving and not variant:
         try:
             serve = serving(T, scenes, torch, np)
-            # the same requests with the Chebyshev refinements of concurrent
-            # requests batched into persistent kernels
+            # the same requests with the solves of concurrent requests batched
+            # into persistent kernels
             bat = serving(T, scenes, torch, np, batch_solves=True, plain=False)
             serve["batched_refinements_on"] = {k: bat[k] for k in (
                 "saturation_scenes_per_s", "scenes_per_s", "p50_ms", "p99_ms", "max_ms", "all_converged",
@@ -767,10 +767,12 @@ def main():
             dist.destroy_process_group()
         return
 
-    # ---- roofline of the dominant kernel: the Chebyshev step of the inner
-    # iterations (q = K p over all slots, then r, d, p updated per row)
+    # ---- roofline of the dominant kernel: the persistent solve, per product
+    # with K (scenes it does not take: the Chebyshev step of the inner
+    # iterations, q = K p over all slots, then r, d, p updated per row)
     peak, peak_kind = peaks()
-    n_sp, ms_sp = prof.get("cheb", (0, 0.0))
+    n_ps, ms_ps = prof.get("persist", (0, 0.0))
+    n_sp, ms_sp = (n_ps, ms_ps) if n_ps else prof.get("cheb", (0, 0.0))
     kernels = {}
     for name, (n, ms) in prof.items():
         if n:
@@ -787,12 +789,14 @@ def main():
     if n_sp:
         avg_s = ms_sp / n_sp / 1000.0
         ach = spmv_bytes / avg_s / 1e9
-        roof = {"kernel": "k_tile<6, OpCheb<float>> (FP32 Chebyshev step: q = K p over the rows of K with p "
+        roof = {"kernel": "k_persist<float> (BiCGStab steps with K on the chip and in L2; per product with K, "
+                          "the solve's set-up, barriers and residuals included)" if n_ps else
+                          "k_tile<6, OpCheb<float>> (FP32 Chebyshev step: q = K p over the rows of K with p "
                           "gathered from a shared-memory tile, then r, d, p updated per row)", "bound": "hbm",
                 "achieved": ach,
                 "peak": peak,
                 "unit": "GB/s", "frac": ach / peak, "peak_kind": peak_kind + " (hbm_gbs, copy)",
-                "traffic": traffic_record("k_tile_OpCheb") if not variant else None,
+                "traffic": traffic_record("k_tile_OpCheb") if not variant and not n_ps else None,
                 "algorithmic_bytes_per_launch": spmv_bytes,
                 "avg_launch_us": avg_s * 1e6}
     # ---- the edge form's terms: the contraction (tcgen05, TF32 split in

@@ -62,7 +62,8 @@ typedef enum {
 
 enum { TURSCA_FP64 = 0, TURSCA_FP32_REFINE = 1 };
 enum { TURSCA_COUPLING_NONE = 0, TURSCA_COUPLING_WEIGHT = 1 };
-enum { TURSCA_SOLVER_AUTO = 0, TURSCA_SOLVER_NEUMANN = 1, TURSCA_SOLVER_GMRES = 2, TURSCA_SOLVER_CHEBYSHEV = 3 };
+enum { TURSCA_SOLVER_AUTO = 0, TURSCA_SOLVER_NEUMANN = 1, TURSCA_SOLVER_GMRES = 2, TURSCA_SOLVER_CHEBYSHEV = 3,
+       TURSCA_SOLVER_BICGSTAB = 4 /* reported by TURSCA_SOLVER_AUTO; not a value to ask for */ };
 
 /* Grid and method parameters (fixed for the life of a scene).
  *   nx, ny >= 2 R + 1 (x and y are periodic), nz >= R.
@@ -171,14 +172,19 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
  * evaluated in FP64, with at most max_iter inner steps (a sweep, a Chebyshev
  * step, or a GMRES step, which applies K twice).  The outer loop is FP64
  * residual refinement; each refinement solves for the correction with inner
- * iterations in the scene's precision: FP32_REFINE scenes first run a few
- * Neumann sweeps (the series of Eq. fs_sum) that also estimate the largest
- * eigenvalue of K, then Chebyshev iterations on the interval that estimate
- * implies, or GMRES when the estimate is 0.85 or more or a Chebyshev
+ * iterations in the scene's precision.  Scenes whose matrix stays on the chip
+ * and in L2 (in FP32 up to about 1100 groups of 128 rows at radius 2: the 64 x
+ * 64 x 32 plume) are solved in one cooperative launch, by BiCGStab from the
+ * source to the refined solution.  Others run pass by pass: FP32_REFINE scenes
+ * first a few Neumann sweeps (the series of Eq. fs_sum) that also estimate the
+ * largest eigenvalue of K, then Chebyshev iterations on the interval that
+ * estimate implies, or GMRES when the estimate is 0.85 or more or a Chebyshev
  * refinement under-delivers; FP64 scenes run GMRES.  GMRES(30) (FP64: 40)
  * is right-preconditioned with I + K, the first two terms of that series.
- * Synchronises once per refinement (GMRES: once per step).  info may be
- * NULL. */
+ * TURSCA_OPT_GROUP_WARPS, TURSCA_OPT_STAGE_VALUES and TURSCA_OPT_RESIDUAL_FP64
+ * name how passes run, so setting one of them selects the passes.
+ * Synchronises once (the passes: once per refinement, GMRES: once per step).
+ * info may be NULL. */
 tursca_status tursca_solve(tursca_scene *scene, double rtol, int max_iter, tursca_solve_info *info);
 
 /* Same as tursca_solve with an explicit solver choice (TURSCA_SOLVER_*). */
@@ -366,7 +372,8 @@ typedef struct {
                            contraction and ground leaving power), "ani_transport" (one
                            term's transport and stopping test; terms launched past
                            convergence return at once and count too), "ani_residual" (one
-                           residual evaluation of the FP32 refinement) */
+                           residual evaluation of the FP32 refinement), "persist" (the
+                           persistent solve, counted as its products with K) */
     long long launches; /* launches since the last read */
     double total_ms;    /* summed event time of those launches */
 } tursca_kernel_stat;
@@ -475,25 +482,21 @@ typedef struct {
 typedef struct {
     size_t budget_bytes, used_bytes, peak_bytes;
     int slots, busy_slots, pending, evictions, slots_built;
-    /* batched Chebyshev refinements (see tursca_server_configure): launches,
-     * refinements run in them, and the most in one launch */
+    /* batched solves (see tursca_server_configure): launches, solves run in
+     * them, and the most in one launch */
     long long batches, batched_refinements;
     int max_batch;
 } tursca_server_stats;
 
 /* Server options (tursca_server_configure), to be set before the first
  * request:
- *   TURSCA_SERVER_BATCH_SOLVES: 0 (default) runs every request's passes on
- *     its own stream; 1 batches the Chebyshev refinements of the requests
- *     that run at the same time: a refinement handed over while others wait
- *     is launched together with them in one persistent kernel, which runs
- *     every request's row groups step after step with a grid-wide barrier
- *     between steps (every wait bounded); each request keeps its own step
- *     count and coefficients, and each group is computed by the same device
- *     code as the request's own Chebyshev pass, so a result does not depend
- *     on what it ran beside.  FP32 + refinement scenes whose pass has at most
- *     640 row groups (larger ones fill the GPU by themselves); two such
- *     launches may run at once, each on at most half the GPU. */
+ *   TURSCA_SERVER_BATCH_SOLVES: 0 (default) runs every request's solve on
+ *     its own stream; 1 batches the solves of the requests that run at the
+ *     same time: the solves that wait while a launch runs are launched
+ *     together in one persistent kernel, side by side, each on its own blocks
+ *     with its own barrier (every wait bounded) and its own convergence, so a
+ *     result does not depend on what it ran beside.  FP32 + refinement scenes
+ *     whose solve takes at most three quarters of the GPU's blocks. */
 enum { TURSCA_SERVER_BATCH_SOLVES = 1 };
 tursca_status tursca_server_configure(tursca_server *srv, int option, double value);
 

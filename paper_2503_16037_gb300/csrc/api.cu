@@ -15,6 +15,7 @@
 #include "first_order.h"
 #include "kern.h"
 #include "batch.h"
+#include "persist.h"
 #include "select.h"
 #include "aniso.h"
 #include "tursca.h"
@@ -153,8 +154,19 @@ struct tursca_scene {
     // its selection: per-chain keys, the radix histogram, the last threshold,
     // the number of chains with a receiver
     long long max_couplings = 0;
-    // the serving loop's batcher of Chebyshev refinements (null: own passes)
-    tk::ChebBatcher *batcher = nullptr;
+    // the persistent solve: plans of K and of K^T (nb = 0: not used), their
+    // tables, the exchange's block sums, the barrier word and the result
+    struct PsDev {
+        tk::PsPlan plan;
+        int2 *tpos = nullptr;
+        int *run = nullptr;
+    };
+    PsDev ps, psT;
+    double *ps_part = nullptr;
+    unsigned char *ps_ctl = nullptr;
+    bool x_pair = false;  // xh holds x in FP32 (of the forward solve)
+    // the serving loop's batcher of solves (null: own launches)
+    tk::SolveBatcher *batcher = nullptr;
     cudaEvent_t bready = nullptr, bdone = nullptr;
     unsigned long long *topk_keys = nullptr;
     unsigned int *topk_hist = nullptr, *topk_hist_h = nullptr;
@@ -206,18 +218,19 @@ struct tursca_scene {
 namespace {
 const char *const kProfNames[] = {"spmv",   "resid64",    "assemble_rows", "assemble_pre",  "render",
                                   "cheb",   "gmres_orth", "select",        "gmres_prod",    "set_medium",
-                                  "solve",  "ani_leave",  "ani_transport", "ani_residual"};
-constexpr int kNProf = 14;
+                                  "solve",  "ani_leave",  "ani_transport", "ani_residual", "persist"};
+constexpr int kNProf = 15;
 // P_GPROD: the passes over K of one Arnoldi step (preconditioner and product
 // with I - K), counted as launches; P_MEDIUM: the copies of set_medium;
 // P_SOLVE: a whole solve, from its first to its last operation on the stream
 // (the other categories of the solve lie inside it); P_ALEAVE, P_AMOVE: the
 // edge form's per-term leaving power (contraction and ground) and transport
 // (with its stopping test), terms past convergence included; P_ARESID: a
-// whole residual evaluation of its refinement
+// whole residual evaluation of its refinement; P_PERSIST: the persistent
+// solve's launch, counted as its products with K
 enum {
     P_SPMV = 0, P_RESID = 1, P_ROWS = 2, P_PRE = 3, P_RENDER = 4, P_CHEB = 5, P_ORTH = 6, P_SEL = 7, P_GPROD = 8,
-    P_MEDIUM = 9, P_SOLVE = 10, P_ALEAVE = 11, P_AMOVE = 12, P_ARESID = 13
+    P_MEDIUM = 9, P_SOLVE = 10, P_ALEAVE = 11, P_AMOVE = 12, P_ARESID = 13, P_PERSIST = 14
 };
 
 // NVTX range around one call of the C ABI (a stage of the path), for
@@ -598,9 +611,8 @@ struct SolveState {
     double rel = 1.0, rho = 0.0;
 };
 
-template <typename T>
-tursca_status read_red(tursca_scene *sc, int n) {
-    CK(cudaMemcpyAsync(sc->hred, sc->dred, n * sizeof(double), cudaMemcpyDeviceToHost, sc->st), "d2h");
+// waits for the stream and reports what the status word holds
+tursca_status read_status(tursca_scene *sc) {
     // the status word rides along: a bounded wait that gave up shows here
     int *hst = (int *)(sc->hred + 255);
     CK(cudaMemcpyAsync(hst, sc->status, sizeof(int), cudaMemcpyDeviceToHost, sc->st), "d2h");
@@ -610,6 +622,12 @@ tursca_status read_red(tursca_scene *sc, int n) {
     if (*hst & tk::STATUS_BAD_FIELD) return fail(sc, TURSCA_E_INVALID, "field values must be finite and non-negative");
     if (*hst & tk::STATUS_TIMEOUT) return fail(sc, TURSCA_E_TIMEOUT, "a bounded device wait gave up");
     return TURSCA_OK;
+}
+
+template <typename T>
+tursca_status read_red(tursca_scene *sc, int n) {
+    CK(cudaMemcpyAsync(sc->hred, sc->dred, n * sizeof(double), cudaMemcpyDeviceToHost, sc->st), "d2h");
+    return read_status(sc);
 }
 
 // Neumann (source) iteration on (I - K) d = b: d <- b + K d, n sweeps after d = b.
@@ -791,6 +809,7 @@ struct SolveIO {
     const T *val;
     const T *s;
     double *x;
+    const tursca_scene::PsDev *ps;
 };
 
 template <typename T>
@@ -801,7 +820,118 @@ SolveIO<T> forward_io(tursca_scene *sc) {
     io.val = (const T *)sc->val;
     io.s = (const T *)sc->s;
     io.x = sc->x64;
+    io.ps = &sc->ps;
     return io;
+}
+
+// The plan of the persistent solve for templates tstart (layers 0 .. nz, the
+// ground at nz) whose entries gather from layer src_layer at in-layer haloed
+// offset off, uploaded with its tables.  Scenes that do not fit get no plan.
+tursca_status upload_persist(tursca_scene *sc, tursca_scene::PsDev &P, const std::vector<int> &tstart,
+                             const std::vector<int> &src_layer, const std::vector<int> &off) {
+    const tk::GridC g = grid_c(sc);
+    std::vector<int> nt(g.nz + 1);
+    for (int z = 0; z <= g.nz; ++z) nt[z] = tstart[z + 1] - tstart[z];
+    // every source lies within R of its row in the order ground, layer 0, 1, ...
+    std::vector<int2> tp(src_layer.size());
+    for (int z = 0; z <= g.nz; ++z)
+        for (int i = tstart[z]; i < tstart[z + 1]; ++i) {
+            const int zz = z == g.nz ? 0 : z + 1, zs = src_layer[i] == g.nz ? 0 : src_layer[i] + 1;
+            if (std::abs(zs - zz) > g.R || std::abs(off[i]) > g.H * g.nxp + g.H) return TURSCA_OK;
+            tp[i] = make_int2(zs, off[i]);
+        }
+    int dev = 0, nsm = 0, smem = 0, coop = 0;
+    CK(cudaGetDevice(&dev), "device");
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "device");
+    CK(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), "device");
+    CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev), "device");
+    tk::PsPlan plan;
+    if (coop) plan = tk::ps_plan(tk::ps_geom(g), nt, (int)sc->es, nsm, (size_t)smem, tk::ps_fixed_smem());
+    if (plan.nb > 0) {
+        CK(upload(sc, sc->allocs, P.tpos, tp.data(), std::max<size_t>(1, tp.size()) * sizeof(int2)), "upload plan");
+        CK(upload(sc, sc->allocs, P.run, plan.run.data(), plan.run.size() * sizeof(int)), "upload plan");
+        if (!sc->ps_part) {
+            CK(dalloc(sc->allocs, sc->ps_part, (size_t)3 * tk::kPsDots * std::max(nsm, 1) * sizeof(double)), "alloc plan");
+            CK(dalloc(sc->allocs, sc->ps_ctl, 256), "alloc plan");
+        }
+        CK(cudaStreamSynchronize(sc->st), "sync");  // tp dies here
+    }
+    P.plan = std::move(plan);
+    return TURSCA_OK;
+}
+
+// Solve with the persistent kernel.  *done is false when the scene has no
+// plan, the launch is refused or the iteration gave up; the caller's loop
+// then solves from x = 0.
+template <typename T>
+tursca_status persist_solve(tursca_scene *sc, const SolveIO<T> &io, double rtol, int max_iter,
+                            tursca_solve_info *info, bool *done) {
+    *done = false;
+    const tk::PsPlan &P = io.ps->plan;
+    if (P.nb <= 0) return TURSCA_OK;
+    tk::PsJob J;
+    J.g = io.g;
+    J.tstart = io.gp.tstart;
+    J.voff = io.gp.voff;
+    J.tpos = io.ps->tpos;
+    J.run = io.ps->run;
+    J.val = io.val;
+    J.s = io.s;
+    J.x = io.x;
+    J.xh = sc->xh;
+    J.xl = sc->xl;
+    J.pub[0] = sc->d0;
+    J.pub[1] = sc->d1;
+    J.pub[2] = sc->w;
+    J.part = sc->ps_part;
+    J.bar = (unsigned *)sc->ps_ctl;
+    J.status = sc->status;
+    J.info = (tk::PsInfo *)(sc->ps_ctl + 64);
+    J.rtol = rtol;
+    J.max_iter = max_iter;
+    J.block0 = 0;
+    J.nb = P.nb;
+    J.nl = P.nl;
+    J.tl = P.tl;
+    J.nchunk = P.nchunk;
+    J.wpg = P.wpg;
+    J.it = P.it;
+    J.kcap = P.kcap;
+    CK(cudaMemsetAsync(sc->ps_ctl, 0, 256, sc->st), "memset plan");
+    const int pi = prof_begin(sc, P_PERSIST);
+    bool launched = false;
+    if (sc->batcher && sizeof(T) == 4) {  // in a server: launched together with other requests' solves
+        CK(cudaEventRecord(sc->bready, sc->st), "batch event");
+        if (tk::batcher_run(sc->batcher, J, P.smem, sc->bready, sc->bdone)) {
+            CK(cudaStreamWaitEvent(sc->st, sc->bdone, 0), "batch wait");
+            launched = true;
+        }
+    }
+    if (!launched && tk::launch_persist(sc->st, &J, 1, P.nb, P.smem, sizeof(T) == 8) != cudaSuccess) {
+        cudaGetLastError();  // e.g. no room for a cooperative launch: the caller's loop solves
+        prof_end(sc, pi, 0);
+        return TURSCA_OK;
+    }
+    sc->launches++;
+    tk::PsInfo *h = (tk::PsInfo *)sc->hred;
+    CK(cudaMemcpyAsync(h, sc->ps_ctl + 64, sizeof(tk::PsInfo), cudaMemcpyDeviceToHost, sc->st), "d2h");
+    prof_end(sc, pi);
+    const tursca_status rs = read_status(sc);
+    if (rs) return rs;
+    if (pi >= 0) sc->ev_n[pi] = h->iters;
+    if (h->state != tk::PS_CONVERGED && h->state != tk::PS_MAX_ITER) return TURSCA_OK;
+    *done = true;
+    if (info) {
+        info->iters = h->iters;
+        info->refinements = h->refinements;
+        info->rel_resid64 = h->rel;
+        info->rho_est = 0.0;
+        info->solver = TURSCA_SOLVER_BICGSTAB;
+    }
+    sc->x_pair = sizeof(T) == 4 && io.x == sc->x64;
+    sc->solved = true;
+    if (h->state == tk::PS_MAX_ITER) return fail(sc, TURSCA_E_NOT_CONVERGED, "solver stopped above rtol");
+    return TURSCA_OK;
 }
 
 // The values of K in the persisting part of L2 for the passes of one solve
@@ -852,6 +982,13 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     SolveState ss;
     (void)nb;
     const bool fp64 = sc->d.precision == TURSCA_FP64;
+    sc->x_pair = false;
+    // the persistent solve: automatic choice, with no option that names how the passes run
+    if (solver == TURSCA_SOLVER_AUTO && sc->wq_auto && !sc->stage_values && !sc->resid_fp64) {
+        bool done = false;
+        const tursca_status e = persist_solve<T>(sc, io, rtol, max_iter, info, &done);
+        if (e || done) return e;
+    }
     if (solver == TURSCA_SOLVER_AUTO) solver = fp64 ? TURSCA_SOLVER_GMRES : TURSCA_SOLVER_CHEBYSHEV;
     auto ensure_basis = [&]() -> tursca_status {
         int m = fp64 ? 40 : TK_GMRES_M32;
@@ -953,55 +1090,20 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
             T *r = bb, *d = (T *)sc->w, *p0 = (T *)sc->d0, *p1 = (T *)sc->d1;
             tk::launch_cheb_start<T>(sc->st, n, sc->r64, 1.0 / cp.theta, r, d, p0);
             sc->launches++;
-            // in a server: hand the refinement to the batcher, which runs it
-            // in one persistent launch with the refinements of other requests
-            bool batched = false;
-            if constexpr (sizeof(T) == 4) {
-                if (sc->batcher && tk::batch_eligible(g, nc)) {
-                    tk::ChebJob job;
-                    std::memset(&job, 0, sizeof(job));
-                    job.g = g;
-                    job.gp = gp;
-                    job.val = (const float *)val;
-                    job.r = (float *)r;
-                    job.d = (float *)d;
-                    job.p[0] = (float *)p0;
-                    job.p[1] = (float *)p1;
-                    job.x64 = io.x;
-                    job.xh = ds ? sc->xh : nullptr;
-                    job.xl = ds ? sc->xl : nullptr;
-                    job.nsteps = nc;
-                    job.W = g.wq;
-                    double rk = 1.0 / cp.sigma;
-                    for (int k = 0; k < nc; ++k) {  // the coefficients the scene's own passes would take
-                        const double rk1 = 1.0 / (2.0 * cp.sigma - rk);
-                        job.c1[k] = (float)(rk1 * rk);
-                        job.c2[k] = (float)(2.0 * rk1 / cp.delta);
-                        rk = rk1;
-                    }
-                    CK(cudaEventRecord(sc->bready, sc->st), "batch event");
-                    if (tk::batcher_run(sc->batcher, job, sc->bready, sc->bdone)) {
-                        CK(cudaStreamWaitEvent(sc->st, sc->bdone, 0), "batch wait");
-                        batched = true;
-                    }
-                }
+            double rk = 1.0 / cp.sigma;
+            int pi = prof_begin(sc, P_CHEB);
+            for (int k = 0; k < nc; ++k) {
+                double rk1 = 1.0 / (2.0 * cp.sigma - rk);
+                // the last step also applies x += d row by row
+                const bool last = k == nc - 1;
+                tk::launch_cheb<T>(sc->st, g, gp, val, p0, r, d, p1, rk1 * rk, 2.0 * rk1 / cp.delta,
+                                   last ? io.x : nullptr, last && ds ? sc->xh : nullptr,
+                                   last && ds ? sc->xl : nullptr);
+                std::swap(p0, p1);
+                rk = rk1;
             }
-            if (!batched) {
-                double rk = 1.0 / cp.sigma;
-                int pi = prof_begin(sc, P_CHEB);
-                for (int k = 0; k < nc; ++k) {
-                    double rk1 = 1.0 / (2.0 * cp.sigma - rk);
-                    // the last step also applies x += d row by row
-                    const bool last = k == nc - 1;
-                    tk::launch_cheb<T>(sc->st, g, gp, val, p0, r, d, p1, rk1 * rk, 2.0 * rk1 / cp.delta,
-                                       last ? io.x : nullptr, last && ds ? sc->xh : nullptr,
-                                       last && ds ? sc->xl : nullptr);
-                    std::swap(p0, p1);
-                    rk = rk1;
-                }
-                prof_end(sc, pi, nc);
-                sc->launches += nc;
-            }
+            prof_end(sc, pi, nc);
+            sc->launches += nc;
             ss.iters += nc;
             dd = d;
             x_done = true;
@@ -1103,6 +1205,8 @@ tursca_status do_render(tursca_scene *sc, void *radiance, void *reflectance) {
         const T *xc;
         if constexpr (sizeof(T) == 8) {
             xc = (const T *)sc->x64;
+        } else if (sc->x_pair) {
+            xc = (const T *)sc->xh;  // the solve left x in FP32
         } else {
             tk::launch_convert<double, T>(sc->st, (int)g.npad, sc->x64, (T *)sc->w);
             sc->launches++;
@@ -1157,8 +1261,17 @@ tursca_status ensure_adjoint(tursca_scene *sc) {
             sc->tile_tlT = tl.tl;
         }
     }
+    {
+        std::vector<int> off(ne);
+        for (int z = 0; z <= g.nz; ++z)
+            for (int e = Tt.tstart[z]; e < Tt.tstart[z + 1]; ++e)
+                off[e] = Tt.flat_h[e] - (Tt.recv_layer[e] - z) * g.lp;
+        const tursca_status e = upload_persist(sc, sc->psT, Tt.tstart, Tt.recv_layer, off);
+        if (e) return e;
+    }
     const size_t es = sc->es;
-    CK(dalloc(sc->allocs, sc->valT, (size_t)G.nval * es), "alloc K^T");
+    CK(dalloc(sc->allocs, sc->valT, ((size_t)G.nval + tk::kPsPad) * es), "alloc K^T");
+    CK(cudaMemsetAsync((char *)sc->valT + (size_t)G.nval * es, 0, tk::kPsPad * es, sc->st), "memset K^T");
     CK(dalloc(sc->allocs, sc->lam64, (size_t)g.npad * sizeof(double)), "alloc adjoint");
     CK(dalloc(sc->allocs, sc->Lbar, (size_t)sc->geom.npx * sc->geom.npy * es), "alloc adjoint");
     const size_t nn = (size_t)g.n_nodes, na = (size_t)g.n_atm, np = (size_t)g.npad;
@@ -1215,6 +1328,7 @@ tursca_status do_adjoint(tursca_scene *sc, const void *dJ_dL, void *dJ_dmu_abs) 
     io.val = (const T *)sc->valT;
     io.s = ad.xbar;
     io.x = sc->lam64;
+    io.ps = &sc->psT;
     tursca_solve_info info;
     const double rtol = sc->d.precision == TURSCA_FP64 ? 1e-12 : 1e-9;
     tursca_status rs = do_solve<T>(sc, TURSCA_SOLVER_AUTO, rtol, 5000, &info, io);
@@ -1921,7 +2035,8 @@ tursca_status tursca_build_graph(tursca_scene *sc) {
         }
     }
     CK(upload(sc, sc->allocs, sc->voff, G.voff.data(), G.voff.size() * sizeof(long long)), "upload tmpl");
-    CK(dalloc(sc->allocs, sc->val, (size_t)G.nval * sc->es), "alloc val");
+    CK(dalloc(sc->allocs, sc->val, ((size_t)G.nval + tk::kPsPad) * sc->es), "alloc val");
+    CK(cudaMemsetAsync((char *)sc->val + (size_t)G.nval * sc->es, 0, tk::kPsPad * sc->es, sc->st), "memset val");
     const size_t es = sc->es;
     CK(dalloc(sc->allocs, sc->tinf, (size_t)G.up_dirs.size() * G.n_atm * es), "alloc tinf");
     const size_t Hh = (size_t)sc->d.stencil_radius;
@@ -1991,6 +2106,16 @@ tursca_status tursca_build_graph(tursca_scene *sc) {
     cudaError_t ce = cudaStreamSynchronize(sc->st);
     if (ce != cudaSuccess) return cuda_fail(sc, ce, "build_graph");
     if (sc->wq_auto) sc->wq = tk::choose_wq(grid_c(sc), sc->d.precision == TURSCA_FP64);
+    {
+        const int nxp = sc->d.nx + 2 * sc->d.stencil_radius;
+        std::vector<int> lay(G.tmpl.size()), off(G.tmpl.size());
+        for (size_t i = 0; i < G.tmpl.size(); ++i) {
+            lay[i] = G.tmpl[i].sz >= 0 ? G.tmpl[i].sz : sc->d.nz;
+            off[i] = G.tmpl[i].sdy * nxp + G.tmpl[i].sdx;
+        }
+        e = upload_persist(sc, sc->ps, G.tmpl_start, lay, off);
+        if (e) return e;
+    }
     for (int i = 0; i < 3; ++i) CK(cudaStreamCreateWithFlags(&sc->aux[i], cudaStreamNonBlocking), "aux stream");
     for (int i = 0; i < 5; ++i) CK(cudaEventCreateWithFlags(&sc->fork[i], cudaEventDisableTiming), "aux event");
     sc->built = true;
@@ -2618,7 +2743,7 @@ tursca_status tursca_profile_read(tursca_scene *sc, tursca_kernel_stat *out, int
 
 tursca_status tursca_selftest_barrier(void *cuda_stream, int blocks, int arrive) {
     if (blocks < 1 || blocks > 1024) return fail(nullptr, TURSCA_E_INVALID, "blocks must be in 1..1024");
-    const int r = tk::batch_barrier_selftest((cudaStream_t)cuda_stream, blocks, arrive);
+    const int r = tk::barrier_selftest((cudaStream_t)cuda_stream, blocks, arrive);
     if (r < 0) return fail(nullptr, TURSCA_E_CUDA, "barrier self-test: CUDA error");
     return r ? TURSCA_E_TIMEOUT : TURSCA_OK;
 }
@@ -2731,7 +2856,7 @@ tursca_status tursca_last_error(const tursca_scene *sc, char *buf, size_t n) {
 }  // extern "C"
 
 namespace tk {
-void scene_attach_batcher(tursca_scene *sc, ChebBatcher *b) {
+void scene_attach_batcher(tursca_scene *sc, SolveBatcher *b) {
     if (!sc || sc->d.precision == TURSCA_FP64) return;
     if (b && !sc->bready) {
         if (cudaEventCreateWithFlags(&sc->bready, cudaEventDisableTiming) != cudaSuccess ||

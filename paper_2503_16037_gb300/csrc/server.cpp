@@ -80,7 +80,7 @@ struct tursca_server {
     int evictions = 0, built = 0, reserving = 0;
     bool stop = false;
     bool batch_solves = false;          // TURSCA_SERVER_BATCH_SOLVES
-    tk::ChebBatcher *batcher = nullptr;  // created with the first FP32 slot
+    tk::SolveBatcher *batcher = nullptr;  // created with the first FP32 slot
     Clock::time_point t0 = Clock::now();
 
     double now_ms() const { return std::chrono::duration<double, std::milli>(Clock::now() - t0).count(); }

@@ -459,18 +459,15 @@ struct tile_op<Op, std::void_t<decltype(Op::kTile)>> {
 // previous pass has completed, and every slot then gathers from the tile:
 // tile[ttile[t] + rl], with rl the row's position within one tile layer.
 // Products and their order are those of k_plain.
-// One group gi of the tiled driver, shared by k_tile (one block per group,
-// kPdl: the previous pass is waited for after the graph data are read) and
-// the persistent batch of Chebyshev steps across requests (kCoherent: the
-// gathered vector was written by other blocks of the same launch since this
-// block last read it, so it is read around L1).  sh, tile, s_lay: the
-// block's shared memory; a block may run several groups one after another.
-template <int W, class Op, bool kPdl, bool kCoherent>
-__device__ __forceinline__ void tile_group(const GridC &g, const GraphP &gp, const float *__restrict__ val,
-                                           const Op &op, int gi, typename Op::A (*sh)[Op::NA][32], float *tile,
-                                           int *s_lay) {
+template <int W, class Op>
+__global__ void __launch_bounds__(32 * W, TK_TILE_WARPS / W) k_tile(GridC g, GraphP gp, const float *__restrict__ val, Op op) {
     using A = typename Op::A;
     constexpr int NA = Op::NA;
+    __shared__ A sh[W][NA][32];
+    extern __shared__ float tile[];
+    __shared__ int s_lay[kTileLayers];
+    pdl_trigger();
+    const int gi = blockIdx.x;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const GroupRows G = group_rows(g, gp, gi);
     // the tile's source layers are graph data: read them before waiting
@@ -495,7 +492,7 @@ __device__ __forceinline__ void tile_group(const GridC &g, const GraphP &gp, con
     if (tA < G.nt) ld_quad(v + (size_t)tA * kGroup, v0);
     if (tB < G.nt) ld_quad(v + (size_t)tB * kGroup, v1);
     const int ttA = tA < G.nt ? __ldg(gp.ttile + G.t0 + tA) : 0, ttB = tB < G.nt ? __ldg(gp.ttile + G.t0 + tB) : 0;
-    if constexpr (kPdl) pdl_wait();
+    pdl_wait();
     const typename Op::Pre pre = load_pre(op, G);
     const int ts = kTileLayers * g.tl;  // floats per vector's tile
     __syncthreads();  // s_lay
@@ -507,7 +504,7 @@ __device__ __forceinline__ void tile_group(const GridC &g, const GraphP &gp, con
             if (lay < 0) break;  // the used tile layers come first
             const float *s = src + (long long)lay * g.lp;
             float *d = tile + iv * ts + ls * g.tl;
-            for (int j = threadIdx.x; j < tla; j += 32 * W) d[j] = kCoherent ? __ldcg(s + j) : s[j];
+            for (int j = threadIdx.x; j < tla; j += 32 * W) d[j] = s[j];
         }
     }
     __syncthreads();
@@ -534,17 +531,6 @@ __device__ __forceinline__ void tile_group(const GridC &g, const GraphP &gp, con
     for (int m = 0; m < NA; ++m) sh[w][m][lane] = a[m];
     __syncthreads();
     finish_rows<W>(op, sh, G, pre, gi);
-}
-
-template <int W, class Op>
-__global__ void __launch_bounds__(32 * W, TK_TILE_WARPS / W) k_tile(GridC g, GraphP gp, const float *__restrict__ val, Op op) {
-    using A = typename Op::A;
-    constexpr int NA = Op::NA;
-    __shared__ A sh[W][NA][32];
-    extern __shared__ float tile[];
-    __shared__ int s_lay[kTileLayers];
-    pdl_trigger();
-    tile_group<W, Op, true, false>(g, gp, val, op, blockIdx.x, sh, tile, s_lay);
 }
 
 // pipelined launch: one block per run (one run per SM, at most one per group)
