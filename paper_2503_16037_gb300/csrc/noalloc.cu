@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "tursca.h"
 
@@ -22,7 +23,8 @@ constexpr size_t kOffB = 0;                        // float  [kMaxNodes] right-h
 constexpr size_t kOffD0 = kOffB + 4ull * kMaxNodes;  // float  [kMaxNodes] sweep buffer
 constexpr size_t kOffD1 = kOffD0 + 4ull * kMaxNodes; // float  [kMaxNodes] sweep buffer
 constexpr size_t kOffPart = kOffD1 + 4ull * kMaxNodes; // double [kPartBlocks]
-constexpr size_t kScratchBytes = kOffPart + 8ull * kPartBlocks;  // about 12 MiB
+constexpr size_t kOffBar = kOffPart + 8ull * kPartBlocks;  // barrier word of the one-launch form
+constexpr size_t kScratchBytes = kOffBar + 256;            // about 12 MiB
 
 // Shared by every call on a device; holds the previous call's contents.
 static __device__ __align__(256) unsigned char g_solve_scratch[kScratchBytes];
@@ -99,6 +101,304 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
     *out = t;
 }
 
+// ---------------------------------------------------------------------------
+// The whole solve in one cooperative launch, for systems whose matrix stays
+// in L2.
+//
+// What bounds a sweep of one launch each (k_na_sweep) is the gather of v: 32
+// unrelated addresses per warp load, 24 us for 6.1M entries (65,536 rows of a
+// band of +-4096), where the matrix itself (49 MB) would take 5 us from L2.
+// Here a block owns the same rows for the whole solve, keeps in shared memory
+// the window of v that its rows reach (columns modulo n, so a band that wraps
+// around is one window) and as many of its entries as fit beside it, as 4-byte
+// values and 2-byte window indices; the other entries come from L2, where
+// they stay because a line is only ever read by one SM.  Blocks exchange v
+// through global memory with one grid barrier per sweep.  A block whose rows
+// reach too far for a window gathers from global memory.
+//
+// Kept rows are packed to whole quads (zero padding), so a lane takes four
+// entries per step with two loads of values and indices; 8 lanes (32 where
+// rows average more than 256 entries) share a row.  80 sweeps over the 65,536
+// rows: 2010 us with a launch per sweep, 1159 us in one launch entry by entry
+// (a warp per row, bound by its 47 instructions per 32 entries), 1085 us as
+// here.
+constexpr int kNsThreads = 1024, kNsWarps = kNsThreads / 32;
+constexpr int kNsMaxRows = 4096;     // rows a block may keep
+constexpr int kNsMaxNodes = 131072;  // above this the matrix no longer stays in L2: a launch per sweep
+constexpr long long kNsPolls = 1ll << 21;  // polls of one barrier: about 1.5 s
+
+struct NsArgs {
+    int n, sweeps, refinements, smem;
+    const int32_t *row_ptr, *col;
+    const float *val, *s;
+    double *x, *resid2, *part;
+    float *b, *d0, *d1;
+    unsigned *bar;
+};
+
+__global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constant__ NsArgs A) {
+    extern __shared__ __align__(16) unsigned char ns_dyn[];
+    __shared__ int sh_r[2], sh_min[kNsWarps], sh_max[kNsWarps], sh_ok;
+    __shared__ double sh_red[kNsWarps];
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, n = A.n, nb = gridDim.x, blk = blockIdx.x;
+    const int32_t *__restrict__ rp = A.row_ptr;
+    // rows [r0, r1): equal shares of entries, a row counted as 16 more
+    if (tid < 2) {
+        const long long base = rp[0], total = (long long)rp[n] - base + 16ll * n;
+        const long long target = total * (blk + tid) / nb;
+        int lo = 0, hi = n;
+        while (lo < hi) {
+            const int m = (lo + hi) >> 1;
+            if ((long long)rp[m] - base + 16ll * m < target) lo = m + 1;
+            else hi = m;
+        }
+        sh_r[tid] = blk + tid == nb ? n : lo;
+    }
+    __syncthreads();
+    const int r0 = sh_r[0], r1 = sh_r[1], e0 = rp[r0], ne = rp[r1] - e0;
+    // the window: the smallest and largest column, as offsets from r0 modulo n
+    int mn = 0x7fffffff, mx = -0x7fffffff;
+    for (int e = tid; e < ne; e += kNsThreads) {
+        int d = __ldg(A.col + e0 + e) - r0;
+        if (d > n / 2) d -= n;
+        else if (d < -(n / 2)) d += n;
+        mn = min(mn, d);
+        mx = max(mx, d);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (lane == 0) {
+        sh_min[w] = mn;
+        sh_max[w] = mx;
+    }
+    __syncthreads();
+    for (int q = 0; q < kNsWarps; ++q) {
+        mn = min(mn, sh_min[q]);
+        mx = max(mx, sh_max[q]);
+    }
+    int w0 = r0 + mn, W = mx - mn + 1;
+    if (ne == 0) w0 = W = 0;
+    else if (W >= n) { w0 = 0; W = n; }
+    if (w0 < 0) w0 += n;
+    else if (w0 >= n) w0 -= n;
+    const bool win4 = W <= 32768;                         // v in shared memory
+    const bool win8 = W <= 12288;                         // x too (FP64)
+    const int wbytes = win4 ? ((win8 ? 8 : 4) * W + 15) / 16 * 16 : 0;
+    // rows kept, from the first on: packed row starts (in quads), values, indices
+    const int capq = win4 ? (A.smem - wbytes - kNsMaxRows * 2 - 64) / 24 : 0;  // quads that fit
+    float *win = (float *)ns_dyn;
+    double *winx = (double *)ns_dyn;
+    float4 *sval = (float4 *)(ns_dyn + wbytes);
+    uint2 *sidx = (uint2 *)(sval + capq);
+    uint16_t *srow = (uint16_t *)(sidx + capq);
+    auto local = [&](int c) {
+        int d = c - w0;
+        d += d < 0 ? n : 0;
+        return d;
+    };
+    int kept = 0;  // rows [r0, r0 + kept)
+    if (capq > 0) {
+        int carry = 0;
+        const int most = min(r1 - r0, kNsMaxRows - 1);
+        for (int base = 0; base < most; base += kNsThreads) {
+            const int r = base + tid;
+            const int q = r < most ? (__ldg(rp + r0 + r + 1) - __ldg(rp + r0 + r) + 3) / 4 : 0;
+            int v = q;  // inclusive scan over the block
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            __syncthreads();
+            if (lane == 31) sh_min[w] = v;
+            __syncthreads();
+            int before = carry, all = 0;
+            for (int k = 0; k < kNsWarps; ++k) {
+                if (k < w) before += sh_min[k];
+                all += sh_min[k];
+            }
+            v += before;
+            const bool fits = r < most && v <= capq;
+            if (fits) srow[r + 1] = (uint16_t)v;
+            if (r == 0) srow[0] = 0;
+            const int nf = __syncthreads_count(fits);  // a prefix of the rows: v never falls
+            kept = base + nf;
+            carry += all;
+            if (nf < kNsThreads) break;
+        }
+    }
+    __syncthreads();
+    for (int r = tid / 8; r < kept; r += kNsThreads / 8) {
+        const int p = __ldg(rp + r0 + r), len = __ldg(rp + r0 + r + 1) - p, q0 = srow[r];
+        float *v = (float *)(sval + q0);
+        uint16_t *ix = (uint16_t *)(sidx + q0);
+        for (int i = tid % 8; i < (len + 3) / 4 * 4; i += 8) {
+            v[i] = i < len ? __ldg(A.val + p + i) : 0.f;
+            ix[i] = (uint16_t)local(__ldg(A.col + p + min(i, len - 1)));
+        }
+    }
+    unsigned gen = 0;
+    auto barrier = [&]() -> bool {
+        ++gen;
+        __syncthreads();
+        if (tid == 0) {
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(A.bar) : "memory");
+            int ok = 0;
+            for (long long i = 0; i < kNsPolls; ++i) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.bar) : "memory");
+                if ((int)(v - gen * (unsigned)nb) >= 0) {
+                    ok = 1;
+                    break;
+                }
+            }
+            sh_ok = ok;
+        }
+        __syncthreads();
+        return sh_ok != 0;
+    };
+    // Every row's sum over its entries of val times the gathered vector (from
+    // the kept entries; else from L2 with the window, or from global memory),
+    // handed to out(row, sum) in one lane of the row's L lanes.  The rows that
+    // are not kept go first: their loads take longest.
+    auto rows = [&](auto lanes_c, auto zero, const auto *vec, const auto *window, bool windowed, auto out) {
+        constexpr int L = decltype(lanes_c)::value;
+        using V = decltype(zero);
+        const int sl = lane & (L - 1), first = tid / 32 * (32 / L) + lane / L, lanes = kNsThreads / L;
+        auto sum = [&](V acc, int row, bool on) {
+            __syncwarp();
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (sl == 0 && on) out(row, acc);
+        };
+        const int k0 = windowed ? kept : 0;
+        for (int b = r0 + k0; b < r1; b += lanes) {
+            const int row = b + first;
+            const bool on = row < r1;
+            const int p = on ? __ldg(rp + row) : 0, end = on ? __ldg(rp + row + 1) : 0;
+            V acc = zero;
+            constexpr int U = sizeof(V) == 4 ? 6 : 4;
+            for (int e = p + sl; e < end; e += U * L) {
+                float v[U];
+                int c[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = e + u * L < end;
+                    v[u] = in ? __ldg(A.val + e + u * L) : 0.f;
+                    c[u] = in ? __ldg(A.col + e + u * L) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (c[u] >= 0) acc += (V)v[u] * (windowed ? window[local(c[u])] : vec[c[u]]);
+            }
+            sum(acc, row, on);
+        }
+        for (int b = 0; b < k0; b += lanes) {
+            const int r = b + first;
+            const bool on = r < k0;
+            const int q0 = on ? srow[r] : 0, q1 = on ? srow[r + 1] : 0;
+            V acc = zero;
+#pragma unroll 2
+            for (int q = q0 + sl; q < q1; q += L) {
+                const float4 v = sval[q];
+                const uint2 ix = sidx[q];
+                acc += (V)v.x * window[ix.x & 0xffffu];
+                acc += (V)v.y * window[ix.x >> 16];
+                acc += (V)v.z * window[ix.y & 0xffffu];
+                acc += (V)v.w * window[ix.y >> 16];
+            }
+            sum(acc, r0 + r, on);
+        }
+    };
+    const bool wide = (long long)rp[n] - rp[0] > 256ll * n;
+    auto all_rows = [&](auto zero, const auto *vec, const auto *window, bool windowed, auto out) {
+        if (wide) rows(std::integral_constant<int, 32>(), zero, vec, window, windowed, out);
+        else rows(std::integral_constant<int, 8>(), zero, vec, window, windowed, out);
+    };
+    bool ok = true;
+    for (int i = r0 + tid; i < r1; i += kNsThreads) {
+        A.x[i] = 0.0;
+        A.b[i] = A.s[i];
+    }
+    ok = barrier();
+    for (int r = 0; ok && r < A.refinements; ++r) {
+        const float *cur = A.b;
+        for (int k = 0; ok && k < A.sweeps; ++k) {
+            float *nxt = (k & 1) ? A.d1 : A.d0;
+            if (win4) {
+#pragma unroll 8
+                for (int j = tid; j < W; j += kNsThreads) {
+                    const int g = w0 + j;
+                    win[j] = __ldcg(cur + (g >= n ? g - n : g));
+                }
+                __syncthreads();
+            }
+            all_rows(0.f, cur, win, win4, [&](int row, float v) { nxt[row] = A.b[row] + v; });
+            cur = nxt;
+            ok = barrier();
+        }
+        if (!ok) break;
+        for (int i = r0 + tid; i < r1; i += kNsThreads) A.x[i] += (double)cur[i];
+        ok = barrier();
+        if (!ok) break;
+        if (win8) {
+#pragma unroll 4
+            for (int j = tid; j < W; j += kNsThreads) {
+                const int g = w0 + j;
+                winx[j] = __ldcg(A.x + (g >= n ? g - n : g));
+            }
+            __syncthreads();
+        }
+        double loc = 0.0;
+        all_rows(0.0, A.x, winx, win8, [&](int row, double v) {
+            const double res = (double)A.s[row] - A.x[row] + v;
+            A.b[row] = (float)res;
+            loc += res * res;
+        });
+        if (r == A.refinements - 1 && A.resid2) {
+            for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+            if (lane == 0) sh_red[w] = loc;
+            __syncthreads();
+            if (tid == 0) {
+                double t = 0.0;
+                for (int q = 0; q < kNsWarps; ++q) t += sh_red[q];
+                A.part[blk] = t;
+            }
+        }
+        if (r + 1 < A.refinements || A.resid2) ok = barrier();
+    }
+    if (!ok) {  // a barrier gave up (the launch is cooperative, so none should): no half result
+        for (int i = r0 + tid; i < r1; i += kNsThreads) A.x[i] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+    if (A.resid2 && blk == 0 && tid == 0) {
+        double t = ok ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+        for (int q = 0; ok && q < nb; ++q) t += __ldcg(A.part + q);
+        *A.resid2 = t;
+    }
+}
+
+// launches k_na_solve; false when this device cannot (the caller then runs a
+// launch per sweep)
+bool one_launch(const NsArgs &a0, cudaStream_t st) {
+    int dev = 0, nsm = 0, smem = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop || nsm < 1 ||
+        smem < 160 * 1024)
+        return false;
+    NsArgs a = a0;
+    a.smem = smem - 4 * 1024;  // beside the static shared memory
+    int nb = (a.n + kNsWarps - 1) / kNsWarps;
+    if (nb > nsm) nb = nsm;
+    if (nb > kPartBlocks) nb = kPartBlocks;
+    if (cudaFuncSetAttribute(k_na_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem) != cudaSuccess) return false;
+    if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned), st) != cudaSuccess) return false;
+    void *args[] = {(void *)&a};
+    return cudaLaunchCooperativeKernel((const void *)k_na_solve, dim3(nb), dim3(kNsThreads), args, a.smem, st) == cudaSuccess;
+}
+
 }  // namespace
 
 extern "C" tursca_status tursca_csr_solve_noalloc(const int32_t *row_ptr, const int32_t *col, const float *val,
@@ -122,6 +422,26 @@ extern "C" tursca_status tursca_csr_solve_noalloc(const int32_t *row_ptr, const 
     const long long rows_blocks = ((long long)n_nodes * 32 + th - 1) / th;
     int nres = (n_nodes + 7) / 8;
     if (nres > kPartBlocks) nres = kPartBlocks;
+    if (n_nodes <= kNsMaxNodes) {
+        NsArgs a;
+        a.n = n_nodes;
+        a.sweeps = sweeps;
+        a.refinements = refinements;
+        a.smem = 0;
+        a.row_ptr = row_ptr;
+        a.col = col;
+        a.val = val;
+        a.s = s;
+        a.x = x;
+        a.resid2 = resid2;
+        a.part = part;
+        a.b = b;
+        a.d0 = d0;
+        a.d1 = d1;
+        a.bar = (unsigned *)(p + kOffBar);
+        if (one_launch(a, st)) return TURSCA_OK;
+        cudaGetLastError();  // its own error only: none was pending
+    }
     k_na_init<<<nvec, th, 0, st>>>(n_nodes, s, x, b);
     // a launch that fails (a bad stream, say) fails them all: stop at the first
     if (cudaGetLastError() != cudaSuccess) return TURSCA_E_CUDA;
