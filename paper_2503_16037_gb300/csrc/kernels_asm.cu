@@ -827,14 +827,14 @@ __device__ __forceinline__ double q_of<double>(double t) { return -expm1(-t); }
 // an upward chain, P = T_pre Q(tau_seg + tau_inf).  PRE: the chain has
 // segments before the receiver (then the first receiver is not the
 // receiver itself).  T = exp(-tau), Q = 1 - T.
-template <typename T, int S, int FT, bool PRE>
-__device__ __forceinline__ void slot_fast(const GridC &g, const FieldP<T> &f, const GroupRows &G, const int (&rowc)[4],
-                                          const T (&rho)[4], const T (&rtr)[4], int src, int pre, int seg, int n1,
+template <typename T, int S, int FT, bool PRE, int NK>
+__device__ __forceinline__ void slot_fast(const GridC &g, const FieldP<T> &f, const GroupRows &G, const int (&rowc)[NK],
+                                          const T (&rho)[NK], const T (&rtr)[NK], int src, int pre, int seg, int n1,
                                           int aux, T q, T qd, T dinv, const T (&qsun)[S], const T (&hv)[S],
-                                          T (&kv)[4], T (&acc_s)[4], T (&acc_g)[4][S]) {
+                                          T (&kv)[NK], T (&acc_s)[NK], T (&acc_g)[NK][S]) {
     constexpr int RS = srec_stride(S);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < NK; ++k) {
         const int rp = G.rp[k], j = rp + src;
         T ep = T(1);
         if (PRE) ep = fast_exp_neg<T>(__ldg(f.tseg + pre + rp));
@@ -879,14 +879,28 @@ inline size_t asm0_smem(const GridC &g) {
     const size_t red = (size_t)W * (4 + 4 * g.S) * 32 * sizeof(T);
     return desc > red ? desc : red;
 }
-template <typename T, int S, int W, int MINB>
+// NK: row blocks (of 32 rows) a block takes of its group: 4, or 1 with four
+// blocks per group where the grid has too few groups to fill the GPU (the
+// 16^3 plume: 34 groups; FP64 rows cost 16 issue slots per operation, so the
+// plain 8^3 scene's 9 groups kept 9 SMs busy for 63 us).  A row's sums do not
+// depend on NK.
+template <typename T, int S, int W, int MINB, int NK>
 __global__ void __launch_bounds__(32 * W, MINB)
     k_asm0(GridC g, GraphP gp, FieldP<T> f, ViewC vc) {
     constexpr int RS = srec_stride(S);
     constexpr int NW = aslot_words<T>();
     extern __shared__ __align__(16) unsigned char asm0_dyn[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const GroupRows G = group_rows(g, gp, blockIdx.x);
+    GroupRows G = group_rows(g, gp, blockIdx.x / (4 / NK));
+    const int kb = NK == 4 ? 0 : blockIdx.x % (4 / NK) * NK;  // first row block
+    if constexpr (NK == 1) {
+#pragma unroll
+        for (int k = 1; k < 4; ++k)
+            if (k == kb) {
+                G.row[0] = G.row[k];
+                G.rp[0] = G.rp[k];
+            }
+    }
     const bool ground_row = G.z == g.nz;
     int4 *sdesc = reinterpret_cast<int4 *>(asm0_dyn);
     T *sconst = reinterpret_cast<T *>(sdesc + (size_t)NW * G.nt);
@@ -894,10 +908,10 @@ __global__ void __launch_bounds__(32 * W, MINB)
     stage_template<T, S>(g, gp, f, G.t0, G.nt, ground_row, sdesc, sconst);
     __syncthreads();
     const T rt_lamb = dsqrt<T>((T)(vc.albedo * __longlong_as_double((long long)*f.mus_max_bits)));
-    T rho[4], rtr[4];
-    int rowc[4];
+    T rho[NK], rtr[NK];
+    int rowc[NK];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < NK; ++k) {
         rowc[k] = G.row[k] >= 0 ? G.row[k] : G.z * g.nxy;  // rows past the layer's end read a valid node
         rtr[k] = __ldg(f.rt_h + G.rp[k]);
         if (!ground_row) {
@@ -907,11 +921,13 @@ __global__ void __launch_bounds__(32 * W, MINB)
             rho[k] = (T)vc.albedo;
         }
     }
-    T acc_s[4] = {T(0), T(0), T(0), T(0)}, acc_g[4][S];
+    T acc_s[NK], acc_g[NK][S];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < NK; ++k)
 #pragma unroll
         for (int sp = 0; sp < S; ++sp) acc_g[k][sp] = T(0);
+#pragma unroll
+    for (int k = 0; k < NK; ++k) acc_s[k] = T(0);
     T *vout = f.val + G.vb + 4 * lane;
     for (int t = w; t < G.nt; t += W) {
         int4 a0, a1, a2;
@@ -942,31 +958,31 @@ __global__ void __launch_bounds__(32 * W, MINB)
         const int ft = (bits >> 13) & 3;
         const int pre_n = taps & 0xff, seg_n = (taps >> 8) & 0xff, hit_n = (taps >> 16) & 0xff;
         const T qd = q * dinv;
-        T kv[4];
+        T kv[NK];
         if (ft == 1) {
             if (has_pre)
-                slot_fast<T, S, 1, true>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 1, true, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                          acc_s, acc_g);
             else
-                slot_fast<T, S, 1, false>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 1, false, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                           acc_s, acc_g);
         } else if (ft == 2) {
             if (has_pre)
-                slot_fast<T, S, 2, true>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 2, true, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                          acc_s, acc_g);
             else
-                slot_fast<T, S, 2, false>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 2, false, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                           acc_s, acc_g);
         } else if (ft == 3) {
             if (has_pre)
-                slot_fast<T, S, 3, true>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 3, true, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                          acc_s, acc_g);
             else
-                slot_fast<T, S, 3, false>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
+                slot_fast<T, S, 3, false, NK>(g, f, G, rowc, rho, rtr, src, pre, seg, n1, aux, q, qd, dinv, qsun, hv, kv,
                                           acc_s, acc_g);
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < NK; ++k) {
                 const int rp = G.rp[k];
                 const int j = rp + src;
                 // deposit fraction P of the slot (chain lumping of what lies beyond)
@@ -1027,20 +1043,21 @@ __global__ void __launch_bounds__(32 * W, MINB)
                 for (int sp = 0; sp < S; ++sp) acc_g[k][sp] += hv[sp] * sun;
             }
         }
-        st_quad_cs(vout + (size_t)t * kGroup, kv);
+        if constexpr (NK == 4) st_quad_cs(vout + (size_t)t * kGroup, kv);
+        else __stcs(vout + (size_t)t * kGroup + kb, kv[0]);
     }
     __syncthreads();  // every warp is done with the staged template
-    T(*sh)[4 + 4 * S][32] = reinterpret_cast<T(*)[4 + 4 * S][32]>(asm0_dyn);
+    T(*sh)[NK + NK * S][32] = reinterpret_cast<T(*)[NK + NK * S][32]>(asm0_dyn);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < NK; ++k) {
         sh[w][k][lane] = acc_s[k];
 #pragma unroll
-        for (int sp = 0; sp < S; ++sp) sh[w][4 + 4 * sp + k][lane] = acc_g[k][sp];
+        for (int sp = 0; sp < S; ++sp) sh[w][NK + NK * sp + k][lane] = acc_g[k][sp];
     }
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < NK; ++k) {
             if (G.row[k] < 0) continue;
             T a = T(0);
 #pragma unroll
@@ -1052,7 +1069,7 @@ __global__ void __launch_bounds__(32 * W, MINB)
                 for (int sp = 0; sp < S; ++sp) {
                     T c = T(0);
 #pragma unroll
-                    for (int qq = 0; qq < W; ++qq) c += sh[qq][4 + 4 * sp + k][lane];
+                    for (int qq = 0; qq < W; ++qq) c += sh[qq][NK + NK * sp + k][lane];
                     b += f.wsp[(size_t)sp * g.n_atm + G.row[k]] * c;
                 }
                 f.gsun[G.row[k]] = b;
@@ -1123,15 +1140,20 @@ void launch_assemble_rows(cudaStream_t st, const GridC &g, const GraphP &gp, con
     const int nb = (g.nz + 1) * g.gpl;
     constexpr int W0 = TK_ASM0_W, B0 = TK_ASM0_MINB;
     const size_t sm = asm0_smem<T, W0>(g);
-    auto go = [&](auto kern) {
-        if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        kern<<<nb, 32 * W0, sm, st>>>(g, gp, f, vc);
+    // four blocks per group while they still run in one wave (3 blocks per SM)
+    int dev = 0, nsm = 0;
+    const bool split = cudaGetDevice(&dev) == cudaSuccess &&
+                       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && 4 * nb <= 3 * nsm;
+    auto go = [&](auto kern, auto kern1) {
+        auto k = split ? kern1 : kern;
+        if (sm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k<<<split ? 4 * nb : nb, 32 * W0, sm, st>>>(g, gp, f, vc);
     };
     switch (g.S) {  // the species count as a compile-time constant
-        case 1: go(k_asm0<T, 1, W0, B0>); break;
-        case 2: go(k_asm0<T, 2, W0, B0>); break;
-        case 3: go(k_asm0<T, 3, W0, B0>); break;
-        default: go(k_asm0<T, 4, W0, B0>); break;
+        case 1: go(k_asm0<T, 1, W0, B0, 4>, k_asm0<T, 1, W0, B0, 1>); break;
+        case 2: go(k_asm0<T, 2, W0, B0, 4>, k_asm0<T, 2, W0, B0, 1>); break;
+        case 3: go(k_asm0<T, 3, W0, B0, 4>, k_asm0<T, 3, W0, B0, 1>); break;
+        default: go(k_asm0<T, 4, W0, B0, 4>, k_asm0<T, 4, W0, B0, 1>); break;
     }
     if (launches) *launches += 1;
 }
