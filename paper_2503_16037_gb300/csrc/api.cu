@@ -160,10 +160,21 @@ struct tursca_scene {
         tk::PsPlan plan;
         int2 *tpos = nullptr;
         int *run = nullptr;
+        // scenes without a plan: the rounds of the streamed passes (rd_nb = 0: none)
+        int *rd_first = nullptr, *rd_own = nullptr, *rd_off = nullptr;
+        int4 *rd_round = nullptr;
+        int2 *rd_chunk = nullptr;
+        int rd_nb = 0, rd_tl = 0, rd_nc = 0, rd_near = 0;
     };
     PsDev ps, psT;
     double *ps_part = nullptr;
     unsigned char *ps_ctl = nullptr;
+    // BiCGStab pass by pass: two vectors, block sums, the state on the device
+    // and the events of its read-backs (allocated with the first use)
+    void *bi_v = nullptr, *bi_t = nullptr;
+    double *bi_part = nullptr;
+    unsigned char *bi_state = nullptr;
+    cudaEvent_t bi_ev[2] = {nullptr, nullptr};
     bool x_pair = false;  // xh holds x in FP32 (of the forward solve)
     // the serving loop's batcher of solves (null: own launches)
     tk::SolveBatcher *batcher = nullptr;
@@ -358,10 +369,24 @@ tk::GridC grid_c(const tursca_scene *sc) {
     g.npad = (long long)(g.nz + 1) * g.lp;
     g.stage = (sc->stage_values && sc->d.precision != TURSCA_FP64 && tk::stage_fits(G.max_row)) ? 1 : 0;
     g.tl = sc->gather_tile ? sc->tile_tl : 0;
+    // (options that name how the passes run select those passes)
+    g.run = sc->ps.rd_nb > 0 && sc->wq_auto && !g.stage ? 1 : 0;
     g.hx = sc->d.hx;
     g.hy = sc->d.hy;
     g.hz = sc->d.hz;
     return g;
+}
+
+void set_rounds(tk::GraphP &p, const tursca_scene::PsDev &d) {
+    p.rd_first = d.rd_first;
+    p.rd_round = d.rd_round;
+    p.rd_chunk = d.rd_chunk;
+    p.rd_own = d.rd_own;
+    p.rd_off = d.rd_off;
+    p.rd_nb = d.rd_nb;
+    p.rd_tl = d.rd_tl;
+    p.rd_nc = d.rd_nc;
+    p.rd_near = d.rd_near;
 }
 
 tk::GraphP graph_p(const tursca_scene *sc) {
@@ -403,6 +428,7 @@ tk::GraphP graph_p(const tursca_scene *sc) {
     p.aslot = sc->aslot;
     p.tap_h = sc->tap_h;
     p.dir_h = sc->dir_h;
+    set_rounds(p, sc->ps);
     for (int k = 0; k < 2; ++k) {
         p.run_g[k] = sc->run_g[k];
         p.run_v[k] = sc->run_v[k];
@@ -769,6 +795,61 @@ tursca_status gmres(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &gp, 
     return TURSCA_OK;
 }
 
+// BiCGStab on (I - K) d = b, b = r64, to ||b - (I - K) d|| <= tol ||b|| (the
+// recursion's residual) in at most maxit products, then x += d with the FP32
+// pair of x.  norm: ||r64||.  Steps are queued kBiChunk at a time, one chunk
+// ahead of the read-back of the state; the passes after the end return at
+// once.  *ok false: the iteration broke down and x is unchanged.
+constexpr int kBiChunk = 1;
+template <typename T>
+tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &gp, const T *val, double norm,
+                       double tol, int maxit, double *x, float *xh, float *xl, SolveState &ss, bool *ok) {
+    const int n = (int)g.npad;
+    *ok = false;
+    if (!sc->bi_v) {
+        CK(dalloc(sc->allocs, sc->bi_t, (size_t)n * sizeof(T)), "alloc bicgstab");
+        CK(dalloc(sc->allocs, sc->bi_part, tk::bi_part_words(g) * sizeof(double)), "alloc bicgstab");
+        CK(dalloc(sc->allocs, sc->bi_state, 256), "alloc bicgstab");
+        for (int k = 0; k < 2; ++k)
+            if (!sc->bi_ev[k]) CK(cudaEventCreateWithFlags(&sc->bi_ev[k], cudaEventDisableTiming), "event");
+        CK(dalloc(sc->allocs, sc->bi_v, (size_t)n * sizeof(T)), "alloc bicgstab");
+    }
+    T *b = (T *)sc->b, *r = (T *)sc->d1, *p = (T *)sc->w, *d = (T *)sc->d0, *v = (T *)sc->bi_v, *t = (T *)sc->bi_t;
+    tk::BiState<T> *st = (tk::BiState<T> *)sc->bi_state;
+    // at unit scale, so that FP32 squares neither overflow nor underflow
+    const int ex = std::min(120, std::max(-120, std::ilogb(norm)));
+    const double bb = std::ldexp(norm, -ex) * std::ldexp(norm, -ex);
+    tk::launch_bi_start<T>(sc->st, n, sc->r64, std::ldexp(1.0, -ex), bb, tol * tol * bb, b, r, p, d, st);
+    sc->launches++;
+    const int chunks = std::max(1, (maxit + 2 * kBiChunk - 1) / (2 * kBiChunk));
+    tk::BiState<T> *h = (tk::BiState<T> *)(sc->hred + 192);  // two read-back slots of 64 bytes
+    static_assert(sizeof(tk::BiState<T>) <= 64, "read-back slots");
+    auto slot = [&](int c) { return (tk::BiState<T> *)((char *)h + (c & 1) * 64); };
+    for (int c = 0; c <= chunks; ++c) {
+        if (c < chunks) {
+            const int pi = prof_begin(sc, P_GPROD);
+            for (int k = 0; k < kBiChunk; ++k)
+                tk::launch_bi_step<T>(sc->st, g, gp, val, b, r, p, v, t, d, sc->bi_part, st);
+            prof_end(sc, pi, 2 * kBiChunk);
+            sc->launches += 6 * kBiChunk;
+            CK(cudaMemcpyAsync(slot(c), st, sizeof(*st), cudaMemcpyDeviceToHost, sc->st), "d2h");
+            CK(cudaEventRecord(sc->bi_ev[c & 1], sc->st), "event");
+        }
+        if (c == 0) continue;
+        CK(cudaEventSynchronize(sc->bi_ev[(c - 1) & 1]), "sync");
+        if (slot(c - 1)->done || c == chunks) {
+            const tk::BiState<T> e = *slot(c - 1);
+            ss.iters += 2 * e.steps;
+            if (!std::isfinite((double)e.rn)) return TURSCA_OK;
+            break;
+        }
+    }
+    tk::launch_bi_end<T>(sc->st, n, d, std::ldexp(1.0, ex), x, xh, xl);
+    sc->launches++;
+    *ok = true;
+    return TURSCA_OK;
+}
+
 // The solve's schedule constants: the power sweeps of the first refinement
 // and the lower end of the Chebyshev interval as a fraction of its upper end.
 // Chosen on a model of this loop (float32 K from an FP64 reference, the same
@@ -856,6 +937,25 @@ tursca_status upload_persist(tursca_scene *sc, tursca_scene::PsDev &P, const std
         }
         CK(cudaStreamSynchronize(sc->st), "sync");  // tp dies here
     }
+    if (plan.nb == 0 && sc->es == 4) {
+        const tk::RunPlan rp = tk::run_plan(tk::ps_geom(g), nt, nsm, 46 * 1024);
+        if (rp.nb > 0) {
+            std::vector<int> ro(tp.size());
+            for (int z = 0; z <= g.nz; ++z)
+                for (int i = tstart[z]; i < tstart[z + 1]; ++i)
+                    ro[i] = (tp[i].x - (z == g.nz ? 0 : z + 1)) * rp.tl + tp[i].y + g.H * g.nxp + g.H;
+            CK(upload(sc, sc->allocs, P.rd_first, rp.first.data(), rp.first.size() * sizeof(int)), "upload rounds");
+            CK(upload(sc, sc->allocs, P.rd_round, rp.round.data(), rp.round.size() * sizeof(int)), "upload rounds");
+            CK(upload(sc, sc->allocs, P.rd_chunk, rp.chunk.data(), rp.chunk.size() * sizeof(int)), "upload rounds");
+            CK(upload(sc, sc->allocs, P.rd_own, rp.own.data(), rp.own.size() * sizeof(int)), "upload rounds");
+            CK(upload(sc, sc->allocs, P.rd_off, ro.data(), ro.size() * sizeof(int)), "upload rounds");
+            CK(cudaStreamSynchronize(sc->st), "sync");  // the host tables die here
+            P.rd_nb = rp.nb;
+            P.rd_tl = rp.tl;
+            P.rd_nc = rp.nc;
+            P.rd_near = rp.near;
+        }
+    }
     P.plan = std::move(plan);
     return TURSCA_OK;
 }
@@ -897,6 +997,7 @@ tursca_status persist_solve(tursca_scene *sc, const SolveIO<T> &io, double rtol,
     J.wpg = P.wpg;
     J.it = P.it;
     J.kcap = P.kcap;
+    J.near = P.near;
     CK(cudaMemsetAsync(sc->ps_ctl, 0, 256, sc->st), "memset plan");
     const int pi = prof_begin(sc, P_PERSIST);
     bool launched = false;
@@ -989,6 +1090,9 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
         const tursca_status e = persist_solve<T>(sc, io, rtol, max_iter, info, &done);
         if (e || done) return e;
     }
+    // the automatic choice goes on with BiCGStab where the other solvers take
+    // GMRES (until BiCGStab breaks down, which hands over to GMRES)
+    bool bi = solver == TURSCA_SOLVER_AUTO;
     if (solver == TURSCA_SOLVER_AUTO) solver = fp64 ? TURSCA_SOLVER_GMRES : TURSCA_SOLVER_CHEBYSHEV;
     auto ensure_basis = [&]() -> tursca_status {
         int m = fp64 ? 40 : TK_GMRES_M32;
@@ -1047,7 +1151,8 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
             else if (rho + widen >= 0.85 || use_gmres)
                 kind = TURSCA_SOLVER_GMRES;
         }
-        if (power || kind != TURSCA_SOLVER_CHEBYSHEV) {
+        if (kind == TURSCA_SOLVER_GMRES && bi) kind = TURSCA_SOLVER_BICGSTAB;
+        if (power || (kind != TURSCA_SOLVER_CHEBYSHEV && kind != TURSCA_SOLVER_BICGSTAB)) {
             tk::launch_convert<double, T>(sc->st, n, sc->r64, bb);
             sc->launches++;
         }
@@ -1108,6 +1213,27 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
             dd = d;
             x_done = true;
             ss.solver = TURSCA_SOLVER_CHEBYSHEV;
+        } else if (kind == TURSCA_SOLVER_BICGSTAB) {
+            if (sn < 0.0) {
+                rs = read_red<T>(sc, 5);
+                if (rs) return rs;
+                sn = std::sqrt(sc->hred[4]);
+                if (sn == 0.0) {  // s = 0: x = 0
+                    rel = 0.0;
+                    break;
+                }
+            }
+            const double tol = std::max(0.3 * rtol / rel, fp64 ? 1e-15 : 2e-6);
+            bool ok = false;
+            const tursca_status e = bicgstab<T>(sc, g, gp, val, rel * sn, tol, budget, io.x, ds ? sc->xh : nullptr,
+                                                ds ? sc->xl : nullptr, ss, &ok);
+            if (e) return e;
+            if (!ok) {
+                bi = false;
+                continue;
+            }
+            x_done = true;
+            ss.solver = TURSCA_SOLVER_BICGSTAB;
         } else if (kind == TURSCA_SOLVER_GMRES) {
             tursca_status e = ensure_basis();
             if (e) return e;
@@ -1154,6 +1280,8 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
             double avg = (f > 0 && f < 1) ? std::pow(f, 1.0 / (n1 + 1)) : 0.0;
             rho = std::min(0.9999, std::max(est, avg));
             ss.rho = rho;
+        } else if (kind == TURSCA_SOLVER_BICGSTAB) {
+            if (!(f < 0.5) && rel > rtol) bi = false;
         } else if (kind == TURSCA_SOLVER_CHEBYSHEV) {
             if (f > std::max(30.0 * predicted, 3.0 * floor32) && rel > rtol) {
                 // the interval missed part of the spectrum: widen it once toward 1,
@@ -1304,6 +1432,7 @@ tursca_status do_adjoint(tursca_scene *sc, const void *dJ_dL, void *dJ_dmu_abs) 
     gpT.tflat = sc->flatT;
     gpT.ttile = sc->ttileT;  // gather tiles of the K^T templates
     gpT.tlay = sc->tlayT;
+    set_rounds(gpT, sc->psT);
     tk::AdjP<T> ad;
     T **slot[10] = {&ad.Ebar, &ad.Ebar_h, &ad.e1bar, &ad.e1bar_h, &ad.xbar,
                     &ad.mubar, &ad.mubar_h, &ad.tsegbar, &ad.tinfbar, &ad.tinfgbar};
@@ -1323,6 +1452,7 @@ tursca_status do_adjoint(tursca_scene *sc, const void *dJ_dL, void *dJ_dmu_abs) 
     SolveIO<T> io;
     g.stage = 0;
     g.tl = sc->gather_tile ? sc->tile_tlT : 0;
+    g.run = sc->psT.rd_nb > 0 && sc->wq_auto ? 1 : 0;
     io.g = g;
     io.gp = gpT;
     io.val = (const T *)sc->valT;
@@ -1744,6 +1874,8 @@ tursca_status tursca_scene_destroy(tursca_scene *sc) {
     if (sc->topk_hist_h) cudaFreeHost(sc->topk_hist_h);
     if (sc->bready) cudaEventDestroy(sc->bready);
     if (sc->bdone) cudaEventDestroy(sc->bdone);
+    for (cudaEvent_t e : sc->bi_ev)
+        if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : sc->ev) cudaEventDestroy(e);
     for (int i = 0; i < 3; ++i)
         if (sc->aux[i]) cudaStreamDestroy(sc->aux[i]);

@@ -78,6 +78,7 @@ struct GridC {
     long long npad;              // (nz + 1) * lp
     int stage;                   // 1: FP32 sweeps stage each group's values in shared memory
     int tl;                      // floats per layer of a group's gather tile (0: passes gather from global memory)
+    int run;                     // 1: FP32 passes run as rounds of groups on persistent blocks (GraphP::rd)
     double hx, hy, hz;
 };
 
@@ -129,6 +130,17 @@ struct GraphP {
     // lattice segments of the canonical directions, for the segment-table
     // kernel: per canonical direction (first entry in ctap, tap count, u_z, 0)
     // and the graph tap index of each of its taps
+    // Rounds of the streamed passes over large scenes (persist_plan.h): block b
+    // runs rounds rd_first[b] .. rd_first[b + 1], each (first group, groups,
+    // first chunk, chunks); rd_chunk: (haloed index, elements) of each chunk;
+    // rd_own: per round and group the chunk of its own rows; rd_off: per
+    // template entry the tile offset from the row's own chunk
+    const int *rd_first;
+    const int4 *rd_round;
+    const int2 *rd_chunk;
+    const int *rd_own;
+    const int *rd_off;
+    int rd_nb, rd_tl, rd_nc, rd_near;
     const int4 *cseg;
     const int *ctap;
     int nctap;                     // total taps of the canonical directions
@@ -382,6 +394,27 @@ template <typename T>
 void launch_axpby(cudaStream_t st, int n, double a, const T *x, double b, const T *y, T *out);  // out = a x + b y
 template <typename T>
 void launch_imk(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const T *x, T *y);  // y = x - K x
+
+// BiCGStab pass by pass: the state of a solve of (I - K) d = b (device)
+template <typename T>
+struct BiState {
+    T rho, alpha, best, stop2, rn;  // rn: the last step's ||r||^2
+    int done, steps, since;
+    unsigned left;  // blocks of the current step's last kernel that have finished
+};
+// b = r64 * down (a power of two), r = p = b, d = 0; bb = ||b||^2, stop2 the
+// squared residual norm to reach
+template <typename T>
+void launch_bi_start(cudaStream_t st, int n, const double *r64, double down, double bb, double stop2, T *b, T *r,
+                     T *p, T *d, BiState<T> *state);
+// one step (two products); part: bi_part_words(g) doubles
+template <typename T>
+void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const T *r0, T *r, T *p, T *v,
+                    T *t, T *d, double *part, BiState<T> *state);
+// x += up d, with the FP32 pair of x when xh is set
+template <typename T>
+void launch_bi_end(cudaStream_t st, int n, const T *d, double up, double *x, float *xh, float *xl);
+size_t bi_part_words(const GridC &g);
 
 // ---- adjoint (kernels_adjoint.cu)
 // Transposed templates of K (rows = sources), see tg::Transposed

@@ -36,6 +36,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "dots.cuh"
 #include "kern.h"
 #include "persist.h"
 
@@ -67,94 +68,6 @@ __device__ __forceinline__ bool ps_barrier(unsigned *bar, unsigned target, int *
     return *ok_sh != 0;
 }
 
-// ---- exact-product sums: FP32 pairs for FP32 scenes, FP64 otherwise
-template <typename T>
-struct Dot;
-template <>
-struct Dot<float> {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float p = __fmul_rn(a, b);
-        add2(p, fmaf(a, b, -p));
-    }
-    __device__ __forceinline__ void add2(float p, float e) {
-        const float s = __fadd_rn(h, p);
-        const float bb = __fsub_rn(s, h);
-        const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-        h = s;
-        l = __fadd_rn(l, __fadd_rn(err, e));
-    }
-    __device__ __forceinline__ Dot xch(int o) const {
-        Dot r;
-        r.h = __shfl_xor_sync(0xffffffffu, h, o);
-        r.l = __shfl_xor_sync(0xffffffffu, l, o);
-        return r;
-    }
-    __device__ __forceinline__ void join(const Dot &q) { add2(q.h, q.l); }
-    // c * (this) added to d, c exact
-    __device__ __forceinline__ void add_to(Dot &d, float c) const {
-        d.add(c, h);
-        d.l = fmaf(c, l, d.l);
-    }
-    __device__ __forceinline__ float value() const { return h + l; }
-    __device__ __forceinline__ double bits() const {
-        return __hiloint2double(__float_as_int(h), __float_as_int(l));
-    }
-    __device__ __forceinline__ static Dot from(double b) {
-        Dot d;
-        d.h = __int_as_float(__double2hiint(b));
-        d.l = __int_as_float(__double2loint(b));
-        return d;
-    }
-};
-template <>
-struct Dot<double> {
-    double h = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { h = fma(a, b, h); }
-    __device__ __forceinline__ Dot xch(int o) const {
-        Dot r;
-        r.h = __shfl_xor_sync(0xffffffffu, h, o);
-        return r;
-    }
-    __device__ __forceinline__ void join(const Dot &q) { h += q.h; }
-    __device__ __forceinline__ void add_to(Dot &d, double c) const { d.h = fma(c, h, d.h); }
-    __device__ __forceinline__ double value() const { return h; }
-    __device__ __forceinline__ double bits() const { return h; }
-    __device__ __forceinline__ static Dot from(double b) {
-        Dot d;
-        d.h = b;
-        return d;
-    }
-};
-
-// N = 8 sums over the warp in 9 joins: the lanes split the sums between
-// them stage by stage; lane i ends with sum number (i >> 2)
-template <typename T>
-__device__ __forceinline__ Dot<T> warp_dots8(Dot<T> (&v)[8]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int st = 4; st >= 1; st >>= 1) {
-        const int o = 4 * st;  // 16, 8, 4
-        const bool hi = lane & o;
-#pragma unroll
-        for (int i = 0; i < st; ++i) {
-            const Dot<T> give = hi ? v[i] : v[i + st];
-            Dot<T> keep = hi ? v[i + st] : v[i];
-            keep.join(give.xch(o));
-            v[i] = keep;
-        }
-    }
-    v[0].join(v[0].xch(2));
-    v[0].join(v[0].xch(1));
-    return v[0];
-}
-template <typename T>
-__device__ __forceinline__ Dot<T> warp_dot1(Dot<T> v) {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v.join(v.xch(o));
-    return v;
-}
-
 // the FP32-pair accumulation of the refinement residual (see OpResidDS)
 __device__ __forceinline__ void ps_ds(float &hi, float &lo, float v, float xh, float xl) {
     const float p = __fmul_rn(v, xh);
@@ -180,19 +93,15 @@ __device__ __forceinline__ void ps_quad(const double *p, double (&v)[4]) {
     v[2] = b.x;
     v[3] = b.y;
 }
-__device__ __forceinline__ void ps_quad_g(const float *p, float (&v)[4]) {
-    const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = q.z;
-    v[3] = q.w;
+// the same from global memory, with an L2 policy
+__device__ __forceinline__ void ps_quad_g(const float *p, unsigned long long pol, float (&v)[4]) {
+    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+        : "l"(p), "l"(pol));
 }
-__device__ __forceinline__ void ps_quad_g(const double *p, double (&v)[4]) {
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = b.x;
-    v[3] = b.y;
+__device__ __forceinline__ void ps_quad_g(const double *p, unsigned long long pol, double (&v)[4]) {
+    asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v[0]), "=d"(v[1]) : "l"(p), "l"(pol));
+    asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v[2]), "=d"(v[3]) : "l"(p + 2), "l"(pol));
 }
 
 // what a block knows of one of its groups
@@ -201,7 +110,7 @@ struct PsGroup {
     int nt, zz, z;  // slots, position, layer
     int seg;        // strip
     int own;        // tile offset of the group's own rows (added to rlt)
-    int ks;         // its values in shared memory (slot rows), -1: streamed from L2
+    int ks;         // its values in shared memory (slot rows), -1: streamed from L2, -2: from HBM
 };
 
 struct PsShared {
@@ -273,6 +182,14 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
         }
         for (int i = 0; i < S.nseg; ++i) S.segk[i] = min(4, (nxy - S.segq[i] * kGroup + 31) / 32);
         const int er = ps_first_resident(0, nl, J.kcap, wpg, (int)sizeof(T), [&](int l) { return S.grp[l].nt; });
+        // streamed groups beyond what L2 holds for all blocks come from HBM
+        // every time, marked to leave L2 first, so that they do not push the
+        // others out
+        int near = J.near;
+        for (int l = er - 1; l >= 0; --l) {
+            near -= S.grp[l].nt;
+            if (near < 0) S.grp[l].ks = -2;
+        }
         int ks = 0;
         for (int l = er; l < nl; ++l) {
             S.grp[l].ks = ks;
@@ -317,11 +234,17 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
     auto stream = [&](int l) -> const T * {  // the warp's first value of group l, null: not streamed
         return l < nl && S.grp[l].ks < 0 ? val + S.grp[l].vb + wi * kGroup + 4 * lane : nullptr;
     };
+    unsigned long long keep, pass_by;
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
+    auto policy = [&](int l) { return l < nl && S.grp[l].ks == -2 ? pass_by : keep; };
     {
-        const T *p = stream(set < nsets ? set : nl);
+        const int l = set < nsets ? set : nl;
+        const T *p = stream(l);
         if (p) {
+            const unsigned long long pol = policy(l);
 #pragma unroll
-            for (int i = 0; i < PF; ++i) ps_quad_g(p + i * step, pf[i]);
+            for (int i = 0; i < PF; ++i) ps_quad_g(p + i * step, pol, pf[i]);
         }
     }
     // the first EB tile elements of this thread: where they come from
@@ -491,6 +414,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
             const int *to = toff + (l * wpg + wi) * it;
             const int n = ps_padded(G.nt, wpg, (int)sizeof(T)) / wpg;  // the warp's slots
             const T *nx_ = stream(l + nsets < nl ? l + nsets : set);
+            const unsigned long long pol = policy(l), poln = policy(l + nsets < nl ? l + nsets : set);
             if (G.ks >= 0) {  // in shared memory
                 const T *ksm = sK + (size_t)G.ks * kGroup + wi * kGroup + 4 * lane;
                 auto round = [&](auto cnt_c, int i0) {
@@ -522,12 +446,13 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
                 }
                 if (nx_) {
 #pragma unroll
-                    for (int i = 0; i < PF; ++i) ps_quad_g(nx_ + i * step, pf[i]);
+                    for (int i = 0; i < PF; ++i) ps_quad_g(nx_ + i * step, poln, pf[i]);
                 }
             } else {  // streamed from L2: PF slots are there; each one's successor is requested as it is used
                 const T *kg = val + G.vb + wi * kGroup + 4 * lane;
                 for (int i0 = 0; i0 < n; i0 += PF) {
                     const T *p = i0 + PF < n ? kg + (i0 + PF) * step : nx_ ? nx_ : kg;
+                    const unsigned long long pp = i0 + PF < n || !nx_ ? pol : poln;
                     int off[PF];
 #pragma unroll
                     for (int i = 0; i < PF; i += 4) {
@@ -540,7 +465,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
 #pragma unroll
                     for (int i = 0; i < PF; ++i) {
                         if (sizeof(T) == 4 || i0 + i < n) add(pf[i], off[i]);
-                        ps_quad_g(p + i * step, pf[i]);
+                        ps_quad_g(p + i * step, pp, pf[i]);
                     }
                 }
             }

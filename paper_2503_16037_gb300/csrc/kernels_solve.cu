@@ -8,6 +8,7 @@
 // fixed-order trees.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -151,6 +152,53 @@ struct OpSweepPow {
         store_h(y, G, k, vv);
         xu.apply(G, k, vv);
         return (double)(dd * dd);
+    }
+};
+
+// The two products of a BiCGStab step: y = x - K x with its dot products.
+// ND 1: r0.y; ND 5: y.x, y.y, r0.x, r0.y, x.x
+template <typename T, int ND>
+struct OpBi {
+    using A = T;
+    static constexpr int NA = 4;
+    static constexpr bool kPart = false;
+    static constexpr int kDots = ND;
+    struct Pre {
+        T u, q0;
+    };
+    const T *x, *r0;
+    T *y;
+    double *part;
+    size_t pstride;
+    const BiState<T> *st;
+    static constexpr int kTile = sizeof(T) == 4 ? 1 : 0;
+    __device__ __forceinline__ bool skip() const { return *(volatile const int *)&st->done != 0; }
+    __device__ __forceinline__ const T *gsrc(int) const { return x; }
+    __device__ __forceinline__ void add_t(A *a, int k, T v, const T *s, int, NoSlot) const { a[k] += v * s[0]; }
+    __device__ __forceinline__ NoSlot slot(const GraphP &, int) const { return NoSlot(); }
+    __device__ __forceinline__ void add(A *a, int k, T v, int j, NoSlot) const { a[k] += v * __ldg(x + j); }
+    __device__ __forceinline__ Pre pre(const GroupRows &G, int k) const {
+        Pre p;
+        p.u = x[G.rp[k]];
+        p.q0 = r0[G.rp[k]];
+        return p;
+    }
+    template <int W>
+    __device__ __forceinline__ static void combine_row(const A (*sh)[NA][32], int lane, int k, A *a) {
+        sum_word<W, A, NA>(sh, lane, k, a);
+    }
+    __device__ __forceinline__ void finish_dots(const GroupRows &G, int k, const A *a, const Pre &p, Dot<T> *d) const {
+        const T v = p.u - a[k];
+        store_h(y, G, k, v);
+        if constexpr (ND == 1) {
+            d[0].add(p.q0, v);
+        } else {
+            d[0].add(v, p.u);
+            d[1].add(v, v);
+            d[2].add(p.q0, p.u);
+            d[3].add(p.q0, v);
+            d[4].add(p.u, p.u);
+        }
     }
 };
 
@@ -615,6 +663,204 @@ void launch_finalize(cudaStream_t st, const double *part, int nblk, double *out)
 }
 
 // ---------------------------------------------------------------------------
+// BiCGStab pass by pass, for scenes too large for the persistent solve.  A
+// step is two passes over K (OpBi), each followed by the sums of its dot
+// products and one vector kernel; the step's scalars stay on the device
+// (every block of the vector kernels forms them from the sums), so steps are
+// queued ahead of the host, which only reads back the state every few steps.
+// Against GMRES(30) with I + K as preconditioner it needs no basis: on the
+// 128 x 128 x 40 cloud an Arnoldi step spent 107 us on orthogonalisation beside
+// its two passes of 72 us.
+constexpr int kBiParts = 8;  // blocks per sum
+template <typename T>
+__global__ void __launch_bounds__(512) k_bi_sums(const double *__restrict__ part, size_t stride, int n,
+                                                 double *__restrict__ out, const BiState<T> *st) {
+    __shared__ double sh[16];
+    pdl_trigger();
+    pdl_wait();
+    if (st->done) return;
+    const double *p = part + (size_t)blockIdx.y * stride;
+    Dot<T> v;
+    const int step = kBiParts * 512;
+#pragma unroll 4
+    for (int i = blockIdx.x * 512 + threadIdx.x; i < n; i += step) v.join(Dot<T>::from(__ldcg(p + i)));
+    v = warp_dot1<T>(v);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v.bits();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        Dot<T> t;
+        if (threadIdx.x < 16) t = Dot<T>::from(sh[threadIdx.x]);
+        t = warp_dot1<T>(t);
+        if (threadIdx.x == 0) out[blockIdx.y * kBiParts + blockIdx.x] = t.bits();
+    }
+}
+// the nd sums, by warps 0 .. nd - 1, into sh (synchronises)
+template <typename T>
+__device__ __forceinline__ void bi_total(const double *sums, int nd, double *sh) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < nd) {
+        Dot<T> v;
+        if (lane < kBiParts) v = Dot<T>::from(__ldcg(sums + w * kBiParts + lane));
+        v = warp_dot1<T>(v);
+        if (lane == 0) sh[w] = v.bits();
+    }
+    __syncthreads();
+}
+// b = r64 scaled by a power of two; r = p = b, d = 0; the state of a new solve
+template <typename T>
+__global__ void k_bi_start(int n, const double *__restrict__ r64, T down, T bb, T stop2, T *__restrict__ b,
+                           T *__restrict__ r, T *__restrict__ p, T *__restrict__ d, BiState<T> *st) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        BiState<T> s{};
+        s.rho = s.best = s.rn = bb;
+        s.stop2 = stop2;
+        *st = s;
+    }
+    if (i >= n) return;
+    const T v = down * (T)r64[i];
+    b[i] = v;
+    r[i] = v;
+    p[i] = v;
+    d[i] = T(0);
+}
+// alpha = rho / r0.v; d += alpha p; r <- s = r - alpha v
+template <typename T>
+__global__ void __launch_bounds__(256) k_bi_s(int n, const double *__restrict__ sums, const T *__restrict__ p,
+                                              const T *__restrict__ v, T *__restrict__ r, T *__restrict__ d,
+                                              BiState<T> *st) {
+    __shared__ double sh[8];
+    __shared__ T sa;
+    pdl_trigger();
+    pdl_wait();
+    if (st->done) return;
+    bi_total<T>(sums, 1, sh);
+    if (threadIdx.x == 0) {
+        const T r0v = Dot<T>::from(sh[0]).value();
+        sa = r0v != T(0) ? st->rho / r0v : T(0);
+        if (blockIdx.x == 0) st->alpha = sa;
+    }
+    __syncthreads();
+    const T a = sa;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        d[i] += a * p[i];
+        r[i] -= a * v[i];
+    }
+}
+// omega, beta and the new rho from the sums; d += omega s; r = s - omega t;
+// p = r + beta (p - omega v).  The last block to finish writes the state,
+// which the others read.
+template <typename T>
+__global__ void __launch_bounds__(256) k_bi_p(int n, const double *__restrict__ sums, const T *__restrict__ v,
+                                              const T *__restrict__ t, T *__restrict__ r, T *__restrict__ p,
+                                              T *__restrict__ d, BiState<T> *st) {
+    __shared__ double sh[8];
+    __shared__ T sv[4];
+    pdl_trigger();
+    pdl_wait();
+    if (st->done) return;
+    bi_total<T>(sums, 5, sh);
+    if (threadIdx.x == 0) {
+        const Dot<T> ts = Dot<T>::from(sh[0]), tt = Dot<T>::from(sh[1]), r0t = Dot<T>::from(sh[3]);
+        Dot<T> r0r = Dot<T>::from(sh[2]), rn = Dot<T>::from(sh[4]);
+        const T om = tt.value() > T(0) ? ts.value() / tt.value() : T(0);
+        r0t.add_to(r0r, -om);       // r0.r = r0.s - omega r0.t
+        ts.add_to(rn, T(-2) * om);  // r.r = s.s - 2 omega t.s + omega^2 t.t
+        Dot<T> ott;
+        tt.add_to(ott, om);
+        ott.add_to(rn, om);
+        sv[0] = om;
+        sv[2] = r0r.value();
+        sv[3] = rn.value();
+        const T rho = st->rho;
+        sv[1] = (rho != T(0) && om != T(0)) ? (sv[2] / rho) * (st->alpha / om) : T(0);
+    }
+    __syncthreads();
+    const T om = sv[0], be = sv[1];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const T s = r[i], rr = s - om * t[i];
+        d[i] += om * s;
+        p[i] = rr + be * (p[i] - om * v[i]);
+        r[i] = rr;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&st->left, 1u) + 1u == gridDim.x) {  // every block has read the old state
+            st->left = 0;
+            st->rho = sv[2];
+            st->rn = sv[3];
+            st->steps += 1;
+            if (sv[3] < st->best) {
+                st->best = sv[3];
+                st->since = 0;
+            } else {
+                st->since += 1;
+            }
+            if (!(sv[3] > st->stop2) || om == T(0) || !(fabs(be) > T(0)) || st->since > 40) st->done = 1;
+        }
+    }
+}
+// x += up * d, with the FP32 pair of the new x
+template <typename T>
+__global__ void k_bi_end(int n, const T *__restrict__ d, T up, double *__restrict__ x, float *__restrict__ xh,
+                         float *__restrict__ xl) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double v = x[i] + (double)(up * d[i]);
+    x[i] = v;
+    if (xh) {
+        const float h = (float)v;
+        xh[i] = h;
+        xl[i] = (float)(v - (double)h);
+    }
+}
+
+size_t bi_part_words(const GridC &g) { return (size_t)5 * sweep_blocks(g) + 8 * kBiParts; }
+
+template <typename T>
+void launch_bi_start(cudaStream_t st, int n, const double *r64, double down, double bb, double stop2, T *b, T *r,
+                     T *p, T *d, BiState<T> *state) {
+    k_bi_start<T><<<(n + 255) / 256, 256, 0, st>>>(n, r64, (T)down, (T)bb, (T)stop2, b, r, p, d, state);
+}
+template <typename T>
+void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const T *r0, T *r, T *p, T *v,
+                    T *t, T *d, double *part, BiState<T> *state) {
+    const int n = (int)g.npad, np = sweep_blocks(g);
+    double *sums = part + (size_t)5 * np;
+    // four blocks of 256 threads on each of 152 SMs, so that the next pass's
+    // blocks fit beside them and fetch their first values meanwhile
+    const int nb = std::min((n + 255) / 256, 608);
+    auto go = [&](auto kern, dim3 blocks, int threads, auto... args) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = blocks;
+        cfg.blockDim = dim3(threads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, kern, args...);
+    };
+    const double *cpart = part, *csums = sums;
+    const T *cp = p, *cv = v, *ct = t;
+    const BiState<T> *cst = state;
+    OpBi<T, 1> ov{p, r0, v, part, (size_t)np, state};
+    run_op(st, g, gp, val, ov, 0);
+    go(k_bi_sums<T>, dim3(kBiParts, 1), 512, cpart, (size_t)np, np, sums, cst);
+    go(k_bi_s<T>, dim3(nb), 256, n, csums, cp, cv, r, d, state);
+    OpBi<T, 5> ot{r, r0, t, part, (size_t)np, state};
+    run_op(st, g, gp, val, ot, 0);
+    go(k_bi_sums<T>, dim3(kBiParts, 5), 512, cpart, (size_t)np, np, sums, cst);
+    go(k_bi_p<T>, dim3(nb), 256, n, csums, cv, ct, r, p, d, state);
+}
+template <typename T>
+void launch_bi_end(cudaStream_t st, int n, const T *d, double up, double *x, float *xh, float *xl) {
+    k_bi_end<T><<<(n + 255) / 256, 256, 0, st>>>(n, d, (T)up, x, xh, xl);
+}
+
+// ---------------------------------------------------------------------------
 // Vector operations
 
 template <typename T, typename U>
@@ -766,6 +1012,16 @@ template <typename T>
 void launch_axpby(cudaStream_t st, int n, double a, const T *x, double b, const T *y, T *out) {
     k_axpby<T><<<(n + 255) / 256, 256, 0, st>>>(n, a, x, b, y, out);
 }
+
+#define BINST(T)                                                                                                   \
+    template void launch_bi_start<T>(cudaStream_t, int, const double *, double, double, double, T *, T *, T *, T *, \
+                                     BiState<T> *);                                                                \
+    template void launch_bi_step<T>(cudaStream_t, const GridC &, const GraphP &, const T *, const T *, T *, T *,   \
+                                    T *, T *, T *, double *, BiState<T> *);                                        \
+    template void launch_bi_end<T>(cudaStream_t, int, const T *, double, double *, float *, float *);
+BINST(float)
+BINST(double)
+#undef BINST
 
 #define INST(T)                                                                                                    \
     template void launch_spmv<T>(cudaStream_t, const GridC &, const GraphP &, const T *, const T *, const T *, T *); \

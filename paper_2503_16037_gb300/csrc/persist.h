@@ -36,7 +36,7 @@ struct PsJob {
     double rtol;
     int max_iter;
     int block0, nb;      // the job's blocks in the launch
-    int nl, tl, nchunk, wpg, it, kcap;
+    int nl, tl, nchunk, wpg, it, kcap, near;
 };
 
 PsGeom ps_geom(const GridC &g);

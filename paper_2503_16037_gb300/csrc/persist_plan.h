@@ -42,6 +42,7 @@ struct PsPlan {
     int wpg = 0;           // warps that share a group: warp wi adds its slots wi, wi + wpg, ...
     int it = 0;            // most slots of a warp and group (a multiple of 8)
     int kcap = 0;          // slot rows (128 values) of K a block can keep in shared memory
+    int near = 0;          // slot rows of a block's streamed groups that L2 can hold
     size_t smem = 0;       // dynamic shared memory
     std::vector<int> run;  // [nb + 1] first group of each block, in strip order
 };
@@ -173,5 +174,22 @@ constexpr size_t kPsPad = (size_t)2 * kPsW * 8 * kPsRows;
 // es: bytes of the compute type, fixed_smem: the kernel's static shared
 // memory.  nb = 0 when the scene does not fit.
 PsPlan ps_plan(const PsGeom &g, const std::vector<int> &nt, int es, int nsm, size_t smem_max, size_t fixed_smem);
+
+// ---- Rounds of the streamed passes (k_run in stage.cuh), for scenes the
+// persistent solve does not take: a block walks its groups in rounds of at most
+// kRunGroups consecutive ones (strip order) whose chunks fit a tile of nc.
+constexpr int kRunGroups = 8;     // groups of a round, two warps each
+constexpr int kRunMaxChunk = 20;  // chunks of a round's tile
+struct RunPlan {
+    int nb = 0;              // blocks (0: the passes run a block per group)
+    int tl = 0, nc = 0;      // elements per chunk, chunks per tile
+    int near = 0;            // rounds of each block whose values L2 can hold
+    std::vector<int> first;  // [nb + 1] first round of each block
+    std::vector<int> round;  // per round: first group, groups, first chunk, chunks
+    std::vector<int> chunk;  // per chunk: haloed index of its first element, elements
+    std::vector<int> own;    // [rounds][kRunGroups] the chunk of each group's own rows
+};
+// tile_bytes: shared memory one tile (of one vector) may take
+RunPlan run_plan(const PsGeom &g, const std::vector<int> &nt, int nsm, size_t tile_bytes);
 
 }  // namespace tk

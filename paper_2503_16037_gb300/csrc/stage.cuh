@@ -6,7 +6,9 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "dots.cuh"
 #include "kern.h"
+#include "persist_plan.h"
 
 namespace tk {
 
@@ -79,16 +81,55 @@ __device__ __forceinline__ void warp_partial(double v, double *part, int idx) {
     if ((threadIdx.x & 31) == 0) part[idx] = v;
 }
 
-// warp k (< 4) finishes row block k of the group: combine, update, partial sum
+// Ops of the BiCGStab passes declare kDots = n (1 or 5), finish_dots (the row
+// update and its products), part and pstride: the sums of row block k of group
+// gi go to part[i * pstride + 4 gi + k], as Dot bits.
+template <class Op, class = void>
+struct dot_op {
+    static constexpr int value = 0;
+};
+template <class Op>
+struct dot_op<Op, std::void_t<decltype(Op::kDots)>> {
+    static constexpr int value = Op::kDots;
+};
+// Ops with a device flag that ends an iteration (skip()): later passes return at once.
+template <class Op>
+__device__ __forceinline__ bool op_skip(const Op &op) {
+    if constexpr (dot_op<Op>::value > 0) return op.skip();
+    else return false;
+}
+
+// row block w of the group: combine the W warps' sums, update, partial sums
+template <int W, class Op>
+__device__ __forceinline__ void finish_block(const Op &op, const typename Op::A (*sh)[Op::NA][32], const GroupRows &G,
+                                             const typename Op::Pre &pre, int gi, int w) {
+    const int lane = threadIdx.x & 31;
+    typename Op::A a[Op::NA];
+    Op::template combine_row<W>(sh, lane, w, a);
+    if constexpr (dot_op<Op>::value > 0) {
+        using D = Dot<typename Op::A>;
+        D d[8];
+        if (G.row[w] >= 0) op.finish_dots(G, w, a, pre, d);
+        if constexpr (Op::kDots == 1) {
+            const D v = warp_dot1<typename Op::A>(d[0]);
+            if (lane == 0) op.part[4 * gi + w] = v.bits();
+        } else {
+            const D v = warp_dots8<typename Op::A>(d);
+            if ((lane & 3) == 0 && (lane >> 2) < Op::kDots)
+                op.part[(size_t)(lane >> 2) * op.pstride + 4 * gi + w] = v.bits();
+        }
+    } else {
+        const double v = G.row[w] >= 0 ? op.finish_row(G, w, a, pre) : 0.0;
+        if constexpr (Op::kPart) warp_partial(v, op.part, 4 * gi + w);
+    }
+}
+
+// warp k (< 4) finishes row block k of the group
 template <int W, class Op>
 __device__ __forceinline__ void finish_rows(const Op &op, const typename Op::A (*sh)[Op::NA][32], const GroupRows &G,
                                             const typename Op::Pre &pre, int gi) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w >= 4) return;
-    typename Op::A a[Op::NA];
-    Op::template combine_row<W>(sh, lane, w, a);
-    const double v = G.row[w] >= 0 ? op.finish_row(G, w, a, pre) : 0.0;
-    if constexpr (Op::kPart) warp_partial(v, op.part, 4 * gi + w);
+    const int w = threadIdx.x >> 5;
+    if (w < 4) finish_block<W>(op, sh, G, pre, gi, w);
 }
 
 // epilogue inputs of row block w (< 4) of the group
@@ -214,6 +255,7 @@ __global__ void __launch_bounds__(32 * (W + 1), 1) k_pipe(GridC g, GraphP gp, co
     A(*cb)[W][NA][32] = (A(*)[W][NA][32])(dyn + (size_t)kPipeStages * kPipeStageFloats * sizeof(float));
     __shared__ __align__(8) unsigned long long full[kPipeStages], empty[kPipeStages];
     __shared__ int abort_flag;
+    if (op_skip(op)) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // this block's run of groups (an equal share of the value stream)
     const int g0 = __ldg(gp.run_g[kind] + blockIdx.x), g1 = __ldg(gp.run_g[kind] + blockIdx.x + 1);
@@ -333,6 +375,12 @@ __device__ __forceinline__ void ld_quad(const float *p, float (&v)[4]) {
     asm(TK_STREAM_QUAL ".v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
 #endif
 }
+// the same with an L2 policy (createpolicy)
+__device__ __forceinline__ void ld_quad(const float *p, float (&v)[4], unsigned long long policy) {
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "l"(p), "l"(policy));
+}
 __device__ __forceinline__ void ld_quad(const double *p, double (&v)[4]) {
     const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
     const double2 b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
@@ -393,6 +441,7 @@ __global__ void __launch_bounds__(32 * W) k_plain(GridC g, GraphP gp, const T *_
     if (tA < G.nt) ld_quad(v + (size_t)tA * kGroup, v0);
     if (tB < G.nt) ld_quad(v + (size_t)tB * kGroup, v1);
     pdl_wait();
+    if (op_skip(op)) return;
     const typename Op::Pre pre = load_pre(op, G);
     if (tA < G.nt) {
         const int fp = __ldg(gp.tflat + G.t0 + tA);
@@ -409,6 +458,7 @@ __global__ void __launch_bounds__(32 * W) k_plain(GridC g, GraphP gp, const T *_
     const int tfirst = w + 2 * W;
 #else
     pdl_wait();
+    if (op_skip(op)) return;
     const typename Op::Pre pre = load_pre(op, G);
     const int tfirst = w;
 #endif
@@ -493,6 +543,7 @@ __global__ void __launch_bounds__(32 * W, TK_TILE_WARPS / W) k_tile(GridC g, Gra
     if (tB < G.nt) ld_quad(v + (size_t)tB * kGroup, v1);
     const int ttA = tA < G.nt ? __ldg(gp.ttile + G.t0 + tA) : 0, ttB = tB < G.nt ? __ldg(gp.ttile + G.t0 + tB) : 0;
     pdl_wait();
+    if (op_skip(op)) return;
     const typename Op::Pre pre = load_pre(op, G);
     const int ts = kTileLayers * g.tl;  // floats per vector's tile
     __syncthreads();  // s_lay
@@ -531,6 +582,181 @@ __global__ void __launch_bounds__(32 * W, TK_TILE_WARPS / W) k_tile(GridC g, Gra
     for (int m = 0; m < NA; ++m) sh[w][m][lane] = a[m];
     __syncthreads();
     finish_rows<W>(op, sh, G, pre, gi);
+}
+
+// ---- Rounds: the streamed driver of FP32 passes over scenes too large for
+// the persistent solve.  What bounds such a pass is HBM (the 128 x 128 x 40
+// cloud: 334 MB of values, 49 us at 6.8 TB/s), but a block per group reached
+// 4.7 TB/s (72 us): each block waits for its tile and its first values before
+// it streams, and 5,289 short blocks do that over and over.  Here one block per
+// SM streams its run of groups without a break: 16 warps, two per group, eight
+// groups to a round; a warp's next kRunPf slots are always in flight, across
+// groups and rounds, and the next round's tile (the chunks of the gathered
+// vector that its groups reach) is copied into the other buffer meanwhile.
+// The probe of this access pattern alone reads 7.0 TB/s.
+constexpr int kRunPf = 8;
+constexpr int kRunSmemMax = 224 * 1024;
+constexpr int kRunThreads = 64 * kRunGroups;
+template <class Op>
+inline size_t run_smem(const GridC &g, const GraphP &gp) {
+    const int it = ((g.ntmax + 1) / 2 + 7) / 8 * 8;
+    return (size_t)2 * tile_op<Op>::value * (gp.rd_nc + 1) * gp.rd_tl * sizeof(float) +
+           (size_t)2 * 2 * kRunGroups * it * sizeof(int) + (size_t)2 * kRunGroups * Op::NA * 32 * sizeof(typename Op::A);
+}
+template <class Op>
+__global__ void __launch_bounds__(kRunThreads, 1) k_run(GridC g, GraphP gp, const float *__restrict__ val, Op op,
+                                                        int kind) {
+    using A = typename Op::A;
+    constexpr int NA = Op::NA, NV = tile_op<Op>::value;
+    extern __shared__ __align__(16) unsigned char rdyn[];
+    pdl_trigger();
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, set = w >> 1, wi = w & 1;
+    const int tl = gp.rd_tl, ts = (gp.rd_nc + 1) * tl, it = ((g.ntmax + 1) / 2 + 7) / 8 * 8;
+    float *tile = (float *)rdyn;                  // [2][NV][ts], the last chunk zero
+    int *toff = (int *)(tile + 2 * NV * ts);      // [2][groups][2][it]
+    A(*sh)[NA][32] = (A(*)[NA][32])(toff + 2 * 2 * kRunGroups * it);  // per warp
+    const int r0 = __ldg(gp.rd_first + blockIdx.x), r1 = __ldg(gp.rd_first + blockIdx.x + 1);
+    for (int i = tid; i < 2 * NV * tl; i += kRunThreads) tile[(i / tl + 1) * ts - tl + i % tl] = 0.f;
+    const int nz1 = g.nz + 1;
+    // group of this set in round r: its index in storage order, -1: none
+    auto group = [&](int r) -> int {
+        if (r >= r1) return -1;
+        const int4 R = __ldg(gp.rd_round + r);
+        if (set >= R.y) return -1;
+        const int e = R.x + set, q = e / nz1, zz = e - q * nz1;
+        if (kind == 1 && zz == 0) return -1;
+        return (zz == 0 ? g.nz : zz - 1) * g.gpl + q;
+    };
+    auto values = [&](int gi) -> const float * {
+        if (gi < 0) return nullptr;
+        const int z = gi / g.gpl, nt = __ldg(gp.tstart + z + 1) - __ldg(gp.tstart + z);
+        return val + __ldg(gp.voff + z) + (long long)(gi - z * g.gpl) * nt * kGroup + wi * kGroup + 4 * lane;
+    };
+    auto fetch = [&](int r, int buf) {  // round r's tile and slot offsets
+        const int4 R = __ldg(gp.rd_round + r);
+        for (int c = w; c < R.w; c += 2 * kRunGroups) {
+            const int2 ch = __ldg(gp.rd_chunk + R.z + c);
+#pragma unroll
+            for (int iv = 0; iv < NV; ++iv) {
+                const float *s = op.gsrc(iv) + ch.x;
+                const unsigned d = smem_addr(tile + (buf * NV + iv) * ts + c * tl);
+                if ((g.nxp & 3) == 0) {  // then every chunk starts and ends on 16 bytes
+                    for (int o = 4 * lane; o < ch.y; o += 128)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
+                } else {
+                    for (int o = lane; o < ch.y; o += 32)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int i = tid; i < 2 * R.y * it; i += kRunThreads) {
+            const int l = i / (2 * it), rem = i - l * 2 * it, ww = rem / it, t = ww + 2 * (rem - ww * it);
+            const int e = R.x + l, zz = e % nz1, z = zz == 0 ? g.nz : zz - 1;
+            const int t0 = __ldg(gp.tstart + z), nt = __ldg(gp.tstart + z + 1) - t0;
+            toff[buf * 2 * kRunGroups * it + i] =
+                t < nt ? __ldg(gp.rd_own + r * kRunGroups + l) * tl + __ldg(gp.rd_off + t0 + t)
+                       : ts - tl + g.H * g.nxp + g.H;  // past the last slot: the zeros
+        }
+    };
+    unsigned long long keep, pass_by;
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
+    auto policy = [&](int r) { return r - r0 < gp.rd_near ? keep : pass_by; };
+    float pf[kRunPf][4];
+    int gi = group(r0);
+    const float *p = values(gi);
+    if (p) {
+        const unsigned long long po = policy(r0);
+#pragma unroll
+        for (int i = 0; i < kRunPf; ++i) ld_quad(p + (size_t)i * 2 * kGroup, pf[i], po);
+    }
+    pdl_wait();
+    if (op_skip(op)) return;
+    if (r0 < r1) fetch(r0, 0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int r = r0; r < r1; ++r) {
+        const int buf = (r - r0) & 1;
+        if (r + 1 < r1) fetch(r + 1, buf ^ 1);
+        const int gn = group(r + 1);
+        const float *pn = values(gn);
+        if (gi >= 0) {
+            const GroupRows G = group_rows(g, gp, gi);
+            typename Op::Pre pre[2] = {};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((k & 1) == wi && G.row[k] >= 0) pre[k >> 1] = op.pre(G, k);
+            const int q = gi - G.z * g.gpl, y0 = q * kGroup / g.nx;
+            int rl[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)  // the row's offset in its chunk, less the halo (ps_row_off)
+                rl[k] = G.row[k] >= 0 ? G.rp[k] - G.z * g.lp - (y0 + g.H) * g.nxp - g.H : 0;
+            A a[NA];
+#pragma unroll
+            for (int m = 0; m < NA; ++m) a[m] = A(0);
+            const int *to = toff + ((buf * kRunGroups + set) * 2 + wi) * it;
+            const float *tb = tile + buf * NV * ts;
+            const int n = (G.nt + 1) / 2;  // both warps walk as many (an odd template: one of zeros)
+            for (int i0 = 0; i0 < n; i0 += kRunPf) {
+                const bool more = i0 + kRunPf < n;
+                const float *src = more ? p + (size_t)(i0 + kRunPf) * 2 * kGroup : pn ? pn : p;
+                const unsigned long long po = policy(more ? r : r + 1);
+                int off[kRunPf];
+#pragma unroll
+                for (int i = 0; i < kRunPf; i += 4) {
+                    const int4 t = *reinterpret_cast<const int4 *>(to + i0 + i);
+                    off[i] = t.x;
+                    off[i + 1] = t.y;
+                    off[i + 2] = t.z;
+                    off[i + 3] = t.w;
+                }
+#pragma unroll
+                for (int i = 0; i < kRunPf; ++i) {
+                    const int t = wi + 2 * (i0 + i);
+                    const auto si = op.slot(gp, G.t0 + (t < G.nt ? t : 0));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) op.add_t(a, k, pf[i][k], tb + off[i] + rl[k], ts, si);
+                    ld_quad(src + (size_t)i * 2 * kGroup, pf[i], po);
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < NA; ++m) sh[w][m][lane] = a[m];
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + set) : "memory");
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((k & 1) == wi) finish_block<2>(op, sh + 2 * set, G, pre[k >> 1], gi, k);
+        } else if (pn) {  // nothing in this round, something in the next
+#pragma unroll
+            for (int i = 0; i < kRunPf; ++i) ld_quad(pn + (size_t)i * 2 * kGroup, pf[i], policy(r + 1));
+        }
+        gi = gn;
+        p = pn;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    }
+}
+
+template <class Op>
+static void run_rounds(cudaStream_t st, const GridC &g, const GraphP &gp, const float *val, const Op &op, int kind) {
+    static bool attr[64] = {false};  // per device: the shared-memory limit of this instantiation is raised
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr[dev]) {
+        cudaFuncSetAttribute(k_run<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunSmemMax);
+        attr[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)gp.rd_nb);
+    cfg.blockDim = dim3(kRunThreads);
+    cfg.dynamicSmemBytes = std::max(run_smem<Op>(g, gp), (size_t)116 * 1024);  // one block per SM
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_run<Op>, g, gp, val, op, kind);
 }
 
 // pipelined launch: one block per run (one run per SM, at most one per group)
@@ -598,6 +824,12 @@ template <typename T, class Op>
 static void run_op(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const Op &op, int kind) {
     const int ngroups = (kind == 0 ? g.nz + 1 : g.nz) * g.gpl;
     if (ngroups <= 0) return;
+    if constexpr (sizeof(T) == 4 && tile_op<Op>::value > 0) {
+        if (g.run && run_smem<Op>(g, gp) <= (size_t)kRunSmemMax) {
+            run_rounds(st, g, gp, val, op, kind);
+            return;
+        }
+    }
     if constexpr (sizeof(T) == 4) {
         if (g.stage) {
             if (g.wq == 4)
