@@ -175,6 +175,9 @@ struct tursca_scene {
     double *bi_part = nullptr;
     unsigned char *bi_state = nullptr;
     cudaEvent_t bi_ev[2] = {nullptr, nullptr};
+    cudaEvent_t ps_ev = nullptr;  // the persistent solve's result has been read back
+    int ps_prof = -1;             // its event pair
+    bool zero_s = false;  // s and g^sun are 0 (first-order assemblies)
     bool x_pair = false;  // xh holds x in FP32 (of the forward solve)
     // the serving loop's batcher of solves (null: own launches)
     tk::SolveBatcher *batcher = nullptr;
@@ -616,12 +619,15 @@ tursca_status ensure_fields(tursca_scene *sc) {
 
 tursca_status sync_check(tursca_scene *sc, const char *where) {
     cudaError_t e = cudaGetLastError();
+    // the status word comes back with the same wait
+    int *hst = sc->hred ? (int *)(sc->hred + 255) : nullptr;
+    const bool have = sc->status && hst;
+    if (e == cudaSuccess && have)
+        e = cudaMemcpyAsync(hst, sc->status, sizeof(int), cudaMemcpyDeviceToHost, sc->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(sc->st);
     if (e != cudaSuccess) return cuda_fail(sc, e, where);
-    if (sc->status) {
-        int stv = 0;
-        e = cudaMemcpy(&stv, sc->status, sizeof(int), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(sc, e, where);
+    if (have) {
+        const int stv = *hst;
         if (stv & tk::STATUS_BAD_FIELD)
             return fail(sc, TURSCA_E_INVALID, "field values must be finite and non-negative");
         if (stv & tk::STATUS_TIMEOUT) return fail(sc, TURSCA_E_TIMEOUT, "a bounded device wait gave up");
@@ -637,17 +643,22 @@ struct SolveState {
     double rel = 1.0, rho = 0.0;
 };
 
+// what a status word read back says
+tursca_status status_error(tursca_scene *sc, const int *hst) {
+    // invalid field values flagged by the assembly (the node-form solve
+    // starts without waiting for it, so they are first seen here)
+    if (*hst & tk::STATUS_BAD_FIELD) return fail(sc, TURSCA_E_INVALID, "field values must be finite and non-negative");
+    if (*hst & tk::STATUS_TIMEOUT) return fail(sc, TURSCA_E_TIMEOUT, "a bounded device wait gave up");
+    return TURSCA_OK;
+}
+
 // waits for the stream and reports what the status word holds
 tursca_status read_status(tursca_scene *sc) {
     // the status word rides along: a bounded wait that gave up shows here
     int *hst = (int *)(sc->hred + 255);
     CK(cudaMemcpyAsync(hst, sc->status, sizeof(int), cudaMemcpyDeviceToHost, sc->st), "d2h");
     CK(cudaStreamSynchronize(sc->st), "sync");
-    // invalid field values flagged by the assembly (the node-form solve
-    // starts without waiting for it, so they are first seen here)
-    if (*hst & tk::STATUS_BAD_FIELD) return fail(sc, TURSCA_E_INVALID, "field values must be finite and non-negative");
-    if (*hst & tk::STATUS_TIMEOUT) return fail(sc, TURSCA_E_TIMEOUT, "a bounded device wait gave up");
-    return TURSCA_OK;
+    return status_error(sc, hst);
 }
 
 template <typename T>
@@ -960,15 +971,16 @@ tursca_status upload_persist(tursca_scene *sc, tursca_scene::PsDev &P, const std
     return TURSCA_OK;
 }
 
-// Solve with the persistent kernel.  *done is false when the scene has no
-// plan, the launch is refused or the iteration gave up; the caller's loop
-// then solves from x = 0.
+// Queue a solve with the persistent kernel and the read-back of its result
+// (an event marks it).  *launched is false when the scene has no plan, an
+// option names how the passes run, or the launch is refused.
 template <typename T>
-tursca_status persist_solve(tursca_scene *sc, const SolveIO<T> &io, double rtol, int max_iter,
-                            tursca_solve_info *info, bool *done) {
-    *done = false;
+tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol, int max_iter, bool *launched_out) {
+    *launched_out = false;
     const tk::PsPlan &P = io.ps->plan;
-    if (P.nb <= 0) return TURSCA_OK;
+    sc->x_pair = false;
+    if (P.nb <= 0 || !sc->wq_auto || sc->stage_values || sc->resid_fp64) return TURSCA_OK;
+    if (!sc->ps_ev) CK(cudaEventCreateWithFlags(&sc->ps_ev, cudaEventDisableTiming), "event");
     tk::PsJob J;
     J.g = io.g;
     J.tstart = io.gp.tstart;
@@ -1014,13 +1026,29 @@ tursca_status persist_solve(tursca_scene *sc, const SolveIO<T> &io, double rtol,
         return TURSCA_OK;
     }
     sc->launches++;
-    tk::PsInfo *h = (tk::PsInfo *)sc->hred;
-    CK(cudaMemcpyAsync(h, sc->ps_ctl + 64, sizeof(tk::PsInfo), cudaMemcpyDeviceToHost, sc->st), "d2h");
     prof_end(sc, pi);
-    const tursca_status rs = read_status(sc);
+    sc->ps_prof = pi;
+    CK(cudaMemcpyAsync(sc->hred, sc->ps_ctl + 64, sizeof(tk::PsInfo), cudaMemcpyDeviceToHost, sc->st), "d2h");
+    CK(cudaMemcpyAsync(sc->hred + 254, sc->status, sizeof(int), cudaMemcpyDeviceToHost, sc->st), "d2h");
+    CK(cudaEventRecord(sc->ps_ev, sc->st), "event");
+    sc->x_pair = sizeof(T) == 4 && io.x == sc->x64;
+    *launched_out = true;
+    return TURSCA_OK;
+}
+
+// Wait for the result of persist_launch.  *done is false when the iteration
+// gave up; the caller's loop then solves from x = 0.
+tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *done) {
+    *done = false;
+    CK(cudaEventSynchronize(sc->ps_ev), "sync");
+    const tursca_status rs = status_error(sc, (const int *)(sc->hred + 254));
     if (rs) return rs;
-    if (pi >= 0) sc->ev_n[pi] = h->iters;
-    if (h->state != tk::PS_CONVERGED && h->state != tk::PS_MAX_ITER) return TURSCA_OK;
+    const tk::PsInfo *h = (const tk::PsInfo *)sc->hred;
+    if (sc->ps_prof >= 0) sc->ev_n[sc->ps_prof] = h->iters;
+    if (h->state != tk::PS_CONVERGED && h->state != tk::PS_MAX_ITER) {
+        sc->x_pair = false;
+        return TURSCA_OK;
+    }
     *done = true;
     if (info) {
         info->iters = h->iters;
@@ -1029,7 +1057,6 @@ tursca_status persist_solve(tursca_scene *sc, const SolveIO<T> &io, double rtol,
         info->rho_est = 0.0;
         info->solver = TURSCA_SOLVER_BICGSTAB;
     }
-    sc->x_pair = sizeof(T) == 4 && io.x == sc->x64;
     sc->solved = true;
     if (h->state == tk::PS_MAX_ITER) return fail(sc, TURSCA_E_NOT_CONVERGED, "solver stopped above rtol");
     return TURSCA_OK;
@@ -1071,7 +1098,7 @@ struct L2Window {
 
 template <typename T>
 tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, tursca_solve_info *info,
-                       const SolveIO<T> &io) {
+                       const SolveIO<T> &io, bool passes = false) {
     const L2Window l2w(sc, io.val, (size_t)sc->G.nval * sizeof(T));
     const tk::GridC &g = io.g;
     const tk::GraphP &gp = io.gp;
@@ -1084,10 +1111,10 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     (void)nb;
     const bool fp64 = sc->d.precision == TURSCA_FP64;
     sc->x_pair = false;
-    // the persistent solve: automatic choice, with no option that names how the passes run
-    if (solver == TURSCA_SOLVER_AUTO && sc->wq_auto && !sc->stage_values && !sc->resid_fp64) {
-        bool done = false;
-        const tursca_status e = persist_solve<T>(sc, io, rtol, max_iter, info, &done);
+    if (solver == TURSCA_SOLVER_AUTO && !passes) {
+        bool launched = false, done = false;
+        tursca_status e = persist_launch<T>(sc, io, rtol, max_iter, &launched);
+        if (!e && launched) e = persist_collect(sc, info, &done);
         if (e || done) return e;
     }
     // the automatic choice goes on with BiCGStab where the other solvers take
@@ -1317,7 +1344,7 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
 }
 
 template <typename T>
-tursca_status do_render(tursca_scene *sc, void *radiance, void *reflectance) {
+tursca_status render_launch(tursca_scene *sc) {
     const tk::GridC g = grid_c(sc);
     const tk::GraphP gp = graph_p(sc);
     tk::FieldP<T> f = field_p<T>(sc);
@@ -1345,14 +1372,52 @@ tursca_status do_render(tursca_scene *sc, void *radiance, void *reflectance) {
     tk::launch_pixels<T>(sc->st, g, f, vc, vp, (const T *)sc->emis, sc->x64, (T *)sc->rad, (T *)sc->refl);
     prof_end(sc, pi);
     sc->launches += 2;
-    size_t np = (size_t)sc->geom.npx * sc->geom.npy;
     CK(cudaGetLastError(), "render launch");
+    return TURSCA_OK;
+}
+
+// the images to the caller (queued by render_launch)
+template <typename T>
+tursca_status render_finish(tursca_scene *sc, void *radiance, void *reflectance) {
+    const size_t np = (size_t)sc->geom.npx * sc->geom.npy;
     if (radiance) CK(cudaMemcpyAsync(radiance, sc->rad, np * sizeof(T), cudaMemcpyDefault, sc->st), "copy radiance");
     if (reflectance)
         CK(cudaMemcpyAsync(reflectance, sc->refl, np * sizeof(T), cudaMemcpyDefault, sc->st), "copy reflectance");
     tursca_status rs = sync_check(sc, "render");
     sc->rendered = rs == TURSCA_OK;
     return rs;
+}
+
+template <typename T>
+tursca_status do_render(tursca_scene *sc, void *radiance, void *reflectance) {
+    const tursca_status e = render_launch<T>(sc);
+    return e ? e : render_finish<T>(sc, radiance, reflectance);
+}
+
+// Solve and render in one go: the render is queued behind the persistent
+// solve, whose result is read while the render runs, so the GPU does not idle
+// between the two (about 12 us per scene).  The images reach the caller only
+// after a solve that succeeded.  *done false: nothing was queued.
+template <typename T>
+tursca_status solve_render(tursca_scene *sc, double rtol, int max_iter, tursca_solve_info *info, void *radiance,
+                           void *reflectance, bool *done) {
+    *done = false;
+    const SolveIO<T> io = forward_io<T>(sc);
+    bool launched = false, solved = false;
+    const int ps = prof_begin(sc, P_SOLVE);
+    tursca_status e = persist_launch<T>(sc, io, rtol, max_iter, &launched);
+    prof_end(sc, ps, launched ? 1 : 0);
+    if (e || !launched) return e;
+    *done = true;
+    e = render_launch<T>(sc);
+    if (e) return e;
+    e = persist_collect(sc, info, &solved);
+    if (e) return e;
+    if (!solved) {
+        e = do_solve<T>(sc, TURSCA_SOLVER_AUTO, rtol, max_iter, info, io, true);
+        return e ? e : do_render<T>(sc, radiance, reflectance);
+    }
+    return render_finish<T>(sc, radiance, reflectance);
 }
 
 // ---------------------------------------------------------------------------
@@ -1874,6 +1939,7 @@ tursca_status tursca_scene_destroy(tursca_scene *sc) {
     if (sc->topk_hist_h) cudaFreeHost(sc->topk_hist_h);
     if (sc->bready) cudaEventDestroy(sc->bready);
     if (sc->bdone) cudaEventDestroy(sc->bdone);
+    if (sc->ps_ev) cudaEventDestroy(sc->ps_ev);
     for (cudaEvent_t e : sc->bi_ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : sc->ev) cudaEventDestroy(e);
@@ -2477,16 +2543,26 @@ tursca_status tursca_assemble_flux(tursca_scene *sc, const tursca_geometry *geom
     const tk::GraphP gp = graph_p(sc);
     const tk::ViewC vc = view_c(sc);
     const tk::ViewP vp = view_p(sc);
+    // the quadrature tables follow the view and the asymmetries
+    double key[6 + tk::MAX_SPECIES] = {vc.s0[0], vc.s0[1], vc.s0[2], vc.v[0], vc.v[1], vc.v[2]};
+    for (int sp = 0; sp < tk::MAX_SPECIES; ++sp) key[6 + sp] = sp < g.S ? vc.g[sp] : 0.0;
+    bool tables = !sc->qt_ok;
+    for (int k = 0; k < 6 + tk::MAX_SPECIES; ++k) tables = tables || key[k] != sc->qt_key[k];
+    sc->qt_ok = true;
+    for (int k = 0; k < 6 + tk::MAX_SPECIES; ++k) sc->qt_key[k] = key[k];
     if (sc->single) {
         // first scattering order: the direct beam and the phase tables only
         int pd = prof_begin(sc, P_PRE);
         if (sc->d.precision == TURSCA_FP64)
-            tk::launch_assemble_direct<double>(sc->st, g, field_p<double>(sc), vc, vp, &sc->launches);
+            tk::launch_assemble_direct<double>(sc->st, g, field_p<double>(sc), vc, vp, tables, &sc->launches);
         else
-            tk::launch_assemble_direct<float>(sc->st, g, field_p<float>(sc), vc, vp, &sc->launches);
+            tk::launch_assemble_direct<float>(sc->st, g, field_p<float>(sc), vc, vp, tables, &sc->launches);
         prof_end(sc, pd);
-        CK(cudaMemsetAsync(sc->s, 0, (size_t)sc->G.n_nodes * sc->es, sc->st), "memset s");
-        CK(cudaMemsetAsync(sc->gsun, 0, (size_t)sc->G.n_atm * sc->es, sc->st), "memset gsun");
+        if (!sc->zero_s) {  // s and g^sun stay 0 until another kind of assembly writes them
+            CK(cudaMemsetAsync(sc->s, 0, (size_t)sc->G.n_nodes * sc->es, sc->st), "memset s");
+            CK(cudaMemsetAsync(sc->gsun, 0, (size_t)sc->G.n_atm * sc->es, sc->st), "memset gsun");
+            sc->zero_s = true;
+        }
         CK(cudaGetLastError(), "assemble launch");
         sc->single_asm = sc->assembled = true;
         sc->sel_asm = sc->aniso_asm = false;
@@ -2495,18 +2571,13 @@ tursca_status tursca_assemble_flux(tursca_scene *sc, const tursca_geometry *geom
     }
     int p0 = prof_begin(sc, P_PRE);
     const cudaStream_t streams[4] = {sc->st, sc->aux[0], sc->aux[1], sc->aux[2]};
-    double key[6 + tk::MAX_SPECIES] = {vc.s0[0], vc.s0[1], vc.s0[2], vc.v[0], vc.v[1], vc.v[2]};
-    for (int sp = 0; sp < tk::MAX_SPECIES; ++sp) key[6 + sp] = sp < g.S ? vc.g[sp] : 0.0;
-    bool tables = !sc->qt_ok;
-    for (int k = 0; k < 6 + tk::MAX_SPECIES; ++k) tables = tables || key[k] != sc->qt_key[k];
     if (sc->d.precision == TURSCA_FP64)
         tk::launch_assemble_pre<double>(streams, sc->fork, g, gp, field_p<double>(sc), vc, vp, sc->segtab_d, tables,
                                         &sc->launches);
     else
         tk::launch_assemble_pre<float>(streams, sc->fork, g, gp, field_p<float>(sc), vc, vp, sc->segtab_f, tables,
                                        &sc->launches);
-    sc->qt_ok = true;
-    for (int k = 0; k < 6 + tk::MAX_SPECIES; ++k) sc->qt_key[k] = key[k];
+    sc->zero_s = false;
     prof_end(sc, p0);
     sc->c_eff = sc->c_min;
     sc->n_couplings = sc->n_kept = -1;
@@ -2571,6 +2642,20 @@ tursca_status tursca_assemble_flux(tursca_scene *sc, const tursca_geometry *geom
     return TURSCA_OK;
 }
 
+// first-order assemblies: s = 0, so x = 0 solves the system exactly, with no
+// products with K
+static tursca_status zero_solution(tursca_scene *sc, int solver, tursca_solve_info *info) {
+    const size_t H = (size_t)sc->d.stencil_radius;
+    const size_t np = (size_t)(sc->d.nz + 1) * (sc->d.nx + 2 * H) * (sc->d.ny + 2 * H);
+    CK(cudaMemsetAsync(sc->x64, 0, np * sizeof(double), sc->st), "memset x");
+    sc->x_pair = false;
+    if (solver == TURSCA_SOLVER_AUTO)
+        solver = sc->d.precision == TURSCA_FP64 ? TURSCA_SOLVER_GMRES : TURSCA_SOLVER_CHEBYSHEV;
+    if (info) *info = tursca_solve_info{0, 0, 0.0, 0.0, solver};
+    sc->solved = true;
+    return TURSCA_OK;
+}
+
 tursca_status tursca_solve_with(tursca_scene *sc, int solver, double rtol, int max_iter, tursca_solve_info *info) {
     const NvtxRange nvtx("tursca_solve");
     if (!sc) return fail(nullptr, TURSCA_E_INVALID, "scene is null");
@@ -2587,17 +2672,7 @@ tursca_status tursca_solve_with(tursca_scene *sc, int solver, double rtol, int m
     } else {
         CK(cudaGetLastError(), "assemble");
     }
-    if (sc->single_asm) {
-        // s = 0: x = 0 solves the system exactly, with no products with K
-        const size_t H = (size_t)sc->d.stencil_radius;
-        const size_t np = (size_t)(sc->d.nz + 1) * (sc->d.nx + 2 * H) * (sc->d.ny + 2 * H);
-        CK(cudaMemsetAsync(sc->x64, 0, np * sizeof(double), sc->st), "memset x");
-        if (solver == TURSCA_SOLVER_AUTO)
-            solver = sc->d.precision == TURSCA_FP64 ? TURSCA_SOLVER_GMRES : TURSCA_SOLVER_CHEBYSHEV;
-        if (info) *info = tursca_solve_info{0, 0, 0.0, 0.0, solver};
-        sc->solved = true;
-        return TURSCA_OK;
-    }
+    if (sc->single_asm) return zero_solution(sc, solver, info);
     const int ps = prof_begin(sc, P_SOLVE);
     tursca_status r;
     if (sc->aniso_asm)
@@ -2631,6 +2706,26 @@ tursca_status tursca_run(tursca_scene *sc, const void *mu_abs, const void *mu_sc
     if (e) return e;
     e = tursca_assemble_flux(sc, geom);
     if (e) return e;
+    if (sc->single_asm && solver >= 0 && solver <= 3 && rtol > 0.0 && max_iter >= 1) {
+        // x = 0: nothing to wait for between the stages; the images reach the
+        // caller after the status word has come back
+        e = zero_solution(sc, solver, info);
+        if (!e) e = sc->d.precision == TURSCA_FP64 ? render_launch<double>(sc) : render_launch<float>(sc);
+        if (!e) e = read_status(sc);
+        if (e) {
+            sc->solved = false;
+            return e;
+        }
+        return sc->d.precision == TURSCA_FP64 ? render_finish<double>(sc, radiance, reflectance)
+                                              : render_finish<float>(sc, radiance, reflectance);
+    }
+    if (solver == TURSCA_SOLVER_AUTO && rtol > 0.0 && max_iter >= 1 && !sc->single_asm && !sc->aniso_asm) {
+        bool done = false;
+        e = sc->d.precision == TURSCA_FP64
+                ? solve_render<double>(sc, rtol, max_iter, info, radiance, reflectance, &done)
+                : solve_render<float>(sc, rtol, max_iter, info, radiance, reflectance, &done);
+        if (e || done) return e;
+    }
     e = tursca_solve_with(sc, solver, rtol, max_iter, info);
     if (e) return e;
     return tursca_render_radiance(sc, radiance, reflectance);

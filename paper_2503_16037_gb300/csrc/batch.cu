@@ -4,13 +4,14 @@
 // Protocol.  A scene's solve records `ready` on its stream, hands the job
 // over and blocks until the job is launched.  The thread waits for the
 // previous launch to finish (the jobs that arrive meanwhile form the next
-// one), takes the waiting jobs of the oldest one's kind (warps per group) in
+// one), and up to kBatchGatherUs for a second job, takes the waiting jobs of the oldest one's kind (warps per group) in
 // order while their blocks fit the GPU side by side, makes its stream wait for every job's `ready`, launches them in one
 // cooperative kernel, records every job's `done` and lets their callers go
 // on: each makes its own stream wait for its `done`.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <condition_variable>
 #include <deque>
 #include <mutex>
@@ -53,6 +54,12 @@ void SolveBatcher::loop() {
         lk.unlock();
         bool ok = cudaEventSynchronize(last) == cudaSuccess;
         lk.lock();
+        // a solve alone waits a moment for one that fits beside it
+        cv.wait_for(lk, std::chrono::microseconds(kBatchGatherUs), [&] {
+            for (size_t i = 1; i < q.size(); ++i)
+                if (q[i]->job->wpg == q[0]->job->wpg && q[0]->job->nb + q[i]->job->nb <= nsm) return true;
+            return stop;
+        });
         std::vector<Pending *> take;
         int blocks = 0;
         size_t smem = 0;

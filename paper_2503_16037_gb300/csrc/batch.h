@@ -18,6 +18,8 @@ namespace tk {
 // A solve is batched when its plan leaves room for another one beside it:
 // at most this share of the GPU's blocks.
 constexpr double kBatchShare = 0.75;
+// How long a solve that is alone waits for one that fits beside it.
+constexpr int kBatchGatherUs = 1000;
 
 // Hand one solve to the batcher and block until its batch has been launched:
 // the batch waits for `ready` (recorded on the scene's stream once the job's

@@ -9,12 +9,13 @@
 
 namespace tk {
 
-// Phase tables (for Theta_i(s0 . v)), extinction and scattering ratios of
+// Phase tables (for Theta_i(s0 . v); skipped when `tables` is false: they are
+// current for this view and these asymmetries), extinction and scattering ratios of
 // every voxel, and the direct beam T_sun and e1 of every node, in stream
 // order on st.  Adds the kernels it launched to *launches.
 template <typename T>
 void launch_assemble_direct(cudaStream_t st, const GridC &g, const FieldP<T> &f, const ViewC &vc, const ViewP &vp,
-                            long long *launches);
+                            bool tables, long long *launches);
 
 // emis[i] = e1_i sum_sp w_sp,i hg_sp(s0 . v) for every atmospheric node i.
 template <typename T>

@@ -1188,19 +1188,21 @@ void launch_assemble_rows_p(cudaStream_t st, const GridC &g, const GraphP &gp, c
 // direct beam, all on the scene stream (the edge tables are not needed).
 template <typename T>
 void launch_assemble_direct(cudaStream_t st, const GridC &g, const FieldP<T> &f, const ViewC &vc, const ViewP &vp,
-                            long long *launches) {
+                            bool tables, long long *launches) {
     const int th = 256;
-    k_tables_cells<T><<<dim3(g.nd, g.S), 128, 0, st>>>(g, f, vc, vp);
-    k_tables_norm<T><<<g.S, 128, 0, st>>>(g, f, vc, vp);
+    if (tables) {
+        k_tables_cells<T><<<dim3(g.nd, g.S), 128, 0, st>>>(g, f, vc, vp);
+        k_tables_norm<T><<<g.S, 128, 0, st>>>(g, f, vc, vp);
+    }
     cudaMemsetAsync(f.mus_max_bits, 0, sizeof(unsigned long long), st);
     k_prep<T><<<(g.n_atm + th - 1) / th, th, 0, st>>>(g, f);
     k_sun<T><<<dim3((g.nxy + kRayBlock - 1) / kRayBlock, g.nz + 1), kRayBlock, 0, st>>>(g, f, vc, vp);
-    if (launches) *launches += 4;
+    if (launches) *launches += tables ? 4 : 2;
 }
 
 #define INST(T)                                                                                                   \
     template void launch_assemble_direct<T>(cudaStream_t, const GridC &, const FieldP<T> &, const ViewC &,       \
-                                            const ViewP &, long long *);                                          \
+                                            const ViewP &, bool, long long *);                                    \
     template void launch_assemble_rows_sel<T>(cudaStream_t, const GridC &, const GraphP &, const FieldP<T> &,     \
                                               const ViewC &, const T *, const T *, long long *);                  \
     template void launch_assemble_rows_p<T>(cudaStream_t, const GridC &, const GraphP &, const FieldP<T> &,       \
