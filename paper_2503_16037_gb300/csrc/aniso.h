@@ -65,6 +65,7 @@ namespace tk {
 constexpr int kAniTileM = 128;
 constexpr int kAniRows = 8;
 
+constexpr int kAniSplit = 2;  // blocks per group of the transport, each a share of the arrival directions
 template <typename T>
 struct AniP {
     T *Q;           // [S][nin][nd] HG quadrature by arrival direction (rows sum to 1)
@@ -80,7 +81,7 @@ struct AniP {
                     // ground sources 1), haloed planes
     T *Pc;          // per slot (K's value layout) the deposit fraction times its chain's Cf: P Cf(src, dir)
     T *b;           // [nin][ldx] first-order term rho T Lsun (the series' source)
-    T *xtg;         // [n_ground] sum over the arrival directions of the current X (ground nodes)
+    T *xtg;         // [kAniSplit][n_ground] sums over the arrival directions of the current X (ground nodes)
     T *xtb;         // [n_ground] the same for b (the series' first term)
     const int4 *tslot; // per layer template: its slots in order of arrival direction, {t, src, dir, 0}
                        // (t: template-local index, src and dir as in the slot descriptor)

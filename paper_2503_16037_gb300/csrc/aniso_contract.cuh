@@ -294,7 +294,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_ani_mma(Op op, int R, int N,
     __shared__ __align__(8) unsigned long long full[NS], empty[NS], rfull[NR], rempty[NR], accf[2], acce[2];
     __shared__ unsigned tmem_slot;
     __shared__ int abort_flag;
-    if (ctl && *(volatile const int *)ctl) return;  // the series has converged
+    pdl_trigger();
+    if (ctl && *(volatile const int *)ctl) {  // the series has converged
+        pdl_wait();
+        return;
+    }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nch = ani_chunks(R);
     if (tid == 0) {
@@ -456,6 +460,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_ani_mma(Op op, int R, int N,
     }
     // every MMA completed before the epilogue's last wait; every copy was
     // waited for by the MMA and the copy warps
+    pdl_wait();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, Sh::TCOLS);
 }
@@ -587,7 +592,7 @@ inline void ani_simt_launch(cudaStream_t st, const Op &op, int S, int R, int N, 
 
 template <int S, int NP, class Op>
 inline void ani_mma_launch(cudaStream_t st, const Op &op, int R, int N, const float *Btab, const CUtensorMap &mx,
-                           const CUtensorMap &mz, const int *ctl, int *status) {
+                           const CUtensorMap &mz, const int *ctl, int *status, bool early) {
     using Sh = MmaShape<S, NP>;
     static int grid_max = 0;  // blocks the GPU holds at once (per instantiation)
     if (grid_max == 0) {
@@ -602,8 +607,19 @@ inline void ani_mma_launch(cudaStream_t st, const Op &op, int R, int N, const fl
     }
     const int ntop = op.jtop < op.g.n_atm ? (op.g.n_atm - op.jtop + kAniTileM - 1) / kAniTileM : 0;
     const int ntiles = ntop + (op.g.n_atm + kAniTileM - 1) / kAniTileM;
-    k_ani_mma<S, NP, Op><<<std::min(ntiles, grid_max), kMmaThreads, Sh::SMEM, st>>>(op, R, N, ntop, ntiles, Btab, mx,
-                                                                                   mz, ctl, status);
+    // early: beside the kernel before it, which writes nothing that this one
+    // reads (the block waits for it before it ends)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(ntiles, grid_max));
+    cfg.blockDim = dim3(kMmaThreads);
+    cfg.dynamicSmemBytes = Sh::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, k_ani_mma<S, NP, Op>, op, R, N, ntop, ntiles, Btab, mx, mz, ctl, status);
 }
 
 }  // namespace tk

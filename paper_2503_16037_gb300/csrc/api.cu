@@ -1708,14 +1708,15 @@ tursca_status ensure_aniso(tursca_scene *sc) {
     CK(dalloc(sc->allocs, sc->ani_CfH, (size_t)g.nd * g.npad * es), "alloc aniso");
     CK(dalloc(sc->allocs, sc->ani_Pc, (size_t)sc->G.nval * es), "alloc aniso");
     CK(dalloc(sc->allocs, sc->ani_b, nin * ani_ldx(g) * es), "alloc aniso");
-    CK(dalloc(sc->allocs, sc->ani_xtg, (size_t)std::max(1, g.n_ground) * es), "alloc aniso");
-    CK(dalloc(sc->allocs, sc->ani_xtb, (size_t)std::max(1, g.n_ground) * es), "alloc aniso");
+    const size_t nxt = (size_t)tk::kAniSplit * std::max(1, g.n_ground) * es;
+    CK(dalloc(sc->allocs, sc->ani_xtg, nxt), "alloc aniso");
+    CK(dalloc(sc->allocs, sc->ani_xtb, nxt), "alloc aniso");
     sc->ani_tables = false;
     CK(cudaMemsetAsync(sc->ani_CfH, 0, (size_t)g.nd * g.npad * es, sc->st), "memset aniso");
     CK(dalloc(sc->allocs, sc->ani_X, nin * ani_ldx(g) * es), "alloc aniso");
     CK(dalloc(sc->allocs, sc->ani_Xn, nin * ani_ldx(g) * es), "alloc aniso");
     CK(dalloc(sc->allocs, sc->ani_acc, 3 * sizeof(double)), "alloc aniso");
-    CK(dalloc(sc->allocs, sc->ani_part, 2 * nblk * sizeof(double)), "alloc aniso");
+    CK(dalloc(sc->allocs, sc->ani_part, 2 * tk::kAniSplit * nblk * sizeof(double)), "alloc aniso");
     CK(dalloc(sc->allocs, sc->ani_ctl, 4 * sizeof(int)), "alloc aniso");
     CK(cudaMemsetAsync(sc->ani_ctl, 0, 4 * sizeof(int), sc->st), "memset aniso");
     if (sc->d.precision != TURSCA_FP64) {
@@ -1849,7 +1850,7 @@ tursca_status do_solve_aniso(tursca_scene *sc, int solver, double rtol, int max_
     T *X = (T *)sc->ani_X, *Xn = (T *)sc->ani_Xn;
     // the first term from X = 0 is b, which the assembly formed (with the ground sums)
     CK(cudaMemcpyAsync(X, sc->ani_b, nx * sizeof(T), cudaMemcpyDeviceToDevice, sc->st), "copy b");
-    CK(cudaMemcpyAsync(sc->ani_xtg, sc->ani_xtb, (size_t)std::max(1, g.n_ground) * sizeof(T),
+    CK(cudaMemcpyAsync(sc->ani_xtg, sc->ani_xtb, (size_t)tk::kAniSplit * std::max(1, g.n_ground) * sizeof(T),
                        cudaMemcpyDeviceToDevice, sc->st),
        "copy b");
     const double tol = sizeof(T) == 8 ? rtol : std::max(rtol, 1e-6);

@@ -215,12 +215,15 @@ __global__ void __launch_bounds__(256) k_ani_ground(GridC g, AniP<T> a, const XT
 // last transport left in a.xtg (one thread per ground node and direction)
 template <typename T>
 __global__ void k_ani_ground_x(GridC g, AniP<T> a, T *Lh, const int *ctl) {
+    pdl_trigger();  // the contraction does not read what this kernel writes
     if (ctl && *(volatile const int *)ctl) return;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= g.n_ground * g.ngd) return;
     const int k = idx / g.n_ground, c = idx - k * g.n_ground;
     const int y = c / g.nx, x = c - y * g.nx;
-    store_halo(Lh + (size_t)k * g.npad, g, x, y, g.nz, a.xtg[c] * a.Wg[(size_t)c * g.ngd + k]);
+    T xt = a.xtg[c];
+    for (int i = 1; i < kAniSplit; ++i) xt += a.xtg[(size_t)i * g.n_ground + c];
+    store_halo(Lh + (size_t)k * g.npad, g, x, y, g.nz, xt * a.Wg[(size_t)c * g.ngd + k]);
 }
 
 // The same for the refinement's residual, in double-single: L = Lsun +
@@ -250,10 +253,14 @@ __global__ void __launch_bounds__(256) k_ani_ground_ds(GridC g, AniP<float> a, c
     }
 }
 
-// Transport as a gather: block = one group of 128 receiver rows (the edge
-// kernel's lane quads), warp w sums the arrival directions w, w + kAniW, ...
-// over the template's slots of that direction (tperm / tseg order), so
-// every X(i, w) is written once, in a fixed order.
+// Transport as a gather: kAniSplit blocks per group of 128 receiver rows (the
+// edge kernel's lane quads), a warp sums every kAniSplit kAniW-th arrival
+// direction over the template's slots of that direction (tperm / tseg order),
+// so every X(i, w) is written once, in a fixed order.  What bounds it is the
+// latency of each direction's loads (L2), so the warps in flight: one block of
+// 8 warps per group took 38 us on the 32 x 32 x 24 plume (200 groups), this 28 us.  Its tables are
+// staged while the contraction still drains (6.0 -> 5.45 ms per run with the
+// contraction's start beside the ground's leave).
 //   MODE 0: Xn = [radd] + rho sum P L, and the change against Xold
 //   MODE 1: Xn = rho sum P L - X with L and X double-single pairs (float2),
 //           the sums in double-single, the residual stored rounded to FP32
@@ -273,7 +280,11 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
                                                               int term) {
     __shared__ double red[2][kAniW];
     extern __shared__ int4 tsm[];
-    if (MODE == 0 && *(volatile const int *)a.ctl) return;
+    const int part = gridDim.x * blockIdx.y + blockIdx.x, nparts = gridDim.x * gridDim.y;
+    if (MODE == 0 && *(volatile const int *)a.ctl) {
+        pdl_wait();
+        return;
+    }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nin = g.nd + g.ngd;
     const GroupRows G = group_rows(g, gp, blockIdx.x);
@@ -301,7 +312,8 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
     using D = T;
     D d2 = D(0), n2 = D(0);
     T gsum[4] = {T(0), T(0), T(0), T(0)};  // ground rows: sum over this warp's directions
-    for (int d = w; d < nin; d += kAniW) {
+    pdl_wait();  // what is above does not change within a series
+    for (int d = w + kAniW * blockIdx.y; d < nin; d += kAniW * kAniSplit) {
         const int e0 = seg[d], e1 = seg[d + 1];
         // this direction's other operands first, so that their loads overlap the gathers
         XT xo[4];
@@ -322,8 +334,7 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
             ld_quad(vrow + (size_t)sl.x * kGroup, P);
             const LT *Ld = Lh + (size_t)sl.z * g.npad + sl.y;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (G.row[k] < 0) continue;
+            for (int k = 0; k < 4; ++k) {  // rows past the layer's end read a valid node
                 if constexpr (MODE == 1) {
                     const float2 l = __ldg(Ld + G.rp[k]);
                     ds_fma(acc[k].x, acl[k], l.x, l.y, P[k]);
@@ -366,7 +377,7 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
             T t = T(0);
 #pragma unroll
             for (int i = 0; i < kAniW; ++i) t += xs[i][threadIdx.x];
-            a.xtg[r] = t;
+            a.xtg[(size_t)blockIdx.y * g.n_ground + r] = t;
         }
     }
     double d2d = (double)d2, n2d = (double)n2;
@@ -385,8 +396,8 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
             s0 += red[0][i];
             s1 += red[1][i];
         }
-        a.part[2 * (size_t)blockIdx.x] = s0;
-        a.part[2 * (size_t)blockIdx.x + 1] = s1;
+        a.part[2 * (size_t)part] = s0;
+        a.part[2 * (size_t)part + 1] = s1;
     }
     if (!check) return;
     // the last block to finish sums the partials in a fixed order (so the
@@ -395,12 +406,12 @@ __global__ void __launch_bounds__(32 * kAniW) k_ani_transport(GridC g, GraphP gp
     __shared__ int last;
     __shared__ double s0[32 * kAniW], s1[32 * kAniW];
     __threadfence();
-    if (threadIdx.x == 0) last = atomicAdd(a.ctl + 2, 1) == (int)gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(a.ctl + 2, 1) == nparts - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
     double p0 = 0.0, p1 = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
         p0 += __ldcg(a.part + 2 * (size_t)i);
         p1 += __ldcg(a.part + 2 * (size_t)i + 1);
     }
@@ -563,12 +574,12 @@ bool rows_map(CUtensorMap &m, const float *base, int n_inner, int ld, int rows) 
 // tensor maps of X and zf cannot be made.
 template <class Op>
 cudaError_t mma_leave(cudaStream_t st, const Op &op, int S, int R, int N, const float *B, const int *ctl,
-                      int *status) {
+                      int *status, bool early) {
     CUtensorMap mx, mz;
     if (!rows_map(mx, op.X, op.g.n_atm, op.ldx, R) || !rows_map(mz, op.zf, op.g.n_atm, op.ldz, R))
         return cudaErrorInvalidValue;
     const int np = ani_leave_np(N, S);
-#define TK_L(SS, NN) ani_mma_launch<SS, NN, Op>(st, op, R, N, B, mx, mz, ctl, status)
+#define TK_L(SS, NN) ani_mma_launch<SS, NN, Op>(st, op, R, N, B, mx, mz, ctl, status, early)
     if (S == 1) {
         if (np == 32) TK_L(1, 32); else if (np == 64) TK_L(1, 64); else if (np == 112) TK_L(1, 112); else TK_L(1, 128);
     } else if (S == 2) {
@@ -586,9 +597,31 @@ cudaError_t mma_leave(cudaStream_t st, const Op &op, int S, int R, int N, const 
 // (the top max(uz) layers)
 inline int top_begin(const GridC &g) { return std::max(0, g.nz - g.R) * g.nxy; }
 
-template <typename T>
-size_t transport_smem(const GridC &g, const AniP<T> &a) {
-    return (size_t)a.max_nt * sizeof(int4) + (size_t)(g.nd + g.ngd + 1) * sizeof(int);
+// one transport; early: beside the end of the contraction (it waits for it
+// after its tables are staged)
+template <typename T, int MODE, typename LT, typename XT>
+void transport(cudaStream_t st, const GridC &g, const GraphP &gp, const FieldP<T> &f, const ViewC &vc, const AniP<T> &a,
+               const T *Pv, const LT *Lh, const XT *Xold, T *Xn, const T *radd, const T *bsrc, int check, double tol,
+               int term, bool early) {
+    auto kern = k_ani_transport<T, MODE, LT, XT>;
+    static bool carve[64] = {false};  // per device: the contraction's split of L1 and shared memory
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !carve[dev]) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        carve[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((g.nz + 1) * g.gpl), kAniSplit);
+    cfg.blockDim = dim3(32 * kAniW);
+    cfg.dynamicSmemBytes = (size_t)a.max_nt * sizeof(int4) + (size_t)(g.nd + g.ngd + 1) * sizeof(int);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kern, g, gp, f, vc, a, Pv, Lh, Xold, Xn, radd, bsrc, check, tol, term);
 }
 
 // the leave contraction; with_top adds the top layers' tiles
@@ -664,8 +697,7 @@ void launch_aniso_prep(cudaStream_t st, const GridC &g, const GraphP &gp, const 
     k_ani_pc<T><<<nblk, 128, 0, st>>>(g, gp, f, a);
     AniP<T> ab = a;  // the ground sums of b go to xtb
     ab.xtg = a.xtb;
-    k_ani_transport<T, 0, T, T><<<nblk, 32 * kAniW, transport_smem(g, a), st>>>(g, gp, f, vc, ab, f.val, a.Lh, nullptr,
-                                                                                  a.b, nullptr, nullptr, 0, 0.0, 0);
+    transport<T, 0, T, T>(st, g, gp, f, vc, ab, f.val, a.Lh, nullptr, a.b, nullptr, nullptr, 0, 0.0, 0, false);
     if (launches) *launches += 5;
     if constexpr (sizeof(T) == 4) {
         if (tables && a.mma) {
@@ -686,18 +718,19 @@ cudaError_t launch_aniso_leave(cudaStream_t st, const GridC &g, const GraphP &gp
                                const AniP<T> &a, const T *X, long long *launches) {
     const int nin = g.nd + g.ngd;
     const LeaveOp<T, T, T, true> lop = leave_op<T>(g, gp, a, f.wsp, X, 0, true);
+    // the ground first: the contraction starts beside it
+    const bool ground = g.n_ground > 0;
+    if (ground) k_ani_ground_x<T><<<(g.n_ground * g.ngd + 255) / 256, 256, 0, st>>>(g, a, a.Lh, a.ctl);
     bool done = false;
     if constexpr (sizeof(T) == 4) {
         if (a.mma) {
-            const cudaError_t e = mma_leave(st, lop, g.S, nin, g.nd, a.Bl, a.ctl, f.status);
+            const cudaError_t e = mma_leave(st, lop, g.S, nin, g.nd, a.Bl, a.ctl, f.status, ground);
             if (e != cudaSuccess) return e;
             done = true;
         }
     }
     if (!done) ani_simt_launch<T>(st, lop, g.S, nin, g.nd, a.ctl);
-    if (g.n_ground > 0)
-        k_ani_ground_x<T><<<(g.n_ground * g.ngd + 255) / 256, 256, 0, st>>>(g, a, a.Lh, a.ctl);
-    if (launches) *launches += g.n_ground > 0 ? 2 : 1;
+    if (launches) *launches += ground ? 2 : 1;
     return cudaSuccess;
 }
 
@@ -705,9 +738,8 @@ template <typename T>
 void launch_aniso_move(cudaStream_t st, const GridC &g, const GraphP &gp, const FieldP<T> &f, const ViewC &vc,
                        const AniP<T> &a, const T *X, T *Xn, const T *radd, bool sun, double tol, int term,
                        long long *launches) {
-    const int nblk = (g.nz + 1) * g.gpl;
-    k_ani_transport<T, 0, T, T><<<nblk, 32 * kAniW, transport_smem(g, a), st>>>(g, gp, f, vc, a, a.Pc, a.Lh, X, Xn, radd,
-                                                                                  sun ? a.b : nullptr, 1, tol, term);
+    transport<T, 0, T, T>(st, g, gp, f, vc, a, a.Pc, a.Lh, X, Xn, radd, sun ? a.b : nullptr, 1, tol, term,
+                          sizeof(T) == 4 && a.mma);
     if (launches) *launches += 1;
 }
 
@@ -845,9 +877,7 @@ void launch_aniso_resid(cudaStream_t st, const GridC &g, const GraphP &gp, const
     k_ani_ds<<<ntop + (g.n_atm + kDsM - 1) / kDsM, kDsThreads, 0, st>>>(g, a, gp.dirs, jtop, a.Ads, a.ldz, a.Atop,
                                                                         ldt, ntop, a.Bds, Kp, g.nd, L);
     if (g.n_ground > 0) k_ani_ground_ds<<<(g.n_ground + 31) / 32, 256, 0, st>>>(g, a, X, L);
-    const int nblk = (g.nz + 1) * g.gpl;
-    k_ani_transport<float, 1, float2, float2><<<nblk, 32 * kAniW, transport_smem(g, a), st>>>(
-        g, gp, f, vc, a, f.val, L, X, r, nullptr, nullptr, 2, 0.0, 0);
+    transport<float, 1, float2, float2>(st, g, gp, f, vc, a, f.val, L, X, r, nullptr, nullptr, 2, 0.0, 0, false);
     if (launches) *launches += g.n_ground > 0 ? 6 : 5;
 }
 
@@ -885,7 +915,7 @@ cudaError_t launch_aniso_contract_test(cudaStream_t st, const GridC &g, const Gr
         RawOp<LeaveOp<float, float, float, true>> op;
         static_cast<LeaveOp<float, float, float, true> &>(op) = leave_op<float>(g, gp, a, f.wsp, X, 0, false);
         op.raw = out;
-        if (mma) return mma_leave(st, op, g.S, nin, g.nd, a.Bl, nullptr, f.status);
+        if (mma) return mma_leave(st, op, g.S, nin, g.nd, a.Bl, nullptr, f.status, false);
         ani_simt_launch<float>(st, op, g.S, nin, g.nd, nullptr);
     } else {
         RawOp<SqcOp<float>> op;
