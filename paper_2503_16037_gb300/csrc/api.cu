@@ -164,7 +164,7 @@ struct tursca_scene {
         int *rd_first = nullptr, *rd_own = nullptr, *rd_off = nullptr;
         int4 *rd_round = nullptr;
         int2 *rd_chunk = nullptr;
-        int rd_nb = 0, rd_tl = 0, rd_nc = 0, rd_near = 0;
+        int rd_nb = 0, rd_tl = 0, rd_nc = 0, rd_near = 0, rd_max = 0;
     };
     PsDev ps, psT;
     double *ps_part = nullptr;
@@ -390,6 +390,7 @@ void set_rounds(tk::GraphP &p, const tursca_scene::PsDev &d) {
     p.rd_tl = d.rd_tl;
     p.rd_nc = d.rd_nc;
     p.rd_near = d.rd_near;
+    p.rd_max = d.rd_max;
 }
 
 tk::GraphP graph_p(const tursca_scene *sc) {
@@ -840,9 +841,8 @@ tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &g
         if (c < chunks) {
             const int pi = prof_begin(sc, P_GPROD);
             for (int k = 0; k < kBiChunk; ++k)
-                tk::launch_bi_step<T>(sc->st, g, gp, val, b, r, p, v, t, d, sc->bi_part, st);
+                tk::launch_bi_step<T>(sc->st, g, gp, val, b, r, p, v, t, d, sc->bi_part, st, &sc->launches);
             prof_end(sc, pi, 2 * kBiChunk);
-            sc->launches += 6 * kBiChunk;
             CK(cudaMemcpyAsync(slot(c), st, sizeof(*st), cudaMemcpyDeviceToHost, sc->st), "d2h");
             CK(cudaEventRecord(sc->bi_ev[c & 1], sc->st), "event");
         }
@@ -965,6 +965,7 @@ tursca_status upload_persist(tursca_scene *sc, tursca_scene::PsDev &P, const std
             P.rd_tl = rp.tl;
             P.rd_nc = rp.nc;
             P.rd_near = rp.near;
+            P.rd_max = rp.rmax;
         }
     }
     P.plan = std::move(plan);

@@ -140,7 +140,7 @@ struct GraphP {
     const int2 *rd_chunk;
     const int *rd_own;
     const int *rd_off;
-    int rd_nb, rd_tl, rd_nc, rd_near;
+    int rd_nb, rd_tl, rd_nc, rd_near, rd_max;
     const int4 *cseg;
     const int *ctap;
     int nctap;                     // total taps of the canonical directions
@@ -410,7 +410,7 @@ void launch_bi_start(cudaStream_t st, int n, const double *r64, double down, dou
 // one step (two products); part: bi_part_words(g) doubles
 template <typename T>
 void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const T *r0, T *r, T *p, T *v,
-                    T *t, T *d, double *part, BiState<T> *state);
+                    T *t, T *d, double *part, BiState<T> *state, long long *launches);
 // x += up d, with the FP32 pair of x when xh is set
 template <typename T>
 void launch_bi_end(cudaStream_t st, int n, const T *d, double up, double *x, float *xh, float *xl);

@@ -694,13 +694,14 @@ __global__ void __launch_bounds__(512) k_bi_sums(const double *__restrict__ part
         if (threadIdx.x == 0) out[blockIdx.y * kBiParts + blockIdx.x] = t.bits();
     }
 }
-// the nd sums, by warps 0 .. nd - 1, into sh (synchronises)
+// nd sums of n values, value i of sum w at sums[w * stride + i], by warps
+// 0 .. nd - 1, into sh (synchronises)
 template <typename T>
-__device__ __forceinline__ void bi_total(const double *sums, int nd, double *sh) {
+__device__ __forceinline__ void bi_total(const double *sums, size_t stride, int n, int nd, double *sh) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w < nd) {
         Dot<T> v;
-        if (lane < kBiParts) v = Dot<T>::from(__ldcg(sums + w * kBiParts + lane));
+        for (int i = lane; i < n; i += 32) v.join(Dot<T>::from(__ldcg(sums + w * stride + i)));
         v = warp_dot1<T>(v);
         if (lane == 0) sh[w] = v.bits();
     }
@@ -726,15 +727,15 @@ __global__ void k_bi_start(int n, const double *__restrict__ r64, T down, T bb, 
 }
 // alpha = rho / r0.v; d += alpha p; r <- s = r - alpha v
 template <typename T>
-__global__ void __launch_bounds__(256) k_bi_s(int n, const double *__restrict__ sums, const T *__restrict__ p,
-                                              const T *__restrict__ v, T *__restrict__ r, T *__restrict__ d,
-                                              BiState<T> *st) {
+__global__ void __launch_bounds__(256) k_bi_s(int n, const double *__restrict__ sums, size_t stride, int ns,
+                                              const T *__restrict__ p, const T *__restrict__ v, T *__restrict__ r,
+                                              T *__restrict__ d, BiState<T> *st) {
     __shared__ double sh[8];
     __shared__ T sa;
     pdl_trigger();
     pdl_wait();
     if (st->done) return;
-    bi_total<T>(sums, 1, sh);
+    bi_total<T>(sums, stride, ns, 1, sh);
     if (threadIdx.x == 0) {
         const T r0v = Dot<T>::from(sh[0]).value();
         sa = r0v != T(0) ? st->rho / r0v : T(0);
@@ -751,7 +752,8 @@ __global__ void __launch_bounds__(256) k_bi_s(int n, const double *__restrict__ 
 // p = r + beta (p - omega v).  The last block to finish writes the state,
 // which the others read.
 template <typename T>
-__global__ void __launch_bounds__(256) k_bi_p(int n, const double *__restrict__ sums, const T *__restrict__ v,
+__global__ void __launch_bounds__(256) k_bi_p(int n, const double *__restrict__ sums, size_t stride, int ns,
+                                              const T *__restrict__ v,
                                               const T *__restrict__ t, T *__restrict__ r, T *__restrict__ p,
                                               T *__restrict__ d, BiState<T> *st) {
     __shared__ double sh[8];
@@ -759,7 +761,7 @@ __global__ void __launch_bounds__(256) k_bi_p(int n, const double *__restrict__ 
     pdl_trigger();
     pdl_wait();
     if (st->done) return;
-    bi_total<T>(sums, 5, sh);
+    bi_total<T>(sums, stride, ns, 5, sh);
     if (threadIdx.x == 0) {
         const Dot<T> ts = Dot<T>::from(sh[0]), tt = Dot<T>::from(sh[1]), r0t = Dot<T>::from(sh[3]);
         Dot<T> r0r = Dot<T>::from(sh[2]), rn = Dot<T>::from(sh[4]);
@@ -825,7 +827,7 @@ void launch_bi_start(cudaStream_t st, int n, const double *r64, double down, dou
 }
 template <typename T>
 void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *val, const T *r0, T *r, T *p, T *v,
-                    T *t, T *d, double *part, BiState<T> *state) {
+                    T *t, T *d, double *part, BiState<T> *state, long long *launches) {
     const int n = (int)g.npad, np = sweep_blocks(g);
     double *sums = part + (size_t)5 * np;
     // four blocks of 256 threads on each of 152 SMs, so that the next pass's
@@ -847,13 +849,21 @@ void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *
     const T *cp = p, *cv = v, *ct = t;
     const BiState<T> *cst = state;
     OpBi<T, 1> ov{p, r0, v, part, (size_t)np, state};
-    run_op(st, g, gp, val, ov, 0);
-    go(k_bi_sums<T>, dim3(kBiParts, 1), 512, cpart, (size_t)np, np, sums, cst);
-    go(k_bi_s<T>, dim3(nb), 256, n, csums, cp, cv, r, d, state);
     OpBi<T, 5> ot{r, r0, t, part, (size_t)np, state};
+    // passes in rounds leave a value per block, which the vector kernels sum
+    // themselves (two launches less per step: 10 us of 152 on the cloud)
+    bool rounds = false;
+    if constexpr (sizeof(T) == 4) rounds = run_in_rounds<OpBi<T, 1>>(g, gp) && run_in_rounds<OpBi<T, 5>>(g, gp);
+    const size_t stride = rounds ? (size_t)np : kBiParts;
+    const int ns = rounds ? gp.rd_nb : kBiParts;
+    if (rounds) csums = part;
+    run_op(st, g, gp, val, ov, 0);
+    if (!rounds) go(k_bi_sums<T>, dim3(kBiParts, 1), 512, cpart, (size_t)np, np, sums, cst);
+    go(k_bi_s<T>, dim3(nb), 256, n, csums, stride, ns, cp, cv, r, d, state);
     run_op(st, g, gp, val, ot, 0);
-    go(k_bi_sums<T>, dim3(kBiParts, 5), 512, cpart, (size_t)np, np, sums, cst);
-    go(k_bi_p<T>, dim3(nb), 256, n, csums, cv, ct, r, p, d, state);
+    if (!rounds) go(k_bi_sums<T>, dim3(kBiParts, 5), 512, cpart, (size_t)np, np, sums, cst);
+    go(k_bi_p<T>, dim3(nb), 256, n, csums, stride, ns, cv, ct, r, p, d, state);
+    *launches += rounds ? 4 : 6;
 }
 template <typename T>
 void launch_bi_end(cudaStream_t st, int n, const T *d, double up, double *x, float *xh, float *xl) {
@@ -1017,7 +1027,7 @@ void launch_axpby(cudaStream_t st, int n, double a, const T *x, double b, const 
     template void launch_bi_start<T>(cudaStream_t, int, const double *, double, double, double, T *, T *, T *, T *, \
                                      BiState<T> *);                                                                \
     template void launch_bi_step<T>(cudaStream_t, const GridC &, const GraphP &, const T *, const T *, T *, T *,   \
-                                    T *, T *, T *, double *, BiState<T> *);                                        \
+                                    T *, T *, T *, double *, BiState<T> *, long long *);                           \
     template void launch_bi_end<T>(cudaStream_t, int, const T *, double, double *, float *, float *);
 BINST(float)
 BINST(double)

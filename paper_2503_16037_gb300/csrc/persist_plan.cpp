@@ -127,7 +127,9 @@ RunPlan run_plan(const PsGeom &g, const std::vector<int> &nt, int nsm, size_t ti
             e += n;
         }
         P.first.push_back((int)P.round.size() / 4);
+        P.rmax = std::max(P.rmax, P.first[b + 1] - P.first[b]);
     }
+    if (P.rmax > kRunMaxRounds || g.nz > kRunMaxNz) return RunPlan();
     double values = 0.0;
     for (int z = 0; z <= g.nz; ++z) values += (double)nt[z] * g.gpl * kPsRows * sizeof(float);
     P.near = (int)(P.round.size() / 4 * std::min(1.0, kPsL2Bytes / values)) / nsm;

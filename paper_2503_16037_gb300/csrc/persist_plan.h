@@ -180,10 +180,12 @@ PsPlan ps_plan(const PsGeom &g, const std::vector<int> &nt, int es, int nsm, siz
 // kRunGroups consecutive ones (strip order) whose chunks fit a tile of nc.
 constexpr int kRunGroups = 8;     // groups of a round, two warps each
 constexpr int kRunMaxChunk = 20;  // chunks of a round's tile
+constexpr int kRunMaxRounds = 128, kRunMaxNz = 510;  // tables in shared memory (at most 24 KB)
 struct RunPlan {
     int nb = 0;              // blocks (0: the passes run a block per group)
     int tl = 0, nc = 0;      // elements per chunk, chunks per tile
     int near = 0;            // rounds of each block whose values L2 can hold
+    int rmax = 0;            // most rounds of a block
     std::vector<int> first;  // [nb + 1] first round of each block
     std::vector<int> round;  // per round: first group, groups, first chunk, chunks
     std::vector<int> chunk;  // per chunk: haloed index of its first element, elements

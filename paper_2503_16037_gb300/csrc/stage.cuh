@@ -26,14 +26,13 @@ struct GroupRows {
     int ay[4];     // offset of the row's halo copy in y (0: none)
 };
 
-__device__ __forceinline__ GroupRows group_rows(const GridC &g, const GraphP &gp, int gi) {
+// rows of group q of layer z (no loads; t0, nt and vb stay unset)
+__device__ __forceinline__ GroupRows group_rows_at(const GridC &g, int z, int q) {
     GroupRows G;
     const int lane = threadIdx.x & 31;
-    G.z = gi / g.gpl;
-    const int q = gi - G.z * g.gpl;
-    G.t0 = __ldg(gp.tstart + G.z);
-    G.nt = __ldg(gp.tstart + G.z + 1) - G.t0;
-    G.vb = __ldg(gp.voff + G.z) + (long long)q * G.nt * kGroup;
+    G.z = z;
+    G.t0 = G.nt = 0;
+    G.vb = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int r = q * kGroup + lane + 32 * k;
@@ -45,6 +44,14 @@ __device__ __forceinline__ GroupRows group_rows(const GridC &g, const GraphP &gp
         G.ax[k] = x < g.H ? g.nx : (x >= g.nx - g.H ? -g.nx : 0);
         G.ay[k] = y < g.H ? g.ny * g.nxp : (y >= g.ny - g.H ? -g.ny * g.nxp : 0);
     }
+    return G;
+}
+__device__ __forceinline__ GroupRows group_rows(const GridC &g, const GraphP &gp, int gi) {
+    const int z = gi / g.gpl, q = gi - z * g.gpl;
+    GroupRows G = group_rows_at(g, z, q);
+    G.t0 = __ldg(gp.tstart + z);
+    G.nt = __ldg(gp.tstart + z + 1) - G.t0;
+    G.vb = __ldg(gp.voff + z) + (long long)q * G.nt * kGroup;
     return G;
 }
 
@@ -100,9 +107,11 @@ __device__ __forceinline__ bool op_skip(const Op &op) {
 }
 
 // row block w of the group: combine the W warps' sums, update, partial sums
+// (of a dot op: into *acc when it is set, sum i in lane 4 i)
 template <int W, class Op>
 __device__ __forceinline__ void finish_block(const Op &op, const typename Op::A (*sh)[Op::NA][32], const GroupRows &G,
-                                             const typename Op::Pre &pre, int gi, int w) {
+                                             const typename Op::Pre &pre, int gi, int w,
+                                             Dot<typename Op::A> *acc = nullptr) {
     const int lane = threadIdx.x & 31;
     typename Op::A a[Op::NA];
     Op::template combine_row<W>(sh, lane, w, a);
@@ -110,14 +119,11 @@ __device__ __forceinline__ void finish_block(const Op &op, const typename Op::A 
         using D = Dot<typename Op::A>;
         D d[8];
         if (G.row[w] >= 0) op.finish_dots(G, w, a, pre, d);
-        if constexpr (Op::kDots == 1) {
-            const D v = warp_dot1<typename Op::A>(d[0]);
-            if (lane == 0) op.part[4 * gi + w] = v.bits();
-        } else {
-            const D v = warp_dots8<typename Op::A>(d);
-            if ((lane & 3) == 0 && (lane >> 2) < Op::kDots)
-                op.part[(size_t)(lane >> 2) * op.pstride + 4 * gi + w] = v.bits();
-        }
+        D v;
+        if constexpr (Op::kDots == 1) v = warp_dot1<typename Op::A>(d[0]);
+        else v = warp_dots8<typename Op::A>(d);
+        if (acc) acc->join(v);
+        else if ((lane & 3) == 0 && (lane >> 2) < Op::kDots) op.part[(size_t)(lane >> 2) * op.pstride + 4 * gi + w] = v.bits();
     } else {
         const double v = G.row[w] >= 0 ? op.finish_row(G, w, a, pre) : 0.0;
         if constexpr (Op::kPart) warp_partial(v, op.part, 4 * gi + w);
@@ -375,7 +381,14 @@ __device__ __forceinline__ void ld_quad(const float *p, float (&v)[4]) {
     asm(TK_STREAM_QUAL ".v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
 #endif
 }
-// the same with an L2 policy (createpolicy)
+template <bool PASS_BY>
+__device__ __forceinline__ unsigned long long l2_policy() {
+    unsigned long long p;
+    if (PASS_BY) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+// the same with an L2 policy
 __device__ __forceinline__ void ld_quad(const float *p, float (&v)[4], unsigned long long policy) {
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
@@ -589,19 +602,35 @@ __global__ void __launch_bounds__(32 * W, TK_TILE_WARPS / W) k_tile(GridC g, Gra
 // cloud: 334 MB of values, 49 us at 6.8 TB/s), but a block per group reached
 // 4.7 TB/s (72 us): each block waits for its tile and its first values before
 // it streams, and 5,289 short blocks do that over and over.  Here one block per
-// SM streams its run of groups without a break: 16 warps, two per group, eight
-// groups to a round; a warp's next kRunPf slots are always in flight, across
-// groups and rounds, and the next round's tile (the chunks of the gathered
-// vector that its groups reach) is copied into the other buffer meanwhile.
-// The probe of this access pattern alone reads 7.0 TB/s.
+// SM streams its run of groups: 16 warps, two per group, eight groups to a
+// round; a warp's next kRunPf slots are always in flight, across groups and
+// rounds, and the next round's tile (the chunks of the gathered vector that its
+// groups reach) is copied into the other buffer meanwhile.  Nothing between two
+// rounds waits for global memory: the tables of the block's rounds and of the
+// layers sit in shared memory, a chunk's address is loaded a round ahead, slot
+// offsets come with the values (with these chains and the rows' divisions
+// between rounds 70 us, now 64; the access pattern alone takes 46 us).  The first
+// rounds of each block are read with the normal policy up to what L2 holds, the
+// others evict-first: 7 % of a solve.
 constexpr int kRunPf = 8;
+constexpr int kRunW = 2;  // warps per group
+constexpr int kRunNb = 4 / kRunW;  // row blocks a warp finishes: wi, wi + kRunW
 constexpr int kRunSmemMax = 224 * 1024;
-constexpr int kRunThreads = 64 * kRunGroups;
+constexpr int kRunThreads = 32 * kRunW * kRunGroups;
+static_assert(kRunMaxChunk <= 2 * kRunW * kRunGroups, "a warp copies two chunks of a tile");
+struct RunSmem {  // byte offsets: tiles [2][NV][ts], per-warp sums, layer table, rounds, their groups
+    size_t sh, voff, round, grp, tst, end;
+};
 template <class Op>
-inline size_t run_smem(const GridC &g, const GraphP &gp) {
-    const int it = ((g.ntmax + 1) / 2 + 7) / 8 * 8;
-    return (size_t)2 * tile_op<Op>::value * (gp.rd_nc + 1) * gp.rd_tl * sizeof(float) +
-           (size_t)2 * 2 * kRunGroups * it * sizeof(int) + (size_t)2 * kRunGroups * Op::NA * 32 * sizeof(typename Op::A);
+__host__ __device__ inline RunSmem run_layout(const GridC &g, int nc, int tl, int rmax) {
+    RunSmem L;
+    L.sh = ((size_t)2 * tile_op<Op>::value * (nc + 1) * tl * sizeof(float) + 15) / 16 * 16;
+    L.voff = L.sh + (size_t)kRunW * kRunGroups * Op::NA * 32 * sizeof(typename Op::A);
+    L.round = (L.voff + (size_t)(g.nz + 2) * sizeof(long long) + 15) / 16 * 16;
+    L.grp = L.round + (size_t)rmax * sizeof(int4);
+    L.tst = L.grp + (size_t)rmax * kRunGroups * sizeof(int4);
+    L.end = L.tst + (size_t)(g.nz + 2) * sizeof(int);
+    return L;
 }
 template <class Op>
 __global__ void __launch_bounds__(kRunThreads, 1) k_run(GridC g, GraphP gp, const float *__restrict__ val, Op op,
@@ -610,131 +639,185 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_run(GridC g, GraphP gp, cons
     constexpr int NA = Op::NA, NV = tile_op<Op>::value;
     extern __shared__ __align__(16) unsigned char rdyn[];
     pdl_trigger();
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, set = w >> 1, wi = w & 1;
-    const int tl = gp.rd_tl, ts = (gp.rd_nc + 1) * tl, it = ((g.ntmax + 1) / 2 + 7) / 8 * 8;
-    float *tile = (float *)rdyn;                  // [2][NV][ts], the last chunk zero
-    int *toff = (int *)(tile + 2 * NV * ts);      // [2][groups][2][it]
-    A(*sh)[NA][32] = (A(*)[NA][32])(toff + 2 * 2 * kRunGroups * it);  // per warp
-    const int r0 = __ldg(gp.rd_first + blockIdx.x), r1 = __ldg(gp.rd_first + blockIdx.x + 1);
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, set = w / kRunW, wi = w % kRunW;
+    const int tl = gp.rd_tl, ts = (gp.rd_nc + 1) * tl;
+    const RunSmem L = run_layout<Op>(g, gp.rd_nc, tl, gp.rd_max);
+    float *tile = (float *)rdyn;  // the last chunk of each is zero
+    A(*sh)[NA][32] = (A(*)[NA][32])(rdyn + L.sh);
+    long long *s_voff = (long long *)(rdyn + L.voff);
+    int4 *s_round = (int4 *)(rdyn + L.round);
+    int4 *s_grp = (int4 *)(rdyn + L.grp);  // (layer or -1, strip, first tile element of its own chunk, -)
+    int *s_tst = (int *)(rdyn + L.tst);
+    const int r0 = __ldg(gp.rd_first + blockIdx.x), nr = __ldg(gp.rd_first + blockIdx.x + 1) - r0;
     for (int i = tid; i < 2 * NV * tl; i += kRunThreads) tile[(i / tl + 1) * ts - tl + i % tl] = 0.f;
+    for (int i = tid; i < nr; i += kRunThreads) s_round[i] = __ldg(gp.rd_round + r0 + i);
     const int nz1 = g.nz + 1;
-    // group of this set in round r: its index in storage order, -1: none
-    auto group = [&](int r) -> int {
-        if (r >= r1) return -1;
-        const int4 R = __ldg(gp.rd_round + r);
-        if (set >= R.y) return -1;
-        const int e = R.x + set, q = e / nz1, zz = e - q * nz1;
-        if (kind == 1 && zz == 0) return -1;
-        return (zz == 0 ? g.nz : zz - 1) * g.gpl + q;
+    for (int i = tid; i < nr * kRunGroups; i += kRunThreads) {
+        const int4 R = __ldg(gp.rd_round + r0 + i / kRunGroups);
+        const int l = i % kRunGroups, e = R.x + l, zz = e % nz1;
+        const bool on = l < R.y && !(kind == 1 && zz == 0);
+        s_grp[i] = make_int4(on ? (zz == 0 ? g.nz : zz - 1) : -1, e / nz1,
+                             __ldg(gp.rd_own + (size_t)r0 * kRunGroups + i) * tl, 0);
+    }
+    for (int i = tid; i < g.nz + 2; i += kRunThreads) {
+        s_tst[i] = __ldg(gp.tstart + i);
+        s_voff[i] = i <= g.nz ? __ldg(gp.voff + i) : 0;
+    }
+    __syncthreads();
+    auto policy = [&](int r) { return r < gp.rd_near ? l2_policy<false>() : l2_policy<true>(); };
+    // this set's group in round r (no slots: none)
+    struct Grp {
+        int t0, nt;
+        const float *p;
     };
-    auto values = [&](int gi) -> const float * {
-        if (gi < 0) return nullptr;
-        const int z = gi / g.gpl, nt = __ldg(gp.tstart + z + 1) - __ldg(gp.tstart + z);
-        return val + __ldg(gp.voff + z) + (long long)(gi - z * g.gpl) * nt * kGroup + wi * kGroup + 4 * lane;
+    auto group = [&](int r) {
+        Grp G{0, 0, val};
+        if (r >= nr) return G;
+        const int4 e = s_grp[r * kRunGroups + set];
+        if (e.x < 0) return G;
+        G.t0 = s_tst[e.x];
+        G.nt = s_tst[e.x + 1] - G.t0;
+        G.p = val + s_voff[e.x] + (long long)e.y * G.nt * kGroup + wi * kGroup + 4 * lane;
+        return G;
     };
-    auto fetch = [&](int r, int buf) {  // round r's tile and slot offsets
-        const int4 R = __ldg(gp.rd_round + r);
-        for (int c = w; c < R.w; c += 2 * kRunGroups) {
-            const int2 ch = __ldg(gp.rd_chunk + R.z + c);
+    // slots 4 s .. of the group, this warp's share, into registers
+    float pf[kRunPf][4];
+    int po[kRunPf];
+    auto load = [&](const Grp &G, unsigned long long policy, int i, int n) {
+        ld_quad(G.p + (size_t)n * kRunW * kGroup, pf[i], policy);
+        po[i] = __ldg(gp.rd_off + G.t0 + min(wi + kRunW * n, G.nt - 1));
+    };
+    auto chunk = [&](int r, int h) {  // a chunk of round r's tile that this warp copies (y = 0: none)
+        if (r >= nr) return make_int2(0, 0);
+        const int4 R = s_round[r];
+        const int c = w + h * kRunW * kRunGroups;
+        return c < R.w ? __ldg(gp.rd_chunk + R.z + c) : make_int2(0, 0);
+    };
+    auto fetch = [&](const int2 ch, int h, int buf) {
 #pragma unroll
-            for (int iv = 0; iv < NV; ++iv) {
-                const float *s = op.gsrc(iv) + ch.x;
-                const unsigned d = smem_addr(tile + (buf * NV + iv) * ts + c * tl);
-                if ((g.nxp & 3) == 0) {  // then every chunk starts and ends on 16 bytes
-                    for (int o = 4 * lane; o < ch.y; o += 128)
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
-                } else {
-                    for (int o = lane; o < ch.y; o += 32)
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
-                }
+        for (int iv = 0; iv < NV; ++iv) {
+            const float *s = op.gsrc(iv) + ch.x;
+            const unsigned d = smem_addr(tile + (buf * NV + iv) * ts + (w + h * kRunW * kRunGroups) * tl);
+            if ((g.nxp & 3) == 0) {  // then every chunk starts and ends on 16 bytes
+                for (int o = 4 * lane; o < ch.y; o += 128)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
+            } else {
+                for (int o = lane; o < ch.y; o += 32)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * o), "l"(s + o) : "memory");
             }
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        for (int i = tid; i < 2 * R.y * it; i += kRunThreads) {
-            const int l = i / (2 * it), rem = i - l * 2 * it, ww = rem / it, t = ww + 2 * (rem - ww * it);
-            const int e = R.x + l, zz = e % nz1, z = zz == 0 ? g.nz : zz - 1;
-            const int t0 = __ldg(gp.tstart + z), nt = __ldg(gp.tstart + z + 1) - t0;
-            toff[buf * 2 * kRunGroups * it + i] =
-                t < nt ? __ldg(gp.rd_own + r * kRunGroups + l) * tl + __ldg(gp.rd_off + t0 + t)
-                       : ts - tl + g.H * g.nxp + g.H;  // past the last slot: the zeros
-        }
     };
-    unsigned long long keep, pass_by;
-    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep));
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
-    auto policy = [&](int r) { return r - r0 < gp.rd_near ? keep : pass_by; };
-    float pf[kRunPf][4];
-    int gi = group(r0);
-    const float *p = values(gi);
-    if (p) {
-        const unsigned long long po = policy(r0);
+    Grp cur = group(0);
+    if (cur.nt > 0) {
 #pragma unroll
-        for (int i = 0; i < kRunPf; ++i) ld_quad(p + (size_t)i * 2 * kGroup, pf[i], po);
+        for (int i = 0; i < kRunPf; ++i) load(cur, policy(0), i, i);
     }
+    int2 ch[2] = {chunk(0, 0), chunk(0, 1)};
     pdl_wait();
     if (op_skip(op)) return;
-    if (r0 < r1) fetch(r0, 0);
+    for (int h = 0; h < 2; ++h) fetch(ch[h], h, 0), ch[h] = chunk(1, h);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (int r = r0; r < r1; ++r) {
-        const int buf = (r - r0) & 1;
-        if (r + 1 < r1) fetch(r + 1, buf ^ 1);
-        const int gn = group(r + 1);
-        const float *pn = values(gn);
-        if (gi >= 0) {
-            const GroupRows G = group_rows(g, gp, gi);
-            typename Op::Pre pre[2] = {};
+    const int zero = ts - tl + g.H * g.nxp + g.H;  // the chunk of zeros, from a row's offset
+    // Of the strip's rows: the gather's offsets in a chunk, less the halo
+    // (ps_row_off), and this warp's row block.  Consecutive groups are of one
+    // strip, and the divisions by nx would cost a round 2 us.
+    Dot<A> dots;  // dot ops: this warp's sums over the block's groups
+    int strip = -1, rl[4], row[kRunNb], rp[kRunNb], ax[kRunNb], ay[kRunNb];
+    for (int r = 0; r < nr; ++r) {
+        const int buf = r & 1;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if ((k & 1) == wi && G.row[k] >= 0) pre[k >> 1] = op.pre(G, k);
-            const int q = gi - G.z * g.gpl, y0 = q * kGroup / g.nx;
-            int rl[4];
+        for (int h = 0; h < 2; ++h) {  // round r + 1
+            fetch(ch[h], h, buf ^ 1);
+            ch[h] = chunk(r + 2, h);
+        }
+        const Grp nxt = group(r + 1);
+        if (cur.nt > 0) {
+            const int4 ge = s_grp[r * kRunGroups + set];
+            const int z = ge.x, q = ge.y, own = ge.z;
+            if (q != strip) {
+                strip = q;
+                const GroupRows G = group_rows_at(g, 0, q);
+                const int y0 = q * kGroup / g.nx;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)  // the row's offset in its chunk, less the halo (ps_row_off)
-                rl[k] = G.row[k] >= 0 ? G.rp[k] - G.z * g.lp - (y0 + g.H) * g.nxp - g.H : 0;
+                for (int k = 0; k < 4; ++k) {
+                    rl[k] = G.row[k] >= 0 ? G.rp[k] - (y0 + g.H) * g.nxp - g.H : 0;
+                    if (k % kRunW == wi) {
+                        row[k / kRunW] = G.row[k];
+                        rp[k / kRunW] = G.rp[k];
+                        ax[k / kRunW] = G.ax[k];
+                        ay[k / kRunW] = G.ay[k];
+                    }
+                }
+            }
+            GroupRows G;  // this warp's row blocks, each in kRunW places
+            G.z = z;
+            G.t0 = cur.t0;
+            G.nt = cur.nt;
+            G.vb = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int b = k / kRunW;
+                G.row[k] = row[b] >= 0 ? z * g.nxy + row[b] : -1;
+                G.rp[k] = z * g.lp + rp[b];
+                G.ax[k] = ax[b];
+                G.ay[k] = ay[b];
+            }
+            typename Op::Pre pre[kRunNb] = {};
+#pragma unroll
+            for (int b = 0; b < kRunNb; ++b)
+                if (row[b] >= 0) pre[b] = op.pre(G, b * kRunW);
             A a[NA];
 #pragma unroll
             for (int m = 0; m < NA; ++m) a[m] = A(0);
-            const int *to = toff + ((buf * kRunGroups + set) * 2 + wi) * it;
             const float *tb = tile + buf * NV * ts;
-            const int n = (G.nt + 1) / 2;  // both warps walk as many (an odd template: one of zeros)
-            for (int i0 = 0; i0 < n; i0 += kRunPf) {
-                const bool more = i0 + kRunPf < n;
-                const float *src = more ? p + (size_t)(i0 + kRunPf) * 2 * kGroup : pn ? pn : p;
-                const unsigned long long po = policy(more ? r : r + 1);
-                int off[kRunPf];
-#pragma unroll
-                for (int i = 0; i < kRunPf; i += 4) {
-                    const int4 t = *reinterpret_cast<const int4 *>(to + i0 + i);
-                    off[i] = t.x;
-                    off[i + 1] = t.y;
-                    off[i + 2] = t.z;
-                    off[i + 3] = t.w;
-                }
+            const int n = (cur.nt + kRunW - 1) / kRunW;  // every warp walks as many (past the last slot: zeros)
+            auto step = [&](int i0, const Grp &from, unsigned long long pol, int next) {
 #pragma unroll
                 for (int i = 0; i < kRunPf; ++i) {
-                    const int t = wi + 2 * (i0 + i);
-                    const auto si = op.slot(gp, G.t0 + (t < G.nt ? t : 0));
+                    const int t = wi + kRunW * (i0 + i);
+                    const bool in = t < cur.nt;
+                    const float *tq = tb + (in ? own + po[i] : zero);
+                    const auto si = op.slot(gp, cur.t0 + (in ? t : 0));
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) op.add_t(a, k, pf[i][k], tb + off[i] + rl[k], ts, si);
-                    ld_quad(src + (size_t)i * 2 * kGroup, pf[i], po);
+                    for (int k = 0; k < 4; ++k) op.add_t(a, k, pf[i][k], tq + rl[k], ts, si);
+                    load(from, pol, i, next + i);
                 }
-            }
+            };
+            int i0 = 0;
+            const unsigned long long pol = policy(r);
+            for (; i0 + kRunPf < n; i0 += kRunPf) step(i0, cur, pol, i0 + kRunPf);
+            step(i0, nxt.nt > 0 ? nxt : cur, policy(r + 1), 0);
 #pragma unroll
             for (int m = 0; m < NA; ++m) sh[w][m][lane] = a[m];
-            asm volatile("bar.sync %0, 64;" ::"r"(1 + set) : "memory");
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(32 * kRunW) : "memory");
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if ((k & 1) == wi) finish_block<2>(op, sh + 2 * set, G, pre[k >> 1], gi, k);
-        } else if (pn) {  // nothing in this round, something in the next
+                if (k % kRunW == wi) finish_block<kRunW>(op, sh + kRunW * set, G, pre[k / kRunW], z * g.gpl + q, k,
+                                                             dot_op<Op>::value > 0 ? &dots : nullptr);
+        } else if (nxt.nt > 0) {  // nothing in this round, something in the next
 #pragma unroll
-            for (int i = 0; i < kRunPf; ++i) ld_quad(pn + (size_t)i * 2 * kGroup, pf[i], policy(r + 1));
+            for (int i = 0; i < kRunPf; ++i) load(nxt, policy(r + 1), i, i);
         }
-        gi = gn;
-        p = pn;
+        cur = nxt;
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
     }
+    if constexpr (dot_op<Op>::value > 0) {  // the block's sums: part[i * pstride + block]
+        double *ds = (double *)sh;
+        if ((lane & 3) == 0) ds[8 * w + (lane >> 2)] = dots.bits();
+        __syncthreads();
+        if (tid < Op::kDots) {
+            Dot<A> t;
+            for (int i = 0; i < kRunW * kRunGroups; ++i) t.join(Dot<A>::from(ds[8 * i + tid]));
+            op.part[(size_t)tid * op.pstride + blockIdx.x] = t.bits();
+        }
+    }
+}
+// whether passes of Op run in rounds
+template <class Op>
+inline bool run_in_rounds(const GridC &g, const GraphP &gp) {
+    return g.run && run_layout<Op>(g, gp.rd_nc, gp.rd_tl, gp.rd_max).end <= (size_t)kRunSmemMax;
 }
 
 template <class Op>
@@ -749,7 +832,7 @@ static void run_rounds(cudaStream_t st, const GridC &g, const GraphP &gp, const 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)gp.rd_nb);
     cfg.blockDim = dim3(kRunThreads);
-    cfg.dynamicSmemBytes = std::max(run_smem<Op>(g, gp), (size_t)116 * 1024);  // one block per SM
+    cfg.dynamicSmemBytes = std::max(run_layout<Op>(g, gp.rd_nc, gp.rd_tl, gp.rd_max).end, (size_t)116 * 1024);  // one block per SM
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -825,7 +908,7 @@ static void run_op(cudaStream_t st, const GridC &g, const GraphP &gp, const T *v
     const int ngroups = (kind == 0 ? g.nz + 1 : g.nz) * g.gpl;
     if (ngroups <= 0) return;
     if constexpr (sizeof(T) == 4 && tile_op<Op>::value > 0) {
-        if (g.run && run_smem<Op>(g, gp) <= (size_t)kRunSmemMax) {
+        if (run_in_rounds<Op>(g, gp)) {
             run_rounds(st, g, gp, val, op, kind);
             return;
         }
