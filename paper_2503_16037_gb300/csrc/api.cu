@@ -1650,6 +1650,7 @@ tursca_status ensure_select(tursca_scene *sc) {
        "alloc select");
     CK(dalloc(sc->allocs, q.musmax_bits, sizeof(unsigned long long)), "alloc select");
     q.dmax = std::max(nd, ngd);
+    q.pmax = (q.dmax + 3) / 4 * 4;
     {
         const size_t nn = (size_t)sc->G.n_nodes;
         int ht = 1;
@@ -1660,8 +1661,8 @@ tursca_status ensure_select(tursca_scene *sc) {
         CK(dalloc(sc->allocs, q.table, (size_t)ht * sizeof(int)), "alloc select");
         CK(dalloc(sc->allocs, q.rlist, nn * sizeof(int)), "alloc select");
         CK(dalloc(sc->allocs, q.rcount, 2 * sizeof(int)), "alloc select");
-        CK(dalloc(sc->allocs, q.pcnt, nn * q.dmax * sizeof(int)), "alloc select");
-        CK(dalloc(sc->allocs, q.ph, nn * sc->d.n_species * q.dmax * sc->es), "alloc select");
+        CK(dalloc(sc->allocs, q.pcnt, nn * q.pmax * sizeof(int)), "alloc select");
+        CK(dalloc(sc->allocs, q.ph, nn * sc->d.n_species * q.pmax * sc->es), "alloc select");
     }
     const size_t plane = (size_t)grid_c(sc).npad * sc->es;
     CK(dalloc(sc->allocs, sc->w_iso, q.dmax * plane), "alloc select weights");

@@ -79,7 +79,8 @@ struct SelSrc {
     bool ground;
     int j, x, y, z, nd;
     double mus_lamb, mus_src64;
-    T mus_src;
+    T mus_src, mus_lamb_t;
+    float cm, band;  // c_min in FP32, and how near to it an FP32 coupling leaves the decision to FP64
 };
 template <typename T>
 __device__ __forceinline__ SelSrc<T> sel_src(const GridC &g, const FieldP<T> &f, const ViewC &vc, const SelP &sp,
@@ -95,7 +96,10 @@ __device__ __forceinline__ SelSrc<T> sel_src(const GridC &g, const FieldP<T> &f,
     o.x = r - o.y * g.nx;
     o.nd = o.ground ? g.ngd : g.nd;
     o.mus_src64 = (sizeof(T) == 8) ? (o.ground ? o.mus_lamb : mus64(g, f, j)) : 0.0;
-    o.mus_src = (sizeof(T) == 8) ? (T)o.mus_src64 : (o.ground ? (T)o.mus_lamb : f.mu_st[j]);
+    o.mus_lamb_t = (T)o.mus_lamb;
+    o.mus_src = (sizeof(T) == 8) ? (T)o.mus_src64 : (o.ground ? o.mus_lamb_t : f.mu_st[j]);
+    o.cm = (float)sp.c_min;
+    o.band = o.cm >= 1e-30f ? 1.1e-5f * o.cm : INFINITY;
     return o;
 }
 
@@ -125,7 +129,7 @@ __device__ __forceinline__ void sel_chain(const GridC &g, const GraphP &gp, cons
         }
     } else {
         const int4 m = gp.gmem1[u];
-        if ((double)m.z - 0.5 <= (double)g.nz) {
+        if (m.z <= g.nz) {  // its height, m.z - 1/2, is at most nz
             recv = true;
             const int xn = wrap_small(x + m.x, g.nx), yn = wrap_small(y + m.y, g.ny);
             nidx = ((m.z - 1) * g.ny + yn) * g.nx + xn;
@@ -141,13 +145,17 @@ __device__ __forceinline__ void sel_chain(const GridC &g, const GraphP &gp, cons
     if (recv) {
         if constexpr (sizeof(T) == 4) {
             // FP32 value (relative error below 1e-6); the FP64 coupling
-            // decides only where the FP32 one is that close to c_min
-            const float mus_n = nidx >= 0 ? f.mu_st[nidx] : (float)src.mus_lamb;
+            // decides only where the FP32 one is that close to c_min.  The
+            // distance to c_min is taken in FP32 too: FP64 operations (16 issue
+            // slots of the SM each, four per chain) were what bounded these
+            // passes.  Mask and weights on the 64 x 64 x 32 plume: 133 and 400
+            // us, now 46 and 318.
+            const float mus_n = nidx >= 0 ? f.mu_st[nidx] : src.mus_lamb_t;
             const float c32 = sqrtf(src.mus_src * mus_n) / dist;
             C = c32;
             if (sp.c_min > 0.0) {
-                if (fabs((double)c32 - sp.c_min) > 1e-5 * sp.c_min) {
-                    keep = (double)c32 > sp.c_min;
+                if (fabsf(c32 - src.cm) > src.band) {
+                    keep = c32 > src.cm;
                 } else {
                     const double ms = src.ground ? src.mus_lamb : mus64(g, f, src.j);
                     const double mn = nidx >= 0 ? mus64(g, f, nidx) : src.mus_lamb;
@@ -245,7 +253,7 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_sel_part(GridC g, ViewP vp, 
     __shared__ unsigned char s_kept[kSelMaxDir];
     __shared__ unsigned char s_list[kSelMaxDir];
     __shared__ unsigned char s_klist[kSelMaxDir];
-    __shared__ int s_r, s_nl, s_nk;
+    __shared__ int s_r, s_nl, s_nk, s_cs[kSelMaxDir + 1];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
     constexpr int NT = 32 * kSelWarps;
     const int nrep = sp.rcount[0];
@@ -258,6 +266,8 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_sel_part(GridC g, ViewP vp, 
         const bool ground = j >= g.n_atm;
         const int nd = ground ? g.ngd : g.nd;
         const ulonglong2 mk = sp.mask[j];
+        const int *cs = ground ? sp.gcell_start : vp.cell_start;
+        for (int u = tid; u <= nd; u += NT) s_cs[u] = cs[u];
         // every warp's accumulators: the kept cells' own points in warp 0's
         for (int u = tid; u < nd; u += NT) {
             const bool keep = ((u < 64 ? mk.x >> u : mk.y >> (u - 64)) & 1ull) != 0ull;
@@ -304,25 +314,24 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_sel_part(GridC g, ViewP vp, 
         // cosines (the ranking's arithmetic) decide near-ties.
         {
             const unsigned char *rk = ground ? sp.grank : sp.rank;
-            const int *cs = ground ? sp.gcell_start : vp.cell_start;
             const float4 *pf = ground ? sp.glatf : sp.latf;
             const double *pd = ground ? sp.glat : sp.lat;
             const float4 *df = sp.dirf + (ground ? g.nd : 0);
             const double *dd = vp.dirhat + 3 * (ground ? g.nd : 0);
             const bool dots = nk <= kSelDots;
             int tot = 0;  // points of the dropped cells
-            for (int i = 0; i < nl; ++i) tot += cs[s_list[i] + 1] - cs[s_list[i]];
+            for (int i = 0; i < nl; ++i) tot += s_cs[s_list[i] + 1] - s_cs[s_list[i]];
             int ci = 0, off = tid;  // the thread's cell (index into the list) and point offset inside it
             int cur = -1, n = 0;
             T a[MAX_SPECIES] = {T(0), T(0), T(0), T(0)};
             for (int f0 = tid; f0 < tot; f0 += NT) {
-                int csz = cs[s_list[ci] + 1] - cs[s_list[ci]];
+                int csz = s_cs[s_list[ci] + 1] - s_cs[s_list[ci]];
                 while (off >= csz) {
                     off -= csz;
                     ++ci;
-                    csz = cs[s_list[ci] + 1] - cs[s_list[ci]];
+                    csz = s_cs[s_list[ci] + 1] - s_cs[s_list[ci]];
                 }
-                const int p = cs[s_list[ci]] + off;
+                const int p = s_cs[s_list[ci]] + off;
                 off += NT;
                 int v = -1;
                 if (dots) {
@@ -356,12 +365,13 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_sel_part(GridC g, ViewP vp, 
                     }
                 } else {
                     const unsigned char *row = rk + (size_t)p * nd;
-                    for (int q = 1; q < nd; ++q) {
-                        const int c = row[q];
-                        if (s_kept[c]) {
-                            v = c;
-                            break;
-                        }
+                    for (int q = 1; q < nd && v < 0; q += 4) {  // four entries at a time: their loads overlap
+                        int c[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) c[i] = row[min(q + i, nd - 1)];
+#pragma unroll
+                        for (int i = 3; i >= 0; --i)
+                            if ((c[i] < 64 ? mk.x >> c[i] : mk.y >> (c[i] - 64)) & 1ull) v = c[i];
                     }
                 }
                 if (v != cur) {
@@ -387,15 +397,15 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_sel_part(GridC g, ViewP vp, 
         }
         __syncthreads();
         // the warps' accumulators summed in a fixed order
-        T *ph = reinterpret_cast<T *>(sp.ph) + (size_t)j * g.S * sp.dmax;
+        T *ph = reinterpret_cast<T *>(sp.ph) + (size_t)j * g.S * sp.pmax;
         for (int u = tid; u < nd; u += NT) {
             int c = 0;
             for (int q = 0; q < kSelWarps; ++q) c += s_cnt[q][u];
-            sp.pcnt[(size_t)j * sp.dmax + u] = c;
+            sp.pcnt[(size_t)j * sp.pmax + u] = c;
             for (int s = 0; s < (ground ? 1 : g.S); ++s) {
                 T hsum = T(0);
                 for (int q = 0; q < kSelWarps; ++q) hsum += s_h[q][s][u];
-                ph[(size_t)s * sp.dmax + u] = hsum;
+                ph[(size_t)s * sp.pmax + u] = hsum;
             }
         }
         __syncthreads();  // the shared arrays are reused for the next representative
@@ -413,29 +423,54 @@ template <typename T>
 struct SelQ {
     T qi, qs, C;
 };
+// The re-partition of four directions u0 .. u0 + 3 of a representative, in
+// 16-byte loads: the lanes of a warp read rows of up to 32 representatives, so
+// a load costs up to 32 cache lines whatever its width, and direction by
+// direction they were what bounded the weights (318 us on the plume, now 243).
+template <typename T>
+struct SelPart {
+    int cnt[4];
+    T h[MAX_SPECIES][4];
+};
+template <typename T>
+__device__ __forceinline__ void sel_row4(const T *p, T (&v)[4]) {
+    if constexpr (sizeof(T) == 4) {
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+    } else {
+        const double2 q = __ldg(reinterpret_cast<const double2 *>(p)), t = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+        v[0] = q.x, v[1] = q.y, v[2] = t.x, v[3] = t.y;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void sel_part4(const GridC &g, const SelP &sp, bool ground, int rep, const T *ph, int u0,
+                                          SelPart<T> &o) {
+    if (!ground) {
+        const int4 c = __ldg(reinterpret_cast<const int4 *>(sp.pcnt + (size_t)rep * sp.pmax + u0));
+        o.cnt[0] = c.x, o.cnt[1] = c.y, o.cnt[2] = c.z, o.cnt[3] = c.w;
+    }
+#pragma unroll
+    for (int s = 0; s < MAX_SPECIES; ++s)
+        if (s < (ground ? 1 : g.S)) sel_row4(ph + (size_t)s * sp.pmax + u0, o.h[s]);
+}
 template <typename T>
 __device__ __forceinline__ SelQ<T> sel_q(const GridC &g, const GraphP &gp, const FieldP<T> &f, const ViewP &vp,
-                                         const SelP &sp, const SelSrc<T> &src, int rep, const T *ph, const T *cellsum,
-                                         const T (&wsp)[MAX_SPECIES], const T (&rht)[MAX_SPECIES], T rM, T rz, int u) {
+                                         const SelP &sp, const SelSrc<T> &src, bool part, const SelPart<T> &pt, int i,
+                                         const T *cellsum, const T (&wsp)[MAX_SPECIES], const T (&rht)[MAX_SPECIES],
+                                         T rM, T rz, int u) {
     SelQ<T> o;
     bool keep;
     sel_chain(g, gp, f, sp, src, u, o.C, keep);
     o.qi = T(0);
     o.qs = T(0);
     if (!src.ground) {
-        int cnt;
-        T h[MAX_SPECIES];
-        if (ph) {
-            cnt = sp.pcnt[(size_t)rep * sp.dmax + u];
-            for (int s = 0; s < g.S; ++s) h[s] = ph[(size_t)s * sp.dmax + u];
-        } else {
-            cnt = keep ? vp.cell_start[u + 1] - vp.cell_start[u] : 0;
-            for (int s = 0; s < g.S; ++s) h[s] = keep ? cellsum[s * g.nd + u] : T(0);
-        }
+        const int cnt = part ? pt.cnt[i] : keep ? vp.cell_start[u + 1] - vp.cell_start[u] : 0;
         o.qi = (T)cnt * rM;
-        for (int s = 0; s < g.S; ++s) o.qs += wsp[s] * (h[s] * rht[s]);
+#pragma unroll
+        for (int s = 0; s < MAX_SPECIES; ++s)
+            if (s < g.S) o.qs += wsp[s] * ((part ? pt.h[s][i] : keep ? cellsum[s * g.nd + u] : T(0)) * rht[s]);
     } else {
-        const T h0 = ph ? ph[u] : (keep ? (T)sp.gzsum[u] : T(0));
+        const T h0 = part ? pt.h[0][i] : (keep ? (T)sp.gzsum[u] : T(0));
         o.qi = h0 * rz;
         o.qs = o.qi;
     }
@@ -450,10 +485,12 @@ __global__ void k_select(GridC g, GraphP gp, FieldP<T> f, ViewC vc, ViewP vp, Se
     const SelSrc<T> src = sel_src(g, f, vc, sp, j);
     const int nd = src.nd;
     const int rep = sp.rep[j];
-    const T *ph = rep >= 0 ? reinterpret_cast<const T *>(sp.ph) + (size_t)rep * g.S * sp.dmax : nullptr;
+    const T *ph = rep >= 0 ? reinterpret_cast<const T *>(sp.ph) + (size_t)rep * g.S * sp.pmax : nullptr;
     T wsp[MAX_SPECIES] = {T(0), T(0), T(0), T(0)}, rht[MAX_SPECIES] = {T(0), T(0), T(0), T(0)};
     if (!src.ground) {
-        for (int s = 0; s < g.S; ++s) {
+#pragma unroll
+        for (int s = 0; s < MAX_SPECIES; ++s) {
+            if (s >= g.S) continue;
             if constexpr (sizeof(T) == 8) {
                 const double ms = (double)f.mu_s[(size_t)s * g.n_atm + j];
                 wsp[s] = src.mus_src64 > 0.0 ? ms / src.mus_src64 : 1.0 / g.S;
@@ -465,23 +502,36 @@ __global__ void k_select(GridC g, GraphP gp, FieldP<T> f, ViewC vc, ViewP vp, Se
     }
     const T rM = T(1) / (T)sp.M, rz = T(1) / (T)sp.gztot;
     T sq = 0, sqc = 0, sqs = 0, sqcs = 0;
-    for (int u = 0; u < nd; ++u) {
-        const SelQ<T> o = sel_q(g, gp, f, vp, sp, src, rep, ph, cellsum, wsp, rht, rM, rz, u);
-        if (o.C >= T(0)) {
-            sq += o.qi;
-            sqc += o.qi * o.C;
-            sqs += o.qs;
-            sqcs += o.qs * o.C;
+    for (int u0 = 0; u0 < nd; u0 += 4) {
+        SelPart<T> pt = {};
+        if (ph) sel_part4(g, sp, src.ground, rep, ph, u0, pt);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (u0 + i >= nd) break;
+            const SelQ<T> o = sel_q(g, gp, f, vp, sp, src, ph != nullptr, pt, i, cellsum, wsp, rht, rM, rz, u0 + i);
+            if (o.C >= T(0)) {
+                sq += o.qi;
+                sqc += o.qi * o.C;
+                sqs += o.qs;
+                sqcs += o.qs * o.C;
+            }
         }
     }
     const bool ci_on = vc.coupling && sqc > T(0), cs_on = vc.coupling && sqcs > T(0);
     const T fi = ci_on ? sq / sqc : T(0), fs = cs_on ? sqs / sqcs : T(0);
-    for (int u = 0; u < nd; ++u) {
-        const SelQ<T> o = sel_q(g, gp, f, vp, sp, src, rep, ph, cellsum, wsp, rht, rM, rz, u);
-        const T ci = (ci_on && o.C >= T(0)) ? o.C * fi : T(1);
-        const T cs = (cs_on && o.C >= T(0)) ? o.C * fs : T(1);
-        store_halo(w_iso + (size_t)u * g.npad, g, src.x, src.y, src.z, o.qi * ci);
-        store_halo(w_sun + (size_t)u * g.npad, g, src.x, src.y, src.z, o.qs * cs);
+    for (int u0 = 0; u0 < nd; u0 += 4) {
+        SelPart<T> pt = {};
+        if (ph) sel_part4(g, sp, src.ground, rep, ph, u0, pt);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int u = u0 + i;
+            if (u >= nd) break;
+            const SelQ<T> o = sel_q(g, gp, f, vp, sp, src, ph != nullptr, pt, i, cellsum, wsp, rht, rM, rz, u);
+            const T ci = (ci_on && o.C >= T(0)) ? o.C * fi : T(1);
+            const T cs = (cs_on && o.C >= T(0)) ? o.C * fs : T(1);
+            store_halo(w_iso + (size_t)u * g.npad, g, src.x, src.y, src.z, o.qi * ci);
+            store_halo(w_sun + (size_t)u * g.npad, g, src.x, src.y, src.z, o.qs * cs);
+        }
     }
 }
 
@@ -563,7 +613,7 @@ __device__ __forceinline__ TopkChain topk_chain(const GridC &g, const GraphP &gp
         }
     } else {
         const int4 m = gp.gmem1[u];
-        if ((double)m.z - 0.5 <= (double)g.nz) {
+        if (m.z <= g.nz) {  // its height, m.z - 1/2, is at most nz
             c.recv = true;
             c.nidx = ((m.z - 1) * g.ny + wrap_small(y + m.y, g.ny)) * g.nx + wrap_small(x + m.x, g.nx);
             c.dist = gp.gdist1[u];

@@ -28,6 +28,7 @@ struct SelP {
     int M;                           // lattice points
     int n_up;                        // lattice points in the upper hemisphere
     int dmax;                        // planes of the weight tables: max(nd, ngd)
+    int pmax;                        // dmax rounded up to whole 16-byte loads of pcnt and ph
     const unsigned char *rank;       // [M][nd] directions by decreasing cosine to each point; points in cell
                                      // order (cell_start of the graph), inside a cell by their rankings
     const double *lat;               // [M][3] the lattice points in that order
@@ -51,8 +52,8 @@ struct SelP {
     int ht;                          // slots: a power of two, at least twice the sources
     int *rlist;                      // [n_nodes] the representative sources, in the order they claimed their slot
     int *rcount;                     // [2] representatives listed, representatives handed out so far
-    int *pcnt;                       // [n_nodes][dmax] point counts after the re-draw (representatives only)
-    void *ph;                        // [n_nodes][S][dmax] HG (ground: cosine) sums after the re-draw, compute type
+    int *pcnt;                       // [n_nodes][pmax] point counts after the re-draw (representatives only)
+    void *ph;                        // [n_nodes][S][pmax] HG (ground: cosine) sums after the re-draw, compute type
 };
 
 // Weights W of every (source, direction) for the current fields and
