@@ -92,7 +92,7 @@ def tf32_peak():
 TRAFFIC_SOURCES = {
     "k_tile_OpCheb": ("kernels_solve.cu", "stage.cuh", "kern.h"),
     "assembly": ("kernels_asm.cu", "asm_util.cuh", "stage.cuh", "kern.h"),
-    "cloud_gmres_prod": ("kernels_solve.cu", "stage.cuh", "kern.h"),
+    "cloud_bicgstab_prod": ("kernels_solve.cu", "stage.cuh", "kern.h"),
 }
 
 
@@ -671,9 +671,9 @@ def main():
                      "solve": {"iters": crn.info.iters, "refinements": crn.info.refinements,
                                "solver": crn.info.solver, "rel_resid64": crn.info.rel_resid64},
                      "timing": "host clock around a synchronised scene, median of 5, L2 flushed"}
-            # roofline of the passes over K inside GMRES (K = 4 nnz bytes of
-            # values, far beyond L2): one profiled scene, events around each
-            # Arnoldi step's run of passes (preconditioner and I - K product)
+            # roofline of the products with K inside BiCGStab (K = 4 nnz bytes
+            # of values, far beyond L2): one profiled scene, events around each
+            # step's two passes and their vector kernels
             flush.zero_()
             T.tursca_profile_enable(crn.handle, True)
             crn.run(ca, cm, rtol=RTOL)
@@ -685,14 +685,14 @@ def main():
                 avg_s = ms_gp / n_gp / 1000.0
                 peak, peak_kind = peaks()
                 cloud["roofline"] = {
-                    "kernel": "passes over K inside GMRES (k_tile<6, OpSpmv/OpImk<float>>: y = b + K x or "
-                              "y = x - K x, K read once per pass)", "bound": "hbm",
+                    "kernel": "BiCGStab steps, per product with K (k_run<OpBi<float>>: y = x - K x with its dot "
+                              "products, K read once per pass; half of k_bi_s and k_bi_p included)", "bound": "hbm",
                     "achieved": pb / avg_s / 1e9, "peak": peak, "unit": "GB/s",
                     "frac": pb / avg_s / 1e9 / peak, "peak_kind": peak_kind + " (hbm_gbs, copy)",
                     "algorithmic_bytes_per_launch": pb, "avg_launch_us": avg_s * 1e6, "launches": n_gp,
-                    "traffic": traffic_record("cloud_gmres_prod"),
-                    "timing": "CUDA events on the scene stream around each Arnoldi step's passes over K, one "
-                              "profiled scene, averaged per pass"}
+                    "traffic": traffic_record("cloud_bicgstab_prod"),
+                    "timing": "CUDA events on the scene stream around each BiCGStab step (two passes over K and "
+                              "two vector kernels), one profiled scene, averaged per pass"}
             crn.close()
         except Exception as e:
             cloud = {"error": str(e)[:200]}

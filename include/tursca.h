@@ -172,18 +172,20 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
  * evaluated in FP64, with at most max_iter inner steps (a sweep, a Chebyshev
  * step, or a GMRES step, which applies K twice).  The outer loop is FP64
  * residual refinement; each refinement solves for the correction with inner
- * iterations in the scene's precision.  Scenes whose matrix stays on the chip
- * and in L2 (in FP32 up to about 1100 groups of 128 rows at radius 2: the 64 x
- * 64 x 32 plume) are solved in one cooperative launch, by BiCGStab from the
- * source to the refined solution.  Others run pass by pass: FP32_REFINE scenes
- * first a few Neumann sweeps (the series of Eq. fs_sum) that also estimate the
- * largest eigenvalue of K, then Chebyshev iterations on the interval that
- * estimate implies, or GMRES when the estimate is 0.85 or more or a Chebyshev
- * refinement under-delivers; FP64 scenes run GMRES.  GMRES(30) (FP64: 40)
- * is right-preconditioned with I + K, the first two terms of that series.
+ * iterations in the scene's precision.  Scenes with up to about 200 MB of
+ * matrix values beyond shared memory (in FP32 up to about 3,000 groups of 128
+ * rows at radius 2: 96 x 96 x 32) are solved in one cooperative launch, by
+ * BiCGStab from the source to the refined solution.  Others run pass by pass:
+ * FP32_REFINE scenes first a few Neumann sweeps (the series of Eq. fs_sum) that
+ * also estimate the largest eigenvalue of K, then Chebyshev iterations on the
+ * interval that estimate implies, or BiCGStab (two products with K per step)
+ * when the estimate is 0.85 or more or a Chebyshev refinement under-delivers;
+ * FP64 scenes run BiCGStab.  Where BiCGStab breaks down, GMRES(30) (FP64: 40),
+ * right-preconditioned with I + K, the first two terms of that series, goes on.
  * TURSCA_OPT_GROUP_WARPS, TURSCA_OPT_STAGE_VALUES and TURSCA_OPT_RESIDUAL_FP64
  * name how passes run, so setting one of them selects the passes.
- * Synchronises once (the passes: once per refinement, GMRES: once per step).
+ * Synchronises once (the passes: once per refinement, BiCGStab and GMRES: once
+ * per step, BiCGStab with the next step already queued).
  * info may be NULL. */
 tursca_status tursca_solve(tursca_scene *scene, double rtol, int max_iter, tursca_solve_info *info);
 
@@ -429,6 +431,10 @@ tursca_status tursca_quadrature(const tursca_grid_desc *desc, double *q_iso, dou
  * the array's address cannot be found; TURSCA_E_CUDA when a launch fails (the
  * call stops at the first failed launch; later asynchronous faults surface at
  * the caller's next synchronisation).
+ * Up to 131,072 nodes the whole solve is one cooperative launch (blocks that
+ * keep their rows in shared memory and meet a bounded grid barrier per sweep;
+ * should a barrier give up, x and resid2 are NaN); larger systems take a
+ * launch per sweep.
  * The call allocates nothing and returns without synchronising. */
 tursca_status tursca_csr_solve_noalloc(const int32_t *row_ptr, const int32_t *col, const float *val, int n_nodes,
                                        const float *s, double *x, int sweeps, int refinements, double *resid2,
@@ -492,8 +498,8 @@ typedef struct {
  * request:
  *   TURSCA_SERVER_BATCH_SOLVES: 0 (default) runs every request's solve on
  *     its own stream; 1 batches the solves of the requests that run at the
- *     same time: the solves that wait while a launch runs are launched
- *     together in one persistent kernel, side by side, each on its own blocks
+ *     same time: the solves that wait while a launch runs (and for up to a
+ *     millisecond, when a solve would run alone) are launched together in one persistent kernel, side by side, each on its own blocks
  *     with its own barrier (every wait bounded) and its own convergence, so a
  *     result does not depend on what it ran beside.  FP32 + refinement scenes
  *     whose solve takes at most three quarters of the GPU's blocks. */

@@ -25,7 +25,8 @@
 // exchange.  Measured on the plume, per step of two products: 6.4 and 6.6 us
 // of products, 1.5 and 2.0 us of barriers, 1.5 and 2.7 us of vector updates.
 // Whole solve 444 us (plume), 400 us (random 45 x 37 x 29: 1160 us with passes
-// and GMRES), 135 us (plume 16^3).  FP64 is kept off the common path of FP32
+// and GMRES), 115 us (plume 16^3), about 1.1 ms (96 x 96 x 32, 150 MB of values
+// of which L2 keeps 80).  FP64 is kept off the common path of FP32
 // scenes (an FP64 warp operation takes 16 issue slots of the SM): dot products
 // are FP32 pairs, 48 bits, and the outer loop's scalars are one thread's.
 //

@@ -670,7 +670,7 @@ void launch_finalize(cudaStream_t st, const double *part, int nblk, double *out)
 // queued ahead of the host, which only reads back the state every few steps.
 // Against GMRES(30) with I + K as preconditioner it needs no basis: on the
 // 128 x 128 x 40 cloud an Arnoldi step spent 107 us on orthogonalisation beside
-// its two passes of 72 us.
+// its two passes of 72 us; a step of this takes 150 us, two passes of 64 us.
 constexpr int kBiParts = 8;  // blocks per sum
 template <typename T>
 __global__ void __launch_bounds__(512) k_bi_sums(const double *__restrict__ part, size_t stride, int n,
