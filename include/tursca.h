@@ -102,7 +102,7 @@ typedef struct {
 } tursca_geometry;
 
 typedef struct {
-    int iters;          /* matrix-vector products with K in the solve */
+    int iters;          /* inner steps and residual evaluations, as max_iter counts them */
     int refinements;    /* outer FP64 residual evaluations */
     double rel_resid64; /* ||s - (I - K) x|| / ||s|| evaluated in FP64 */
     double rho_est;     /* estimate of the spectral radius of K */
@@ -170,7 +170,8 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
 
 /* Solve (I - K) x = s (Eq. flux_system) to ||s - (I - K) x|| <= rtol ||s||
  * evaluated in FP64, with at most max_iter inner steps (a sweep, a Chebyshev
- * step, or a GMRES step, which applies K twice).  The outer loop is FP64
+ * step, or a GMRES or BiCGStab step, which apply K twice); a residual
+ * evaluation counts as a step.  The outer loop is FP64
  * residual refinement; each refinement solves for the correction with inner
  * iterations in the scene's precision.  Scenes with up to about 200 MB of
  * matrix values beyond shared memory (in FP32 up to about 3,000 groups of 128

@@ -808,7 +808,7 @@ tursca_status gmres(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &gp, 
 }
 
 // BiCGStab on (I - K) d = b, b = r64, to ||b - (I - K) d|| <= tol ||b|| (the
-// recursion's residual) in at most maxit products, then x += d with the FP32
+// recursion's residual) in at most maxit steps, then x += d with the FP32
 // pair of x.  norm: ||r64||.  Steps are queued kBiChunk at a time, one chunk
 // ahead of the read-back of the state; the passes after the end return at
 // once.  *ok false: the iteration broke down and x is unchanged.
@@ -833,7 +833,7 @@ tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &g
     const double bb = std::ldexp(norm, -ex) * std::ldexp(norm, -ex);
     tk::launch_bi_start<T>(sc->st, n, sc->r64, std::ldexp(1.0, -ex), bb, tol * tol * bb, b, r, p, d, st);
     sc->launches++;
-    const int chunks = std::max(1, (maxit + 2 * kBiChunk - 1) / (2 * kBiChunk));
+    const int chunks = std::max(1, (maxit + kBiChunk - 1) / kBiChunk);
     tk::BiState<T> *h = (tk::BiState<T> *)(sc->hred + 192);  // two read-back slots of 64 bytes
     static_assert(sizeof(tk::BiState<T>) <= 64, "read-back slots");
     auto slot = [&](int c) { return (tk::BiState<T> *)((char *)h + (c & 1) * 64); };
@@ -850,7 +850,7 @@ tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &g
         CK(cudaEventSynchronize(sc->bi_ev[(c - 1) & 1]), "sync");
         if (slot(c - 1)->done || c == chunks) {
             const tk::BiState<T> e = *slot(c - 1);
-            ss.iters += 2 * e.steps;
+            ss.iters += e.steps;
             if (!std::isfinite((double)e.rn)) return TURSCA_OK;
             break;
         }
@@ -1045,7 +1045,7 @@ tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *d
     const tursca_status rs = status_error(sc, (const int *)(sc->hred + 254));
     if (rs) return rs;
     const tk::PsInfo *h = (const tk::PsInfo *)sc->hred;
-    if (sc->ps_prof >= 0) sc->ev_n[sc->ps_prof] = h->iters;
+    if (sc->ps_prof >= 0) sc->ev_n[sc->ps_prof] = 2 * h->iters - h->refinements;
     if (h->state != tk::PS_CONVERGED && h->state != tk::PS_MAX_ITER) {
         sc->x_pair = false;
         return TURSCA_OK;

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
         }
         put_norm(rr);
     }
-    int iters = 0, refinements = 0, state = PS_RUNNING;
+    int iters = 0, refinements = 0, state = PS_RUNNING;  // iters: steps and residuals
     for (;;) {
         // ---- the residual r of the current x is published: its norm, and the tile
         if (!barrier()) return;
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) k_persist(const __grid_constant
             __syncthreads();
             pass(std::integral_constant<int, PS_T>());
             if (!barrier()) return;
-            iters += 2;
+            ++iters;
             bool stop;
             {
                 const T *pv = (const T *)J.pub[(gen - 2) % 3], *pt = (const T *)J.pub[(gen - 1) % 3];

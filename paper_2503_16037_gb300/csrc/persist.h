@@ -14,7 +14,9 @@ constexpr int kPsMaxJobs = 8;  // solves in one launch
 
 // what the solve reports (device, read back by the host)
 struct PsInfo {
-    int iters, refinements, state, pad;  // state 1: converged, 2: stopped at max_iter, 3: gave up
+    // iters: BiCGStab steps (two products each) and residuals (one each), so
+    // 2 iters - refinements products; state 1: converged, 2: stopped at max_iter, 3: gave up
+    int iters, refinements, state, pad;
     double rel, sn;
 };
 enum { PS_RUNNING = 0, PS_CONVERGED = 1, PS_MAX_ITER = 2, PS_GAVE_UP = 3 };
