@@ -182,7 +182,9 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
  * interval that estimate implies, or BiCGStab (two products with K per step)
  * when the estimate is 0.85 or more or a Chebyshev refinement under-delivers;
  * FP64 scenes run BiCGStab.  Where BiCGStab breaks down, GMRES(30) (FP64: 40),
- * right-preconditioned with I + K, the first two terms of that series, goes on.
+ * right-preconditioned with I + K, the first two terms of that series, goes on
+ * (after the one-launch form: the passes, from the x it reached and with what
+ * is left of max_iter).
  * TURSCA_OPT_GROUP_WARPS, TURSCA_OPT_STAGE_VALUES and TURSCA_OPT_RESIDUAL_FP64
  * name how passes run, so setting one of them selects the passes.
  * Synchronises once (the passes: once per refinement, BiCGStab and GMRES: once

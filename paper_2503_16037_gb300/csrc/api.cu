@@ -1037,14 +1037,15 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     return TURSCA_OK;
 }
 
-// Wait for the result of persist_launch.  *done is false when the iteration
-// gave up; the caller's loop then solves from x = 0.
-tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *done) {
+// Wait for the result of persist_launch (*out).  *done is false when the
+// iteration gave up; do_solve then goes on from where it ended.
+tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *done, tk::PsInfo *out) {
     *done = false;
     CK(cudaEventSynchronize(sc->ps_ev), "sync");
     const tursca_status rs = status_error(sc, (const int *)(sc->hred + 254));
     if (rs) return rs;
     const tk::PsInfo *h = (const tk::PsInfo *)sc->hred;
+    *out = *h;
     if (sc->ps_prof >= 0) sc->ev_n[sc->ps_prof] = 2 * h->iters - h->refinements;
     if (h->state != tk::PS_CONVERGED && h->state != tk::PS_MAX_ITER) {
         sc->x_pair = false;
@@ -1099,7 +1100,7 @@ struct L2Window {
 
 template <typename T>
 tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, tursca_solve_info *info,
-                       const SolveIO<T> &io, bool passes = false) {
+                       const SolveIO<T> &io, const tk::PsInfo *gave_up = nullptr) {
     const L2Window l2w(sc, io.val, (size_t)sc->G.nval * sizeof(T));
     const tk::GridC &g = io.g;
     const tk::GraphP &gp = io.gp;
@@ -1112,15 +1113,31 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     (void)nb;
     const bool fp64 = sc->d.precision == TURSCA_FP64;
     sc->x_pair = false;
-    if (solver == TURSCA_SOLVER_AUTO && !passes) {
+    tk::PsInfo prior;
+    if (solver == TURSCA_SOLVER_AUTO && !gave_up) {
         bool launched = false, done = false;
         tursca_status e = persist_launch<T>(sc, io, rtol, max_iter, &launched);
-        if (!e && launched) e = persist_collect(sc, info, &done);
+        if (!e && launched) e = persist_collect(sc, info, &done, &prior);
         if (e || done) return e;
+        if (launched) gave_up = &prior;
     }
     // the automatic choice goes on with BiCGStab where the other solvers take
-    // GMRES (until BiCGStab breaks down, which hands over to GMRES)
-    bool bi = solver == TURSCA_SOLVER_AUTO;
+    // GMRES (until BiCGStab breaks down, here or in the persistent solve,
+    // which hands over to GMRES)
+    bool bi = solver == TURSCA_SOLVER_AUTO && !gave_up;
+    // A persistent solve that gave up has used its share of max_iter; where it
+    // had gained anything its x is kept.
+    const bool resume = gave_up && gave_up->refinements > 0 && gave_up->rel < 1.0;
+    if (gave_up) {
+        ss.iters = gave_up->iters;
+        ss.refinements = gave_up->refinements;
+        ss.solver = TURSCA_SOLVER_BICGSTAB;
+    }
+    const int refinements0 = ss.refinements;
+    // after a hand-over the steps leave room for the two residuals (of a GMRES
+    // cycle and of the refinement) that follow them
+    const int spare = gave_up ? 2 : 0;
+    const bool room = !resume || ss.iters + 1 + spare < max_iter;
     if (solver == TURSCA_SOLVER_AUTO) solver = fp64 ? TURSCA_SOLVER_GMRES : TURSCA_SOLVER_CHEBYSHEV;
     auto ensure_basis = [&]() -> tursca_status {
         int m = fp64 ? 40 : TK_GMRES_M32;
@@ -1136,22 +1153,41 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     // residual arithmetic: FP32 pairs on FP32 scenes (FP64 runs at a small
     // fraction of the FP32 rate on this GPU), FP64 on FP64 scenes or on request
     const bool ds = !fp64 && !sc->resid_fp64 && tk::resid_ds_ok(g);
-    // x = 0, r = s, ||s||
-    CK(cudaMemsetAsync(io.x, 0, (size_t)n * sizeof(double), sc->st), "memset x");
-    tk::launch_to_halo<T, double>(sc->st, g, io.s, sc->r64);
-    // ||s||^2 goes to dred[4] and is read with the first refinement's residual
-    tk::launch_sumsq<double>(sc->st, g, sc->r64, sc->part, nb, sc->dred + 4);
-    sc->launches += 3;
+    // r = s - x + K x, its ||r||^2 in dred[0]
+    auto residual = [&]() {
+        int pr = prof_begin(sc, P_RESID);
+        if (ds)
+            tk::launch_resid_ds(sc->st, g, gp, (const float *)val, (const float *)io.s, io.x, sc->xh, sc->xl,
+                                sc->r64, sc->part, nbr);
+        else
+            tk::launch_resid64<T>(sc->st, g, gp, val, io.s, io.x, sc->r64, sc->part, nbr);
+        prof_end(sc, pr);
+        tk::launch_finalize(sc->st, sc->part, nbr, sc->dred);
+        sc->launches += 2;
+        ss.iters++;
+    };
     tursca_status rs = TURSCA_OK;
     double sn = -1.0;  // not read yet
     double rel = 1.0;
+    if (resume) {
+        sn = gave_up->sn;
+        rel = gave_up->rel;
+        if (room) residual();
+    } else {
+        // x = 0, r = s, ||s||
+        CK(cudaMemsetAsync(io.x, 0, (size_t)n * sizeof(double), sc->st), "memset x");
+        tk::launch_to_halo<T, double>(sc->st, g, io.s, sc->r64);
+        // ||s||^2 goes to dred[4] and is read with the first refinement's residual
+        tk::launch_sumsq<double>(sc->st, g, sc->r64, sc->part, nb, sc->dred + 4);
+        sc->launches += 3;
+    }
     double rho = -1.0;      // estimate of the largest eigenvalue of K (-1: none yet)
     double widen = 0.0;     // extra margin after a refinement that under-delivered
     int inner_n = 8;        // Neumann sweeps (explicit Neumann solver)
     int stalls = 0;
     bool use_gmres = false;       // Chebyshev under-delivered: GMRES from now on
     const double floor32 = 3e-7;  // relative accuracy the FP32 inner iterations can reach
-    while (rel > rtol && ss.iters < max_iter) {
+    while (room && rel > rtol && ss.iters + spare < max_iter) {
         const int budget = max_iter - ss.iters;
         T *bb = (T *)sc->b;  // r in the compute type (written below, with the first pass of each solver)
         // reduction asked of this refinement: all that is left if one
@@ -1271,7 +1307,7 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
                 sn = std::sqrt(sc->hred[4]);
             }
             double tol = fp64 ? std::max(0.3 * rtol / rel, 1e-15) : std::max(0.3 * rtol / rel, 2e-6);
-            e = gmres<T>(sc, g, gp, val, bb, (T *)sc->d0, tol, budget, ss);
+            e = gmres<T>(sc, g, gp, val, bb, (T *)sc->d0, tol, budget - spare, ss);
             if (e) return e;
             dd = (const T *)sc->d0;
             ss.solver = TURSCA_SOLVER_GMRES;
@@ -1282,18 +1318,9 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
             ss.solver = TURSCA_SOLVER_NEUMANN;
         }
         if (!x_done) tk::launch_update_x<T>(sc->st, n, dd, io.x, ds ? sc->xh : nullptr, ds ? sc->xl : nullptr);
-        int pr = prof_begin(sc, P_RESID);
-        if (ds)
-            tk::launch_resid_ds(sc->st, g, gp, (const float *)val, (const float *)io.s, io.x, sc->xh, sc->xl,
-                                sc->r64, sc->part, nbr);
-        else
-            tk::launch_resid64<T>(sc->st, g, gp, val, io.s, io.x, sc->r64, sc->part,
-                                  nbr);
-        prof_end(sc, pr);
-        tk::launch_finalize(sc->st, sc->part, nbr, sc->dred);
-        sc->launches += 3;
+        residual();
+        sc->launches++;  // the update of x, here or in the last pass
         ss.refinements++;
-        ss.iters++;
         rs = read_red<T>(sc, 5);
         if (rs) return rs;
         if (sn < 0.0) sn = std::sqrt(sc->hred[4]);
@@ -1329,7 +1356,7 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
                 inner_n = std::max(2, std::min(want, 400));
             }
         }
-        if (!(rel <= prev * 1.5) && ss.refinements > 3) break;  // diverging
+        if (!(rel <= prev * 1.5) && ss.refinements - refinements0 > 3) break;  // diverging
         if (stalls > 6) break;
     }
     if (info) {
@@ -1412,10 +1439,11 @@ tursca_status solve_render(tursca_scene *sc, double rtol, int max_iter, tursca_s
     *done = true;
     e = render_launch<T>(sc);
     if (e) return e;
-    e = persist_collect(sc, info, &solved);
+    tk::PsInfo h;
+    e = persist_collect(sc, info, &solved, &h);
     if (e) return e;
     if (!solved) {
-        e = do_solve<T>(sc, TURSCA_SOLVER_AUTO, rtol, max_iter, info, io, true);
+        e = do_solve<T>(sc, TURSCA_SOLVER_AUTO, rtol, max_iter, info, io, &h);
         return e ? e : do_render<T>(sc, radiance, reflectance);
     }
     return render_finish<T>(sc, radiance, reflectance);
