@@ -105,7 +105,8 @@ typedef struct {
     int iters;          /* inner steps and residual evaluations, as max_iter counts them */
     int refinements;    /* outer FP64 residual evaluations */
     double rel_resid64; /* ||s - (I - K) x|| / ||s|| evaluated in FP64 */
-    double rho_est;     /* estimate of the spectral radius of K */
+    double rho_est;     /* estimate of the spectral radius of K, by powers of K on s (0: none was formed, as by
+                           TURSCA_SOLVER_GMRES and by the FP64 passes of TURSCA_SOLVER_AUTO) */
     int solver;         /* TURSCA_SOLVER_* actually used */
 } tursca_solve_info;
 

@@ -1037,8 +1037,38 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     return TURSCA_OK;
 }
 
+// Power estimate of K's spectral radius, s.K^7 s / s.K^6 s, from the first
+// steps of a BiCGStab solve that started at r = s.  Its alpha and beta are
+// those of the Lanczos process of I - K with s on both sides, whose k x k
+// tridiagonal T has the moments s.(I - K)^j s / s.s = e1.T^j e1 for j < 2k
+// (Saad 2003, section 7.1), so the moments of I - T are K's.  Moments below
+// 1e-3 have lost the coefficients' digits: then the last ratio before them.
+template <typename T>
+double rho_estimate(tk::PsInfo h) {
+    const T *co = h.coef<T>();
+    double alpha[tk::kPsRec], beta[tk::kPsRec];
+    for (int j = 0; j < tk::kPsRec; ++j) alpha[j] = co[j], beta[j] = co[tk::kPsRec + j];
+    int k = 0;
+    while (k < tk::kPsRec && std::isfinite(alpha[k]) && alpha[k] != 0.0) ++k;
+    double e[tk::kPsRec], c[tk::kPsRec], y[tk::kPsRec] = {1.0}, m = 1.0, est = 0.0;
+    for (int j = 0; j < k; ++j) {
+        e[j] = 1.0 - 1.0 / alpha[j] - (j > 0 ? beta[j - 1] / alpha[j - 1] : 0.0);
+        c[j] = beta[j] / (alpha[j] * alpha[j]);
+    }
+    for (int i = 1; i < 2 * k && m >= 1e-3; ++i) {
+        double z[tk::kPsRec];
+        for (int j = 0; j < k; ++j)
+            z[j] = e[j] * y[j] - (j > 0 ? y[j - 1] : 0.0) - (j + 1 < k ? c[j] * y[j + 1] : 0.0);
+        std::copy(z, z + k, y);
+        est = z[0] / m;
+        m = z[0];
+    }
+    return std::isfinite(est) ? std::min(0.9999, std::max(0.0, est)) : 0.0;
+}
+
 // Wait for the result of persist_launch (*out).  *done is false when the
 // iteration gave up; do_solve then goes on from where it ended.
+template <typename T>
 tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *done, tk::PsInfo *out) {
     *done = false;
     CK(cudaEventSynchronize(sc->ps_ev), "sync");
@@ -1056,7 +1086,7 @@ tursca_status persist_collect(tursca_scene *sc, tursca_solve_info *info, bool *d
         info->iters = h->iters;
         info->refinements = h->refinements;
         info->rel_resid64 = h->rel;
-        info->rho_est = 0.0;
+        info->rho_est = rho_estimate<T>(*h);
         info->solver = TURSCA_SOLVER_BICGSTAB;
     }
     sc->solved = true;
@@ -1117,7 +1147,7 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     if (solver == TURSCA_SOLVER_AUTO && !gave_up) {
         bool launched = false, done = false;
         tursca_status e = persist_launch<T>(sc, io, rtol, max_iter, &launched);
-        if (!e && launched) e = persist_collect(sc, info, &done, &prior);
+        if (!e && launched) e = persist_collect<T>(sc, info, &done, &prior);
         if (e || done) return e;
         if (launched) gave_up = &prior;
     }
@@ -1131,6 +1161,7 @@ tursca_status do_solve(tursca_scene *sc, int solver, double rtol, int max_iter, 
     if (gave_up) {
         ss.iters = gave_up->iters;
         ss.refinements = gave_up->refinements;
+        ss.rho = rho_estimate<T>(*gave_up);
         ss.solver = TURSCA_SOLVER_BICGSTAB;
     }
     const int refinements0 = ss.refinements;
@@ -1440,7 +1471,7 @@ tursca_status solve_render(tursca_scene *sc, double rtol, int max_iter, tursca_s
     e = render_launch<T>(sc);
     if (e) return e;
     tk::PsInfo h;
-    e = persist_collect(sc, info, &solved, &h);
+    e = persist_collect<T>(sc, info, &solved, &h);
     if (e) return e;
     if (!solved) {
         e = do_solve<T>(sc, TURSCA_SOLVER_AUTO, rtol, max_iter, info, io, &h);

@@ -11,6 +11,7 @@
 namespace tk {
 
 constexpr int kPsMaxJobs = 8;  // solves in one launch
+constexpr int kPsRec = 4;      // steps whose coefficients are reported
 
 // what the solve reports (device, read back by the host)
 struct PsInfo {
@@ -18,6 +19,14 @@ struct PsInfo {
     // 2 iters - refinements products; state 1: converged, 2: stopped at max_iter, 3: gave up
     int iters, refinements, state, pad;
     double rel, sn;
+    // alpha, then beta, of the first kPsRec steps in the compute type, from
+    // which the host estimates K's spectral radius (zero at launch; a residual
+    // counts in iters and leaves its entry 0, so the first refinement's end shows)
+    double rec[2 * kPsRec];
+    template <typename T>
+    __host__ __device__ T *coef() {
+        return reinterpret_cast<T *>(rec);
+    }
 };
 enum { PS_RUNNING = 0, PS_CONVERGED = 1, PS_MAX_ITER = 2, PS_GAVE_UP = 3 };
 

@@ -22,6 +22,7 @@ LIB_PATH = os.path.join(HERE, "libtursca_gb.so")
 FP64, FP32_REFINE = 0, 1
 COUPLING_NONE, COUPLING_WEIGHT = 0, 1
 SOLVER_AUTO, SOLVER_NEUMANN, SOLVER_GMRES, SOLVER_CHEBYSHEV = 0, 1, 2, 3
+SOLVER_BICGSTAB = 4  # reported by SOLVER_AUTO, not a value to ask for
 
 OK, E_INVALID, E_NOMEM, E_CUDA, E_NOT_CONVERGED, E_TIMEOUT, E_STATE, E_UNSUPPORTED = range(8)
 
