@@ -186,8 +186,9 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
  * right-preconditioned with I + K, the first two terms of that series, goes on
  * (after the one-launch form: the passes, from the x it reached and with what
  * is left of max_iter).
- * TURSCA_OPT_GROUP_WARPS, TURSCA_OPT_STAGE_VALUES and TURSCA_OPT_RESIDUAL_FP64
- * name how passes run, so setting one of them selects the passes.
+ * TURSCA_OPT_GROUP_WARPS, TURSCA_OPT_STAGE_VALUES, TURSCA_OPT_RESIDUAL_FP64 and
+ * TURSCA_OPT_GATHER_TILE = 0 name how passes run, so setting one of them
+ * selects the passes.
  * Synchronises once (the passes: once per refinement, BiCGStab and GMRES: once
  * per step, BiCGStab with the next step already queued).
  * info may be NULL. */
@@ -270,8 +271,10 @@ tursca_status tursca_get(tursca_scene *scene, tursca_field which, void *dst, siz
  *     and the emission pass, also over K^T in the adjoint) copy each group's
  *     source rows of the vectors they gather from into shared-memory tiles
  *     (at most 48 KB per block; larger groups gather from global memory);
- *     0 always gathers from global memory.  Results are bit-identical
- *     either way.
+ *     0 always gathers from global memory, so TURSCA_SOLVER_AUTO runs its
+ *     passes in place of the one-launch form and large scenes one block per
+ *     group.  Either way the passes sum the same products, in the same order
+ *     for the same TURSCA_OPT_GROUP_WARPS.
  *   TURSCA_OPT_SINGLE_SCATTER: 0 (default); 1 makes the following
  *     assemblies first-order only (single scattering, the branch of the data
  *     flow of Sec. 3 that stops after the direct beam): assemble_flux computes

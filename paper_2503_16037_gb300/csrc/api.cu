@@ -373,7 +373,7 @@ tk::GridC grid_c(const tursca_scene *sc) {
     g.stage = (sc->stage_values && sc->d.precision != TURSCA_FP64 && tk::stage_fits(G.max_row)) ? 1 : 0;
     g.tl = sc->gather_tile ? sc->tile_tl : 0;
     // (options that name how the passes run select those passes)
-    g.run = sc->ps.rd_nb > 0 && sc->wq_auto && !g.stage ? 1 : 0;
+    g.run = sc->ps.rd_nb > 0 && sc->wq_auto && sc->gather_tile && !g.stage ? 1 : 0;
     g.hx = sc->d.hx;
     g.hy = sc->d.hy;
     g.hz = sc->d.hz;
@@ -980,7 +980,7 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     *launched_out = false;
     const tk::PsPlan &P = io.ps->plan;
     sc->x_pair = false;
-    if (P.nb <= 0 || !sc->wq_auto || sc->stage_values || sc->resid_fp64) return TURSCA_OK;
+    if (P.nb <= 0 || !sc->wq_auto || sc->stage_values || sc->resid_fp64 || !sc->gather_tile) return TURSCA_OK;
     if (!sc->ps_ev) CK(cudaEventCreateWithFlags(&sc->ps_ev, cudaEventDisableTiming), "event");
     tk::PsJob J;
     J.g = io.g;
@@ -1577,7 +1577,7 @@ tursca_status do_adjoint(tursca_scene *sc, const void *dJ_dL, void *dJ_dmu_abs) 
     SolveIO<T> io;
     g.stage = 0;
     g.tl = sc->gather_tile ? sc->tile_tlT : 0;
-    g.run = sc->psT.rd_nb > 0 && sc->wq_auto ? 1 : 0;
+    g.run = sc->psT.rd_nb > 0 && sc->wq_auto && sc->gather_tile ? 1 : 0;
     io.g = g;
     io.gp = gpT;
     io.val = (const T *)sc->valT;
