@@ -259,7 +259,8 @@ tursca_status tursca_get(tursca_scene *scene, tursca_field which, void *dst, siz
  *     return TURSCA_E_TIMEOUT.
  *   TURSCA_OPT_L2_RESIDENT: 0 (default); 1 keeps the values of K in the
  *     persisting part of L2 while a solve runs (every pass of a solve streams
- *     the same values).  Setting 1 raises this CUDA context's persisting-L2
+ *     the same values; the one-launch form and the rounds over large scenes
+ *     load most of them with L2 policies of their own).  Setting 1 raises this CUDA context's persisting-L2
  *     set-aside to the device maximum for the rest of the process; each
  *     solve sets an access-policy window over the values on the scene
  *     stream, and on return removes it and resets every persisting line of

@@ -1463,6 +1463,7 @@ tursca_status solve_render(tursca_scene *sc, double rtol, int max_iter, tursca_s
     *done = false;
     const SolveIO<T> io = forward_io<T>(sc);
     bool launched = false, solved = false;
+    const L2Window l2w(sc, io.val, (size_t)sc->G.nval * sizeof(T));
     const int ps = prof_begin(sc, P_SOLVE);
     tursca_status e = persist_launch<T>(sc, io, rtol, max_iter, &launched);
     prof_end(sc, ps, launched ? 1 : 0);
