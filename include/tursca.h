@@ -506,11 +506,14 @@ typedef struct {
  * request:
  *   TURSCA_SERVER_BATCH_SOLVES: 0 (default) runs every request's solve on
  *     its own stream; 1 batches the solves of the requests that run at the
- *     same time: the solves that wait while a launch runs (and for up to a
- *     millisecond, when a solve would run alone) are launched together in one persistent kernel, side by side, each on its own blocks
+ *     same time: the solves that wait while a launch runs, or up to 0.2 ms
+ *     for one whose request is running and that fits beside them, are launched
+ *     together in one persistent kernel, side by side, each on its own blocks
  *     with its own barrier (every wait bounded) and its own convergence, so a
  *     result does not depend on what it ran beside.  FP32 + refinement scenes
- *     whose solve takes at most three quarters of the GPU's blocks. */
+ *     small enough for another solve beside them: at most three quarters of
+ *     the GPU's SMs at one group of 128 rows each (16 x 16 x 16; larger ones
+ *     run on their own streams). */
 enum { TURSCA_SERVER_BATCH_SOLVES = 1 };
 tursca_status tursca_server_configure(tursca_server *srv, int option, double value);
 

@@ -9,6 +9,7 @@
 #include <cstring>
 #include <string>
 #include <functional>
+#include <utility>
 #include <vector>
 
 #include "graph.h"
@@ -182,6 +183,7 @@ struct tursca_scene {
     // the serving loop's batcher of solves (null: own launches)
     tk::SolveBatcher *batcher = nullptr;
     cudaEvent_t bready = nullptr, bdone = nullptr;
+    int bcoming = 0;  // the batcher expects this scene's solve, of so many blocks (0: it does not)
     unsigned long long *topk_keys = nullptr;
     unsigned int *topk_hist = nullptr, *topk_hist_h = nullptr;
     int *topk_band = nullptr, *topk_cnt = nullptr;  // chains in the FP32 band, [2] listed / above
@@ -1016,7 +1018,7 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     bool launched = false;
     if (sc->batcher && sizeof(T) == 4) {  // in a server: launched together with other requests' solves
         CK(cudaEventRecord(sc->bready, sc->st), "batch event");
-        if (tk::batcher_run(sc->batcher, J, P.smem, sc->bready, sc->bdone)) {
+        if (tk::batcher_run(sc->batcher, J, P.smem, sc->bready, sc->bdone, std::exchange(sc->bcoming, 0))) {
             CK(cudaStreamWaitEvent(sc->st, sc->bdone, 0), "batch wait");
             launched = true;
         }
@@ -3155,5 +3157,8 @@ void scene_attach_batcher(tursca_scene *sc, SolveBatcher *b) {
     }
     sc->batcher = b;
 }
+
+void scene_expected(tursca_scene *sc, int blocks) { sc->bcoming = blocks; }
+int scene_expected_end(tursca_scene *sc) { return std::exchange(sc->bcoming, 0); }
 }  // namespace tk
 

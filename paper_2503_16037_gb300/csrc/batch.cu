@@ -4,10 +4,11 @@
 // Protocol.  A scene's solve records `ready` on its stream, hands the job
 // over and blocks until the job is launched.  The thread waits for the
 // previous launch to finish (the jobs that arrive meanwhile form the next
-// one), and up to kBatchGatherUs for a second job, takes the waiting jobs of the oldest one's kind (warps per group) in
-// order while their blocks fit the GPU side by side, makes its stream wait for every job's `ready`, launches them in one
-// cooperative kernel, records every job's `done` and lets their callers go
-// on: each makes its own stream wait for its `done`.
+// one) and, while a request that can join the oldest job is on its way to its
+// solve, up to kBatchGatherUs for it; takes the waiting jobs in order while
+// their blocks fit the GPU side by side, makes its stream wait for every job's
+// `ready`, launches them in one cooperative kernel, records every job's `done`
+// and lets their callers go on: each makes its own stream wait for its `done`.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,12 +38,14 @@ class SolveBatcher {
         bool launched = false, ok = false;
     };
     std::deque<Pending *> q;
+    std::vector<int> coming;  // blocks of the solves that are on their way
     std::thread th;
     bool stop = false;
     long long batches = 0, jobs = 0;
     int max_jobs = 0;
 
     void loop();
+    void arrived(int nb);  // a solve that was on its way is not any more
 };
 
 void SolveBatcher::loop() {
@@ -54,17 +57,20 @@ void SolveBatcher::loop() {
         lk.unlock();
         bool ok = cudaEventSynchronize(last) == cudaSuccess;
         lk.lock();
-        // a solve alone waits a moment for one that fits beside it
+        // company for the oldest job: here, or on its way
         cv.wait_for(lk, std::chrono::microseconds(kBatchGatherUs), [&] {
+            const int room = nsm - q[0]->job->nb;
             for (size_t i = 1; i < q.size(); ++i)
-                if (q[i]->job->wpg == q[0]->job->wpg && q[0]->job->nb + q[i]->job->nb <= nsm) return true;
-            return stop;
+                if (q[i]->job->nb <= room) return true;
+            for (int nb : coming)
+                if (nb <= room) return stop;
+            return true;
         });
         std::vector<Pending *> take;
         int blocks = 0;
         size_t smem = 0;
         for (auto it = q.begin(); it != q.end() && (int)take.size() < kPsMaxJobs;) {
-            if (blocks + (*it)->job->nb <= nsm && (take.empty() || (*it)->job->wpg == take[0]->job->wpg)) {
+            if (blocks + (*it)->job->nb <= nsm) {
                 blocks += (*it)->job->nb;
                 smem = std::max(smem, (*it)->smem);
                 take.push_back(*it);
@@ -131,8 +137,34 @@ void batcher_destroy(SolveBatcher *b) {
     delete b;
 }
 
-bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done) {
-    if (!b || job.nb > kBatchShare * b->nsm) return false;
+int batcher_expect(SolveBatcher *b, const tursca_grid_desc &d) {
+    // (a plan with one group per block has as many blocks as the grid has groups)
+    const long long ng = ((long long)d.nx * d.ny + kPsRows - 1) / kPsRows * (d.nz + 1);
+    if (!b || d.precision == TURSCA_FP64 || ng > b->nsm || !batch_can_pair(1, (int)ng, b->nsm)) return 0;
+    std::lock_guard<std::mutex> lk(b->mu);
+    b->coming.push_back((int)ng);
+    return (int)ng;
+}
+
+void SolveBatcher::arrived(int nb) {
+    if (nb <= 0) return;
+    const auto it = std::find(coming.begin(), coming.end(), nb);
+    if (it != coming.end()) coming.erase(it);
+    cv.notify_all();
+}
+
+void batcher_expect_end(SolveBatcher *b, int nb) {
+    if (!b || nb <= 0) return;
+    std::lock_guard<std::mutex> lk(b->mu);
+    b->arrived(nb);
+}
+
+bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
+                 int expected) {
+    if (!b || !batch_can_pair(job.nl, job.nb, b->nsm)) {
+        batcher_expect_end(b, expected);
+        return false;
+    }
     SolveBatcher::Pending p;
     p.job = &job;
     p.smem = smem;
@@ -141,6 +173,7 @@ bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t rea
     std::unique_lock<std::mutex> lk(b->mu);
     if (b->stop) return false;
     b->q.push_back(&p);
+    b->arrived(expected);
     b->cv.notify_all();
     b->cv_launched.wait(lk, [&] { return p.launched; });
     return p.ok;

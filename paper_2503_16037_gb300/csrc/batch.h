@@ -15,16 +15,28 @@
 
 namespace tk {
 
-// A solve is batched when its plan leaves room for another one beside it:
-// at most this share of the GPU's blocks.
+// A solve is batched when another one can run beside it: its plan has one
+// group per block and takes at most this share of the GPU's blocks.  With two
+// or more groups per block a plan takes more than half of them (ps_plan takes
+// as few blocks as its largest share allows), and its groups are divided
+// among the warps differently, so nothing that is batched fits beside it.
 constexpr double kBatchShare = 0.75;
-// How long a solve that is alone waits for one that fits beside it.
-constexpr int kBatchGatherUs = 1000;
+inline bool batch_can_pair(int nl, int nb, int nsm) { return nl == 1 && nb <= kBatchShare * nsm; }
+
+// How long a solve waits for one that can run beside it and whose request is
+// on its way (from its start it takes the host about 150 us to hand over its
+// solve).  The wait lies inside the time that the solve's own assembly takes
+// on the GPU; 1,024 mixed requests on eight workers, the 16 x 16 x 16 ones'
+// median service: 1.2 to 1.6 ms with it and without batching alike (2.2 ms
+// with 1 ms waited whether company could come or not).
+constexpr int kBatchGatherUs = 200;
 
 // Hand one solve to the batcher and block until its batch has been launched:
 // the batch waits for `ready` (recorded on the scene's stream once the job's
 // inputs are there) and records `done` when it has finished.  False (nothing
 // launched) when the job cannot be batched; the caller then runs it itself.
-bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done);
+// expected: what batcher_expect returned for it (it is expected no longer).
+bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
+                 int expected = 0);
 
 }  // namespace tk

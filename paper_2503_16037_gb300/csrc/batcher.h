@@ -19,4 +19,14 @@ void batcher_stats(SolveBatcher *b, long long *batches, long long *jobs, int *ma
 // refinement scenes only.
 void scene_attach_batcher(tursca_scene *sc, SolveBatcher *b);
 
+// A request for this grid has been taken up, and other solves may wait a
+// moment for its solve: the blocks it will take (0: it will not be batched).
+// It stops being expected when its scene (scene_expected) hands the solve over
+// or batcher_expect_end is called.
+int batcher_expect(SolveBatcher *b, const tursca_grid_desc &d);
+void batcher_expect_end(SolveBatcher *b, int blocks);
+void scene_expected(tursca_scene *sc, int blocks);
+// what is left of it after the request: the blocks still expected
+int scene_expected_end(tursca_scene *sc);
+
 }  // namespace tk

@@ -80,7 +80,7 @@ struct tursca_server {
     int evictions = 0, built = 0, reserving = 0;
     bool stop = false;
     bool batch_solves = false;          // TURSCA_SERVER_BATCH_SOLVES
-    tk::SolveBatcher *batcher = nullptr;  // created with the first FP32 slot
+    tk::SolveBatcher *batcher = nullptr;  // created with the first FP32 request
     Clock::time_point t0 = Clock::now();
 
     double now_ms() const { return std::chrono::duration<double, std::milli>(Clock::now() - t0).count(); }
@@ -194,6 +194,7 @@ void run_request(tursca_server *srv, Request *r, Slot *slot) {
     tursca_solve_info si;
     std::memset(&si, 0, sizeof(si));
     if (!e) e = tursca_solve(sc, r->rtol, 5000, &si);
+    tk::batcher_expect_end(srv->batcher, tk::scene_expected_end(sc));
     if (!e) e = tursca_render_radiance(sc, r->radiance, nullptr);
     r->info.iters = si.iters;
     r->info.rel_resid64 = si.rel_resid64;
@@ -224,6 +225,11 @@ void worker(tursca_server *srv) {
             srv->cv_done.notify_all();
             continue;
         }
+        int expected = 0;  // blocks of a solve that others may wait for
+        if (srv->batch_solves && r->desc.precision == TURSCA_FP32_REFINE) {
+            if (!srv->batcher) srv->batcher = tk::batcher_create();
+            expected = tk::batcher_expect(srv->batcher, r->desc);
+        }
         if (build) {
             // a new slot, built outside the lock
             lk.unlock();
@@ -235,11 +241,10 @@ void worker(tursca_server *srv) {
             if (!e) e = tursca_scene_create(&r->desc, s->st, &s->sc);
             if (!e) e = tursca_build_graph(s->sc);
             lk.lock();
-            if (!e && srv->batch_solves && r->desc.precision == TURSCA_FP32_REFINE) {
-                if (!srv->batcher) srv->batcher = tk::batcher_create();
+            if (!e && srv->batch_solves && r->desc.precision == TURSCA_FP32_REFINE)
                 tk::scene_attach_batcher(s->sc, srv->batcher);  // a null batcher leaves the scene's own passes
-            }
             if (e) {
+                tk::batcher_expect_end(srv->batcher, expected);
                 if (s->sc) tursca_scene_destroy(s->sc);
                 if (s->st) cudaStreamDestroy(s->st);
                 srv->used -= reserve;
@@ -258,6 +263,7 @@ void worker(tursca_server *srv) {
             srv->built++;
         }
         r->info.slot_reused = build ? 0 : 1;
+        tk::scene_expected(slot->sc, expected);
         lk.unlock();
         run_request(srv, r, slot);
         const size_t real = tursca_scene_device_bytes(slot->sc);
