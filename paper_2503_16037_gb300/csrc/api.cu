@@ -1018,7 +1018,10 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     bool launched = false;
     if (sc->batcher && sizeof(T) == 4) {  // in a server: launched together with other requests' solves
         CK(cudaEventRecord(sc->bready, sc->st), "batch event");
-        if (tk::batcher_run(sc->batcher, J, P.smem, sc->bready, sc->bdone, std::exchange(sc->bcoming, 0))) {
+        const tk::BatchResult r =
+            tk::batcher_run(sc->batcher, J, P.smem, sc->bready, sc->bdone, std::exchange(sc->bcoming, 0));
+        if (r == tk::BATCH_FAILED) return fail(sc, TURSCA_E_CUDA, "a batched solve could not be waited for");
+        if (r == tk::BATCH_LAUNCHED) {
             CK(cudaStreamWaitEvent(sc->st, sc->bdone, 0), "batch wait");
             launched = true;
         }

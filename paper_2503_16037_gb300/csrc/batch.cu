@@ -35,7 +35,8 @@ class SolveBatcher {
         const PsJob *job;
         size_t smem;
         cudaEvent_t ready, done;
-        bool launched = false, ok = false;
+        bool launched = false;
+        BatchResult result = BATCH_NOT_LAUNCHED;
     };
     std::deque<Pending *> q;
     std::vector<int> coming;  // blocks of the solves that are on their way
@@ -90,18 +91,28 @@ void SolveBatcher::loop() {
         const int n = (int)take.size();
         for (Pending *p : take) ok = ok && cudaStreamWaitEvent(st, p->ready, 0) == cudaSuccess;
         ok = ok && launch_persist(st, h.data(), n, blocks, smem, false) == cudaSuccess;
-        for (Pending *p : take) ok = ok && cudaEventRecord(p->done, st) == cudaSuccess;
-        ok = ok && cudaEventRecord(last, st) == cudaSuccess;
         if (!ok) cudaGetLastError();  // a launch error stays with this thread: the callers run their own launches
-        lk.lock();
+        BatchResult result = ok ? BATCH_LAUNCHED : BATCH_NOT_LAUNCHED;
         if (ok) {
+            // From here on the solves run: a caller that was told otherwise
+            // would run a second one on the same vectors and barrier word.
+            // Where an event cannot be recorded, the launch is waited for here.
+            for (Pending *p : take) ok = cudaEventRecord(p->done, st) == cudaSuccess && ok;
+            ok = cudaEventRecord(last, st) == cudaSuccess && ok;
+            if (!ok) {
+                cudaGetLastError();
+                if (cudaStreamSynchronize(st) != cudaSuccess) result = BATCH_FAILED;
+            }
+        }
+        lk.lock();
+        if (result == BATCH_LAUNCHED) {
             batches++;
             jobs += n;
             max_jobs = std::max(max_jobs, n);
         }
         for (Pending *p : take) {
             p->launched = true;
-            p->ok = ok;
+            p->result = result;
         }
         cv_launched.notify_all();
     }
@@ -159,11 +170,11 @@ void batcher_expect_end(SolveBatcher *b, int nb) {
     b->arrived(nb);
 }
 
-bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
-                 int expected) {
+BatchResult batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
+                        int expected) {
     if (!b || !batch_can_pair(job.nl, job.nb, b->nsm)) {
         batcher_expect_end(b, expected);
-        return false;
+        return BATCH_NOT_LAUNCHED;
     }
     SolveBatcher::Pending p;
     p.job = &job;
@@ -171,12 +182,12 @@ bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t rea
     p.ready = ready;
     p.done = done;
     std::unique_lock<std::mutex> lk(b->mu);
-    if (b->stop) return false;
+    if (b->stop) return BATCH_NOT_LAUNCHED;
     b->q.push_back(&p);
     b->arrived(expected);
     b->cv.notify_all();
     b->cv_launched.wait(lk, [&] { return p.launched; });
-    return p.ok;
+    return p.result;
 }
 
 void batcher_stats(SolveBatcher *b, long long *batches, long long *jobs, int *max_jobs) {

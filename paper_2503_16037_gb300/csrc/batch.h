@@ -33,10 +33,13 @@ constexpr int kBatchGatherUs = 200;
 
 // Hand one solve to the batcher and block until its batch has been launched:
 // the batch waits for `ready` (recorded on the scene's stream once the job's
-// inputs are there) and records `done` when it has finished.  False (nothing
-// launched) when the job cannot be batched; the caller then runs it itself.
+// inputs are there) and records `done` when it has finished (or has finished
+// by then).  Not launched: the job cannot be batched, or its launch was
+// refused; the caller runs it itself.  Failed: it was launched and its end is
+// unknown (a CUDA error).
 // expected: what batcher_expect returned for it (it is expected no longer).
-bool batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
-                 int expected = 0);
+enum BatchResult { BATCH_NOT_LAUNCHED = 0, BATCH_LAUNCHED = 1, BATCH_FAILED = 2 };
+BatchResult batcher_run(SolveBatcher *b, const PsJob &job, size_t smem, cudaEvent_t ready, cudaEvent_t done,
+                        int expected = 0);
 
 }  // namespace tk

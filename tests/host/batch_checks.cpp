@@ -1,6 +1,7 @@
 // Host checks of the batcher of solves (batch.cu) against a stand-in for the
 // CUDA runtime and for the launch: which solves it takes, that a solve alone does
-// not wait, and that one waits a moment for company that is on its way.
+// not wait, that one waits a moment for company that is on its way, and what
+// happens when an event cannot be recorded.
 // Built and run by tests/test_host_batcher.py; returns the number of failures.
 #include <cuda_runtime.h>
 
@@ -18,7 +19,8 @@
 namespace {
 constexpr int kSms = 152;
 int failures = 0;
-std::atomic<int> last_jobs{0};
+std::atomic<int> last_jobs{0}, launches{0}, record_fails{0}, syncs_after_launch{0};
+std::atomic<bool> launch_pending{false}, sync_fails{false};
 void check(bool ok, const char *what) {
     std::printf("%s: %s\n", ok ? "ok" : "FAIL", what);
     failures += !ok;
@@ -31,17 +33,26 @@ cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = kSms, cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = (cudaStream_t)1, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    if (launch_pending) ++syncs_after_launch;
+    launch_pending = false;
+    return sync_fails ? cudaErrorUnknown : cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)1, cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) {
+    if (record_fails > 0) return --record_fails, cudaErrorMemoryAllocation;
+    return cudaSuccess;
+}
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 
 namespace tk {
 cudaError_t launch_persist(cudaStream_t, const PsJob *, int njobs, int, size_t, bool) {
     last_jobs = njobs;
+    ++launches;
+    launch_pending = true;
     return cudaSuccess;
 }
 }  // namespace tk
@@ -133,6 +144,21 @@ int main() {
     d.nx = d.ny = 32;  // two groups per block: nothing fits beside it
     d.nz = 24;
     check(tk::batcher_expect(b, d) == 0, "no one waits for a solve that is not batched");
+    // an event that cannot be recorded behind a launch: the caller must not
+    // launch its own solve beside the one that runs
+    for (int at = 1; at <= 2; ++at) {
+        launches = syncs_after_launch = 0;
+        launch_pending = false;
+        record_fails = at;
+        const int r = (int)tk::batcher_run(b, J, 0, nullptr, nullptr);
+        check(launches == 1 && r != 0, "a solve that was launched is not reported as not launched");
+        check(syncs_after_launch == 1, "its launch has ended before the caller goes on");
+        record_fails = 0;
+    }
+    record_fails = 1;
+    sync_fails = true;
+    check((int)tk::batcher_run(b, J, 0, nullptr, nullptr) == 2, "one whose end is unknown is a failure");
+    sync_fails = false;
     tk::batcher_destroy(b);
     return failures;
 }
