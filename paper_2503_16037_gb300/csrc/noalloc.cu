@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 #include <type_traits>
 
 #include "tursca.h"
@@ -102,8 +103,7 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
 }
 
 // ---------------------------------------------------------------------------
-// The whole solve in one cooperative launch, for systems whose matrix stays
-// in L2.
+// The whole solve in one cooperative launch.
 //
 // What bounds a sweep of one launch each (k_na_sweep) is the gather of v: 32
 // unrelated addresses per warp load, 24 us for 6.1M entries (65,536 rows of a
@@ -112,20 +112,46 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
 // the window of v that its rows reach (columns modulo n, so a band that wraps
 // around is one window) and as many of its entries as fit beside it, as 4-byte
 // values and 2-byte window indices; the other entries come from L2, where
-// they stay because a line is only ever read by one SM.  Blocks exchange v
-// through global memory with one grid barrier per sweep.  A block whose rows
-// reach too far for a window gathers from global memory.
+// they stay because a line is only ever read by one SM (what L2 cannot hold
+// comes from HBM).  Blocks exchange v through global memory with one grid
+// barrier per sweep.  A block whose rows reach too far for a window keeps as
+// much of it as shared memory holds and gathers the rest from global memory;
+// with all gathers from there 100,000 rows of 62 to 124 entries in any column
+// took 6,600 us, now 4,010 (a launch per sweep, whose L1 holds more of v: 3,500).
 //
 // Kept rows are packed to whole quads (zero padding), so a lane takes four
 // entries per step with two loads of values and indices; 8 lanes (32 where
 // rows average more than 256 entries) share a row.  80 sweeps over the 65,536
 // rows: 2010 us with a launch per sweep, 1159 us in one launch entry by entry
-// (a warp per row, bound by its 47 instructions per 32 entries), 1085 us as
-// here.
+// (a warp per row, bound by its 47 instructions per 32 entries), 1085 us packed,
+// 1045 us as here (streamed rows read in whole 32-byte sectors).
+//
+// The line at kNsMaxNodes is one on rows because the number of entries is not
+// known to the host.  Both sides, 80 sweeps, one launch against a launch per
+// sweep, us: 2,000 rows of 10 to 20 entries 218 / 380; 131,072 of 62 to 124
+// 1,807 / 3,930; 131,072 of 150 to 300 (236 MB) 5,580 / 5,780; 65,536 of 500 to
+// 1,000 (393 MB) 7,360 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
+// either way, and static shares end unevenly) 14,510 / 13,380.
 constexpr int kNsThreads = 1024, kNsWarps = kNsThreads / 32;
 constexpr int kNsMaxRows = 4096;     // rows a block may keep
-constexpr int kNsMaxNodes = 131072;  // above this the matrix no longer stays in L2: a launch per sweep
+constexpr int kNsMaxNodes = 131072;  // above this a launch per sweep
 constexpr long long kNsPolls = 1ll << 21;  // polls of one barrier: about 1.5 s
+
+// an entry's value or column, with an L2 policy or without
+template <bool POLICY, typename E>
+__device__ __forceinline__ E ns_ld(const E *p, unsigned long long policy) {
+    if constexpr (!POLICY) return __ldg(p);
+    unsigned v;
+    asm("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(policy));
+    E r;
+    memcpy(&r, &v, 4);
+    return r;
+}
+
+enum { NS_ALL = 0, NS_SOME = 1, NS_NONE = 2 };  // columns that a pass finds in shared memory
+
+constexpr int kNsL2Entries = 10000000;  // 80 MB, what L2 keeps of a set that is read over and over (65,536 rows of
+                                        // 500 to 1,000 entries: 7,760 us without the policies)
 
 struct NsArgs {
     int n, sweeps, refinements, smem;
@@ -186,6 +212,18 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     const bool win4 = W <= 32768;                         // v in shared memory
     const bool win8 = W <= 12288;                         // x too (FP64)
     const int wbytes = win4 ? ((win8 ? 8 : 4) * W + 15) / 16 * 16 : 0;
+    // columns of v in shared memory: all of them; or, beside no entries, as many
+    // as fit, around the block's own rows, where its entries gather often enough
+    // to pay for the copy (a 32-byte sector saved for every two of its elements)
+    int wv = W;
+    if (!win4) {
+        wv = ne > W / 2 ? min(W, (A.smem - 64) / 4) : 0;
+        if (W >= n) w0 = (r0 + r1) / 2 - wv / 2;
+        else w0 += (W - wv) / 2;
+        if (w0 < 0) w0 += n;
+        else if (w0 >= n) w0 -= n;
+    }
+    const int wx = win8 ? W : 0;  // and of x
     // rows kept, from the first on: packed row starts (in quads), values, indices
     const int capq = win4 ? (A.smem - wbytes - kNsMaxRows * 2 - 64) / 24 : 0;  // quads that fit
     float *win = (float *)ns_dyn;
@@ -238,6 +276,13 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
             ix[i] = (uint16_t)local(__ldg(A.col + p + min(i, len - 1)));
         }
     }
+    // Entries streamed beyond what L2 holds for all blocks leave it first, so
+    // that they do not push the others out.
+    unsigned long long near_by, pass_by;
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(near_by));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
+    const int streamed = r0 + kept < r1 ? __ldg(rp + r0 + kept) : e0 + ne;  // the first streamed entry
+    const int near_end = e0 + ne - streamed <= kNsL2Entries / nb * 11 / 10 ? 0x7fffffff : streamed + kNsL2Entries / nb;
     unsigned gen = 0;
     auto barrier = [&]() -> bool {
         ++gen;
@@ -259,38 +304,47 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         return sh_ok != 0;
     };
     // Every row's sum over its entries of val times the gathered vector (from
-    // the kept entries; else from L2 with the window, or from global memory),
+    // the kept entries; else from L2, with the window's `width` columns in
+    // shared memory and the others in global memory),
     // handed to out(row, sum) in one lane of the row's L lanes.  The rows that
     // are not kept go first: their loads take longest.
-    auto rows = [&](auto lanes_c, auto zero, const auto *vec, const auto *window, bool windowed, auto out) {
-        constexpr int L = decltype(lanes_c)::value;
+    auto rows = [&](auto lanes_c, auto mode_c, auto zero, const auto *vec, const auto *window, int width, auto out) {
+        constexpr int L = decltype(lanes_c)::value, MODE = decltype(mode_c)::value;
         using V = decltype(zero);
         const int sl = lane & (L - 1), first = tid / 32 * (32 / L) + lane / L, lanes = kNsThreads / L;
+        auto get = [&](int c) {
+            if constexpr (MODE == NS_NONE) return vec[c];
+            const int d = local(c);
+            if constexpr (MODE == NS_ALL) return window[d];
+            return d < width ? window[d] : vec[c];
+        };
         auto sum = [&](V acc, int row, bool on) {
             __syncwarp();
 #pragma unroll
             for (int o = L / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (sl == 0 && on) out(row, acc);
         };
-        const int k0 = windowed ? kept : 0;
+        const int k0 = MODE == NS_ALL ? kept : 0;
         for (int b = r0 + k0; b < r1; b += lanes) {
             const int row = b + first;
             const bool on = row < r1;
             const int p = on ? __ldg(rp + row) : 0, end = on ? __ldg(rp + row + 1) : 0;
             V acc = zero;
             constexpr int U = sizeof(V) == 4 ? 6 : 4;
-            for (int e = p + sl; e < end; e += U * L) {
+            // (a policy operand costs matrices that stay in L2 2 to 4 %: wide rows only)
+            const unsigned long long policy = p < near_end ? near_by : pass_by;
+            for (int e = (p & ~7) + sl; e < end; e += U * L) {  // the lanes' 8 or 32 entries in whole sectors
                 float v[U];
                 int c[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const bool in = e + u * L < end;
-                    v[u] = in ? __ldg(A.val + e + u * L) : 0.f;
-                    c[u] = in ? __ldg(A.col + e + u * L) : -1;
+                    const bool in = e + u * L < end && (u > 0 || e >= p);
+                    v[u] = in ? ns_ld<L == 32>(A.val + e + u * L, policy) : 0.f;
+                    c[u] = in ? ns_ld<L == 32>(A.col + e + u * L, policy) : -1;
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (c[u] >= 0) acc += (V)v[u] * (windowed ? window[local(c[u])] : vec[c[u]]);
+                    if (c[u] >= 0) acc += (V)v[u] * get(c[u]);
             }
             sum(acc, row, on);
         }
@@ -312,9 +366,15 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         }
     };
     const bool wide = (long long)rp[n] - rp[0] > 256ll * n;
-    auto all_rows = [&](auto zero, const auto *vec, const auto *window, bool windowed, auto out) {
-        if (wide) rows(std::integral_constant<int, 32>(), zero, vec, window, windowed, out);
-        else rows(std::integral_constant<int, 8>(), zero, vec, window, windowed, out);
+    auto all_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
+        auto go = [&](auto mode_c) {
+            if (wide) rows(std::integral_constant<int, 32>(), mode_c, zero, vec, window, width, out);
+            else rows(std::integral_constant<int, 8>(), mode_c, zero, vec, window, width, out);
+        };
+        if (width == W) return go(std::integral_constant<int, NS_ALL>());
+        if constexpr (sizeof(zero) == 4)
+            if (width > 0) return go(std::integral_constant<int, NS_SOME>());
+        go(std::integral_constant<int, NS_NONE>());
     };
     bool ok = true;
     for (int i = r0 + tid; i < r1; i += kNsThreads) {
@@ -326,15 +386,15 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         const float *cur = A.b;
         for (int k = 0; ok && k < A.sweeps; ++k) {
             float *nxt = (k & 1) ? A.d1 : A.d0;
-            if (win4) {
+            if (wv > 0) {
 #pragma unroll 8
-                for (int j = tid; j < W; j += kNsThreads) {
+                for (int j = tid; j < wv; j += kNsThreads) {
                     const int g = w0 + j;
                     win[j] = __ldcg(cur + (g >= n ? g - n : g));
                 }
                 __syncthreads();
             }
-            all_rows(0.f, cur, win, win4, [&](int row, float v) { nxt[row] = A.b[row] + v; });
+            all_rows(0.f, cur, win, wv, [&](int row, float v) { nxt[row] = A.b[row] + v; });
             cur = nxt;
             ok = barrier();
         }
@@ -351,7 +411,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
             __syncthreads();
         }
         double loc = 0.0;
-        all_rows(0.0, A.x, winx, win8, [&](int row, double v) {
+        all_rows(0.0, A.x, winx, wx, [&](int row, double v) {
             const double res = (double)A.s[row] - A.x[row] + v;
             A.b[row] = (float)res;
             loc += res * res;

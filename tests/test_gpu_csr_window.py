@@ -1,0 +1,84 @@
+"""tursca_csr_solve_noalloc where a block's rows reach more columns than it can
+keep: part of the window in shared memory, all of it beside no entries, none of
+it (too few entries to pay for the copy), and rows around the window's ends.
+
+Tolerance: that of test_gpu_csr_launch.py (rows of at most 2000 terms).
+"""
+import pytest
+
+from paper_2503_16037_gb300 import tursca as T
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+CASES = {  # rows, entries per row (0 .. 2 k), reach of the columns (0: anywhere)
+    "part": (100000, 93, 0),
+    "part_around_the_rows": (131072, 60, 40000),
+    "all_beside_no_entries": (50000, 100, 0),
+    "none": (131072, 6, 0),
+    "long_rows": (80000, 300, 0),
+    "smallest_part": (65537, 60, 0),
+}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2503_16037_gb300 import build
+    build.build()
+
+
+def system(n, k, reach):
+    g = torch.Generator(device="cuda").manual_seed(n + k)
+    length = torch.randint(0, 2 * k + 1, (n,), generator=g, device="cuda")
+    row_ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    row_ptr[1:] = length.cumsum(0)
+    nnz = int(row_ptr[-1])
+    rows = torch.repeat_interleave(torch.arange(n, device="cuda"), length)
+    if reach:
+        col = (rows + torch.randint(-reach, reach + 1, (nnz,), generator=g, device="cuda")) % n
+    else:
+        col = torch.randint(0, n, (nnz,), generator=g, device="cuda")
+    val = torch.rand(nnz, generator=g, device="cuda") * (0.5 / length.clamp(min=1)[rows]).float()
+    return row_ptr.int(), col.int(), val, torch.rand(n, generator=g, device="cuda"), rows
+
+
+def solve(sys_, n, sweeps, refinements):
+    x = torch.full((n,), float("nan"), dtype=torch.float64, device="cuda")
+    T.tursca_csr_solve_noalloc(sys_[0], sys_[1], sys_[2], n, sys_[3], x, sweeps, refinements, None,
+                               torch.cuda.current_stream().cuda_stream)
+    return x
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_wide_windows(name):
+    n = CASES[name][0]
+    s = system(*CASES[name])
+    x = solve(s, n, 24, 5)
+    ref = s[3].double()
+    for _ in range(60):
+        ref = s[3].double().index_add(0, s[4], s[2].double() * ref[s[1].long()])
+    # 2000 terms 4e-13; FP64 atomics in the reference stay inside the same bound
+    assert float((x - ref).abs().max()) <= 4e-13 * float(ref.abs().max())
+
+
+def test_gathers_from_anywhere_cost_no_more_than_a_launch_per_sweep():
+    """100,000 rows in one launch against 131,073 rows with as many entries,
+    which take a launch per sweep: at most 1.3 times (1.5 with every gather in
+    global memory)."""
+    def ms(n, k):
+        s = system(n, k, 0)
+        solve(s, n, 20, 2)
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            solve(s, n, 20, 2)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best / s[1].numel()
+
+    one, per_sweep = ms(100000, 93), ms(131073, 71)
+    print("per entry, 40 sweeps: one launch %.3g ns, a launch per sweep %.3g ns" % (1e6 * one, 1e6 * per_sweep))
+    assert one <= 1.3 * per_sweep
