@@ -120,22 +120,32 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
 // took 6,600 us, now 4,010 (a launch per sweep, whose L1 holds more of v: 3,500).
 //
 // Kept rows are packed to whole quads (zero padding), so a lane takes four
-// entries per step with two loads of values and indices; 8 lanes (32 where
-// rows average more than 256 entries) share a row.  80 sweeps over the 65,536
+// entries per step with two loads of values and indices; 8 lanes (32 in blocks
+// whose rows average more than 256 entries) share a row.  80 sweeps over the 65,536
 // rows: 2010 us with a launch per sweep, 1159 us in one launch entry by entry
 // (a warp per row, bound by its 47 instructions per 32 entries), 1085 us packed,
 // 1045 us as here (streamed rows read in whole 32-byte sectors).
 //
 // The line at kNsMaxNodes is one on rows because the number of entries is not
 // known to the host.  Both sides, 80 sweeps, one launch against a launch per
-// sweep, us: 2,000 rows of 10 to 20 entries 218 / 380; 131,072 of 62 to 124
-// 1,807 / 3,930; 131,072 of 150 to 300 (236 MB) 5,580 / 5,780; 65,536 of 500 to
-// 1,000 (393 MB) 7,360 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
-// either way, and static shares end unevenly) 14,510 / 13,380.
+// sweep, us: 2,000 rows of 10 to 20 entries 222 / 380; 131,072 of 62 to 124
+// 1,815 / 3,930; 131,072 of 150 to 300 (236 MB) 5,650 / 5,780; 65,536 of 500 to
+// 1,000 (393 MB) 7,430 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
+// either way, and static shares end unevenly) 14,620 / 13,380.
 constexpr int kNsThreads = 1024, kNsWarps = kNsThreads / 32;
 constexpr int kNsMaxRows = 4096;     // rows a block may keep
 constexpr int kNsMaxNodes = 131072;  // above this a launch per sweep
 constexpr long long kNsPolls = 1ll << 21;  // polls of one barrier: about 1.5 s
+// A row longer than kNsLong entries (kNsLongWide in blocks whose rows average
+// more than 256) is cut into chunks of that many, which the block's warps share
+// and whose sums one thread adds in order; left to the lanes that share a
+// common row it would hold up the whole grid: 65,536 rows of 40 to 80 entries
+// and one of 65,536 took 60.5 ms (80 sweeps; a launch per sweep, a warp per row:
+// 11.0 ms), with chunks 1.8 ms; 16 of 20,000 19.5 ms (4.7), with chunks 1.3 ms.
+constexpr int kNsLong = 512, kNsLongWide = 4096;
+constexpr int kNsLongKept = 2048;  // from shared memory the lanes of a common row are quick enough up to here
+constexpr int kNsChunks = 256;  // most chunks of a block (longer chunks where they would not do)
+constexpr unsigned kNsIsLong = 0x8000u;  // flag of a row in the packed row starts
 
 // an entry's value or column, with an L2 policy or without
 template <bool POLICY, typename E>
@@ -164,8 +174,9 @@ struct NsArgs {
 
 __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constant__ NsArgs A) {
     extern __shared__ __align__(16) unsigned char ns_dyn[];
-    __shared__ int sh_r[2], sh_min[kNsWarps], sh_max[kNsWarps], sh_ok;
-    __shared__ double sh_red[kNsWarps];
+    __shared__ int sh_r[2], sh_min[kNsWarps], sh_max[kNsWarps], sh_ok, sh_nch;
+    __shared__ int sh_crow[kNsChunks], sh_cst[kNsChunks];  // per chunk: its row and first entry
+    __shared__ double sh_csum[kNsChunks], sh_red[kNsWarps];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, n = A.n, nb = gridDim.x, blk = blockIdx.x;
     const int32_t *__restrict__ rp = A.row_ptr;
     // rows [r0, r1): equal shares of entries, a row counted as 16 more
@@ -226,7 +237,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     }
     const int wx = win8 ? W : 0;  // and of x
     // rows kept, from the first on: packed row starts (in quads), values, indices
-    const int capq = win4 ? (A.smem - wbytes - kNsMaxRows * 2 - 64) / 24 : 0;  // quads that fit
+    const int capq = win4 ? (A.smem - wbytes - min(r1 - r0 + 1, kNsMaxRows) * 2 - 64) / 24 : 0;  // quads that fit
     float *win = (float *)ns_dyn;
     double *winx = (double *)ns_dyn;
     float4 *sval = (float4 *)(ns_dyn + wbytes);
@@ -237,13 +248,30 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         d += d < 0 ? n : 0;
         return d;
     };
-    int kept = 0;  // rows [r0, r0 + kept)
+    const bool wide = ne > 256ll * (r1 - r0);
+    // long rows: more than `chunk` entries streamed, more than klong kept; the
+    // chunk that lets the block list all of its chunks
+    int chunk = wide ? kNsLongWide : kNsLong;
+    for (;; chunk *= 2) {
+        __syncthreads();
+        if (tid == 0) sh_nch = 0;
+        __syncthreads();
+        for (int r = r0 + tid; r < r1; r += kNsThreads) {
+            const int len = __ldg(rp + r + 1) - __ldg(rp + r);
+            if (len > chunk) atomicAdd(&sh_nch, (len - 1) / chunk + 1);
+        }
+        __syncthreads();
+        if (sh_nch <= kNsChunks) break;
+    }
+    const int klong = max(chunk, kNsLongKept);
+    int kept = 0;  // rows [r0, r0 + kept), the long ones among them left out
     if (capq > 0) {
         int carry = 0;
         const int most = min(r1 - r0, kNsMaxRows - 1);
         for (int base = 0; base < most; base += kNsThreads) {
             const int r = base + tid;
-            const int q = r < most ? (__ldg(rp + r0 + r + 1) - __ldg(rp + r0 + r) + 3) / 4 : 0;
+            const int len = r < most ? __ldg(rp + r0 + r + 1) - __ldg(rp + r0 + r) : 0;
+            const int q = len > klong ? 0 : (len + 3) / 4;
             int v = q;  // inclusive scan over the block
             for (int o = 1; o < 32; o <<= 1) {
                 const int u = __shfl_up_sync(0xffffffffu, v, o);
@@ -259,7 +287,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
             }
             v += before;
             const bool fits = r < most && v <= capq;
-            if (fits) srow[r + 1] = (uint16_t)v;
+            if (fits) srow[r + 1] = (uint16_t)(v | (len > klong ? kNsIsLong : 0u));
             if (r == 0) srow[0] = 0;
             const int nf = __syncthreads_count(fits);  // a prefix of the rows: v never falls
             kept = base + nf;
@@ -269,7 +297,8 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     }
     __syncthreads();
     for (int r = tid / 8; r < kept; r += kNsThreads / 8) {
-        const int p = __ldg(rp + r0 + r), len = __ldg(rp + r0 + r + 1) - p, q0 = srow[r];
+        const int p = __ldg(rp + r0 + r), len = __ldg(rp + r0 + r + 1) - p, q0 = srow[r] & (kNsIsLong - 1);
+        if (len > klong) continue;
         float *v = (float *)(sval + q0);
         uint16_t *ix = (uint16_t *)(sidx + q0);
         for (int i = tid % 8; i < (len + 3) / 4 * 4; i += 8) {
@@ -277,6 +306,21 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
             ix[i] = (uint16_t)local(__ldg(A.col + p + min(i, len - 1)));
         }
     }
+    // the list of the long rows' chunks (no more than were counted: klong >= chunk)
+    auto longest = [&](int row) { return row < r0 + kept ? klong : chunk; };
+    if (tid == 0) sh_nch = 0;
+    __syncthreads();
+    for (int r = r0 + tid; r < r1; r += kNsThreads) {
+        const int p = __ldg(rp + r), len = __ldg(rp + r + 1) - p;
+        if (len <= longest(r)) continue;
+        const int nc = (len - 1) / chunk + 1, c0 = atomicAdd(&sh_nch, nc);
+        for (int c = 0; c < nc; ++c) {
+            sh_crow[c0 + c] = r;
+            sh_cst[c0 + c] = p + c * chunk;
+        }
+    }
+    __syncthreads();
+    const int nch = sh_nch;
     // Entries streamed beyond what L2 holds for all blocks leave it first, so
     // that they do not push the others out.
     unsigned long long near_by, pass_by;
@@ -308,7 +352,8 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     // the kept entries; else from L2, with the window's `width` columns in
     // shared memory and the others in global memory),
     // handed to out(row, sum) in one lane of the row's L lanes.  The rows that
-    // are not kept go first: their loads take longest.
+    // are not kept go first: their loads take longest.  Long rows are skipped
+    // (long_rows).
     auto rows = [&](auto lanes_c, auto mode_c, auto zero, const auto *vec, const auto *window, int width, auto out) {
         constexpr int L = decltype(lanes_c)::value, MODE = decltype(mode_c)::value;
         using V = decltype(zero);
@@ -328,8 +373,13 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         const int k0 = MODE == NS_ALL ? kept : 0;
         for (int b = r0 + k0; b < r1; b += lanes) {
             const int row = b + first;
-            const bool on = row < r1;
-            const int p = on ? __ldg(rp + row) : 0, end = on ? __ldg(rp + row + 1) : 0;
+            int p = 0, end = 0;
+            if (row < r1) {
+                p = __ldg(rp + row);
+                end = __ldg(rp + row + 1);
+            }
+            const bool on = row < r1 && end - p <= (MODE == NS_ALL ? chunk : longest(row));
+            if (!on) end = p;
             V acc = zero;
             constexpr int U = sizeof(V) == 4 ? 6 : 4;
             // (a policy operand costs matrices that stay in L2 2 to 4 %: wide rows only)
@@ -351,8 +401,9 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         }
         for (int b = 0; b < k0; b += lanes) {
             const int r = b + first;
-            const bool on = r < k0;
-            const int q0 = on ? srow[r] : 0, q1 = on ? srow[r + 1] : 0;
+            const unsigned s0 = r < k0 ? srow[r] : 0u, s1 = r < k0 ? srow[r + 1] : kNsIsLong;
+            const bool on = !(s1 & kNsIsLong);
+            const int q0 = s0 & (kNsIsLong - 1), q1 = on ? s1 : q0;
             V acc = zero;
 #pragma unroll 2
             for (int q = q0 + sl; q < q1; q += L) {
@@ -366,8 +417,31 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
             sum(acc, r0 + r, on);
         }
     };
-    const bool wide = (long long)rp[n] - rp[0] > 256ll * n;
+    auto long_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
+        using V = decltype(zero);
+        for (int c = w; c < nch; c += kNsWarps) {
+            const int p = sh_cst[c], re = __ldg(rp + sh_crow[c] + 1), end = re - p > chunk ? p + chunk : re;
+            V acc = zero;
+#pragma unroll 8
+            for (int e = p + lane; e < end; e += 32) {
+                const int k = __ldg(A.col + e), d = local(k);
+                acc += (V)__ldg(A.val + e) * (d < width ? window[d] : vec[k]);
+            }
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) sh_csum[c] = (double)acc;
+        }
+        __syncthreads();
+        for (int c = tid; c < nch; c += kNsThreads) {
+            const int row = sh_crow[c], p = __ldg(rp + row), len = __ldg(rp + row + 1) - p;
+            if (sh_cst[c] != p) continue;  // not the row's first
+            V t = zero;
+            for (int k = 0; k <= (len - 1) / chunk; ++k) t += (V)sh_csum[c + k];
+            out(row, t);
+        }
+        __syncthreads();  // sh_csum
+    };
     auto all_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
+        if (nch > 0) long_rows(zero, vec, window, width, out);
         auto go = [&](auto mode_c) {
             if (wide) rows(std::integral_constant<int, 32>(), mode_c, zero, vec, window, width, out);
             else rows(std::integral_constant<int, 8>(), mode_c, zero, vec, window, width, out);
@@ -450,7 +524,7 @@ bool one_launch(const NsArgs &a0, cudaStream_t st) {
         smem < 160 * 1024)
         return false;
     NsArgs a = a0;
-    a.smem = smem - 4 * 1024;  // beside the static shared memory
+    a.smem = smem - 6 * 1024;  // beside the static shared memory
     int nb = (a.n + kNsWarps - 1) / kNsWarps;
     if (nb > nsm) nb = nsm;
     if (nb > kPartBlocks) nb = kPartBlocks;
