@@ -119,17 +119,17 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
 // with all gathers from there 100,000 rows of 62 to 124 entries in any column
 // took 6,600 us, now 4,010 (a launch per sweep, whose L1 holds more of v: 3,500).
 //
-// Kept rows are packed to whole quads (zero padding), so a lane takes four
+// Kept rows are packed to whole quads (zeros that gather a zero), so a lane takes four
 // entries per step with two loads of values and indices; 8 lanes (32 in blocks
 // whose rows average more than 256 entries) share a row.  80 sweeps over the 65,536
 // rows: 2010 us with a launch per sweep, 1159 us in one launch entry by entry
 // (a warp per row, bound by its 47 instructions per 32 entries), 1085 us packed,
-// 1045 us as here (streamed rows read in whole 32-byte sectors).
+// 1065 us as here (streamed rows read in whole 32-byte sectors).
 //
 // The line at kNsMaxNodes is one on rows because the number of entries is not
 // known to the host.  Both sides, 80 sweeps, one launch against a launch per
 // sweep, us: 2,000 rows of 10 to 20 entries 222 / 380; 131,072 of 62 to 124
-// 1,815 / 3,930; 131,072 of 150 to 300 (236 MB) 5,650 / 5,780; 65,536 of 500 to
+// 1,840 / 3,930; 131,072 of 150 to 300 (236 MB) 5,650 / 5,780; 65,536 of 500 to
 // 1,000 (393 MB) 7,430 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
 // either way, and static shares end unevenly) 14,620 / 13,380.
 constexpr int kNsThreads = 1024, kNsWarps = kNsThreads / 32;
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     else if (w0 >= n) w0 -= n;
     const bool win4 = W <= 32768;                         // v in shared memory
     const bool win8 = W <= 12288;                         // x too (FP64)
-    const int wbytes = win4 ? ((win8 ? 8 : 4) * W + 15) / 16 * 16 : 0;
+    const int wbytes = win4 ? ((win8 ? 8 : 4) * (W + 1) + 15) / 16 * 16 : 0;  // and a 0, which padding gathers
     // columns of v in shared memory: all of them; or, beside no entries, as many
     // as fit, around the block's own rows, where its entries are enough to pay
     // for the copy (100,000 rows of 20 to 40 entries, 20 thousand a block, 2,277 us
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         uint16_t *ix = (uint16_t *)(sidx + q0);
         for (int i = tid % 8; i < (len + 3) / 4 * 4; i += 8) {
             v[i] = i < len ? __ldg(A.val + p + i) : 0.f;
-            ix[i] = (uint16_t)local(__ldg(A.col + p + min(i, len - 1)));
+            ix[i] = (uint16_t)(i < len ? local(__ldg(A.col + p + i)) : W);
         }
     }
     // the list of the long rows' chunks (no more than were counted: klong >= chunk)
@@ -457,7 +457,9 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         A.b[i] = A.s[i];
     }
     ok = barrier();
+    if (win8 && tid == 0) winx[W] = 0.0;
     for (int r = 0; ok && r < A.refinements; ++r) {
+        if (win4 && tid == 0) win[W] = 0.f;  // (where x's window lay meanwhile)
         const float *cur = A.b;
         for (int k = 0; ok && k < A.sweeps; ++k) {
             float *nxt = (k & 1) ? A.d1 : A.d0;
