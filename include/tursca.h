@@ -177,7 +177,9 @@ tursca_status tursca_assemble_flux(tursca_scene *scene, const tursca_geometry *g
  * iterations in the scene's precision.  Scenes with up to about 200 MB of
  * matrix values beyond shared memory (in FP32 up to about 3,000 groups of 128
  * rows at radius 2: 96 x 96 x 32) are solved in one cooperative launch, by
- * BiCGStab from the source to the refined solution.  Others run pass by pass:
+ * BiCGStab from the source to the refined solution (which starts once the GPU
+ * holds all of its blocks, so it waits for the end of a long-running kernel of
+ * another stream).  Others run pass by pass:
  * FP32_REFINE scenes first a few Neumann sweeps (the series of Eq. fs_sum) that
  * also estimate the largest eigenvalue of K, then Chebyshev iterations on the
  * interval that estimate implies, or BiCGStab (two products with K per step)
@@ -441,8 +443,10 @@ tursca_status tursca_quadrature(const tursca_grid_desc *desc, double *q_iso, dou
  * the caller's next synchronisation).
  * Up to 131,072 nodes the whole solve is one cooperative launch (blocks that
  * keep their rows in shared memory and meet a bounded grid barrier per sweep;
- * should a barrier give up, x and resid2 are NaN); larger systems take a
- * launch per sweep.
+ * should a barrier give up, as where two calls overlap, x and resid2 are NaN).
+ * Such a launch starts once the GPU holds all of its blocks, up to one per SM
+ * with all of its shared memory: behind a long-running kernel of another
+ * stream it waits for that one's end.  Larger systems take a launch per sweep.
  * The call allocates nothing and returns without synchronising. */
 tursca_status tursca_csr_solve_noalloc(const int32_t *row_ptr, const int32_t *col, const float *val, int n_nodes,
                                        const float *s, double *x, int sweeps, int refinements, double *resid2,
