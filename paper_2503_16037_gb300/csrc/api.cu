@@ -811,10 +811,9 @@ tursca_status gmres(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &gp, 
 
 // BiCGStab on (I - K) d = b, b = r64, to ||b - (I - K) d|| <= tol ||b|| (the
 // recursion's residual) in at most maxit steps, then x += d with the FP32
-// pair of x.  norm: ||r64||.  Steps are queued kBiChunk at a time, one chunk
-// ahead of the read-back of the state; the passes after the end return at
-// once.  *ok false: the iteration broke down and x is unchanged.
-constexpr int kBiChunk = 1;
+// pair of x.  norm: ||r64||.  One step is queued ahead of the read-back of the
+// state; its passes return at once when the step before was the last.  *ok
+// false: the iteration broke down and x is unchanged.
 template <typename T>
 tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &gp, const T *val, double norm,
                        double tol, int maxit, double *x, float *xh, float *xl, SolveState &ss, bool *ok) {
@@ -835,23 +834,21 @@ tursca_status bicgstab(tursca_scene *sc, const tk::GridC &g, const tk::GraphP &g
     const double bb = std::ldexp(norm, -ex) * std::ldexp(norm, -ex);
     tk::launch_bi_start<T>(sc->st, n, sc->r64, std::ldexp(1.0, -ex), bb, tol * tol * bb, b, r, p, d, st);
     sc->launches++;
-    const int chunks = std::max(1, (maxit + kBiChunk - 1) / kBiChunk);
     tk::BiState<T> *h = (tk::BiState<T> *)(sc->hred + 192);  // two read-back slots of 64 bytes
     static_assert(sizeof(tk::BiState<T>) <= 64, "read-back slots");
-    auto slot = [&](int c) { return (tk::BiState<T> *)((char *)h + (c & 1) * 64); };
-    for (int c = 0; c <= chunks; ++c) {
-        if (c < chunks) {
+    auto slot = [&](int k) { return (tk::BiState<T> *)((char *)h + (k & 1) * 64); };
+    for (int k = 0; k <= maxit; ++k) {
+        if (k < maxit) {
             const int pi = prof_begin(sc, P_GPROD);
-            for (int k = 0; k < kBiChunk; ++k)
-                tk::launch_bi_step<T>(sc->st, g, gp, val, b, r, p, v, t, d, sc->bi_part, st, &sc->launches);
-            prof_end(sc, pi, 2 * kBiChunk);
-            CK(cudaMemcpyAsync(slot(c), st, sizeof(*st), cudaMemcpyDeviceToHost, sc->st), "d2h");
-            CK(cudaEventRecord(sc->bi_ev[c & 1], sc->st), "event");
+            tk::launch_bi_step<T>(sc->st, g, gp, val, b, r, p, v, t, d, sc->bi_part, st, &sc->launches);
+            prof_end(sc, pi, 2);
+            CK(cudaMemcpyAsync(slot(k), st, sizeof(*st), cudaMemcpyDeviceToHost, sc->st), "d2h");
+            CK(cudaEventRecord(sc->bi_ev[k & 1], sc->st), "event");
         }
-        if (c == 0) continue;
-        CK(cudaEventSynchronize(sc->bi_ev[(c - 1) & 1]), "sync");
-        if (slot(c - 1)->done || c == chunks) {
-            const tk::BiState<T> e = *slot(c - 1);
+        if (k == 0) continue;
+        CK(cudaEventSynchronize(sc->bi_ev[(k - 1) & 1]), "sync");
+        if (slot(k - 1)->done || k == maxit) {
+            const tk::BiState<T> e = *slot(k - 1);
             ss.iters += e.steps;
             if (!std::isfinite((double)e.rn)) return TURSCA_OK;
             break;

@@ -666,11 +666,12 @@ void launch_finalize(cudaStream_t st, const double *part, int nblk, double *out)
 // BiCGStab pass by pass, for scenes too large for the persistent solve.  A
 // step is two passes over K (OpBi), each followed by the sums of its dot
 // products and one vector kernel; the step's scalars stay on the device
-// (every block of the vector kernels forms them from the sums), so steps are
-// queued ahead of the host, which only reads back the state every few steps.
+// (every block of the vector kernels forms them from the sums), so a step is
+// queued before the host has read back the state of the one before.
 // Against GMRES(30) with I + K as preconditioner it needs no basis: on the
 // 128 x 128 x 40 cloud an Arnoldi step spent 107 us on orthogonalisation beside
-// its two passes of 72 us; a step of this takes 130 us, two passes of 57 us (64 with cold caches).
+// its two passes of 72 us; a step of this takes 140 us inside a scene's solve, its passes 57 us each with
+// what L2 keeps of K (64 with cold caches).
 constexpr int kBiParts = 8;  // blocks per sum
 template <typename T>
 __global__ void __launch_bounds__(512) k_bi_sums(const double *__restrict__ part, size_t stride, int n,
@@ -884,7 +885,11 @@ void launch_bi_step(cudaStream_t st, const GridC &g, const GraphP &gp, const T *
                     T *t, T *d, double *part, BiState<T> *state, long long *launches) {
     const int n = (int)g.npad, np = sweep_blocks(g);
     double *sums = part + (size_t)5 * np;
-    const int nb = std::max(1, std::min((n / 4 + 255) / 256, 1216));  // at most 8 blocks on each of 152 SMs
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+        nsm = 152;
+    const int nb = std::max(1, std::min((n / 4 + 255) / 256, 8 * nsm));  // at most 8 blocks per SM
     auto go = [&](auto kern, dim3 blocks, int threads, auto... args) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = blocks;

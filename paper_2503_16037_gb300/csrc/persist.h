@@ -1,6 +1,6 @@
 // The persistent solve (kernels_persist.cu): one cooperative launch solves
 // (I - K) x = s from the source to the refined solution, for scenes whose
-// values stay on the chip (shared memory and registers) and in L2.
+// values stay on the chip (shared memory) and in L2.
 #pragma once
 
 #include <cuda_runtime.h>
