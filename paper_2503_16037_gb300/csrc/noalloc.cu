@@ -117,21 +117,21 @@ __global__ void k_na_final(const double *__restrict__ part, int nb, double *__re
 // barrier per sweep.  A block whose rows reach too far for a window keeps as
 // much of it as shared memory holds and gathers the rest from global memory;
 // with all gathers from there 100,000 rows of 62 to 124 entries in any column
-// took 6,600 us, now 4,010 (a launch per sweep, whose L1 holds more of v: 3,500).
+// took 6,600 us, now 4,130 (a launch per sweep, whose L1 holds more of v: 3,500).
 //
 // Kept rows are packed to whole quads (zeros that gather a zero), so a lane takes four
 // entries per step with two loads of values and indices; 8 lanes (32 in blocks
 // whose rows average more than 256 entries) share a row.  80 sweeps over the 65,536
 // rows: 2010 us with a launch per sweep, 1159 us in one launch entry by entry
 // (a warp per row, bound by its 47 instructions per 32 entries), 1085 us packed,
-// 1065 us as here (streamed rows read in whole 32-byte sectors).
+// 1045 us as here (streamed rows read in whole 32-byte sectors).
 //
 // The line at kNsMaxNodes is one on rows because the number of entries is not
 // known to the host.  Both sides, 80 sweeps, one launch against a launch per
-// sweep, us: 2,000 rows of 10 to 20 entries 222 / 380; 131,072 of 62 to 124
-// 1,840 / 3,930; 131,072 of 150 to 300 (236 MB) 5,650 / 5,780; 65,536 of 500 to
-// 1,000 (393 MB) 7,430 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
-// either way, and static shares end unevenly) 14,620 / 13,380.
+// sweep, us: 2,000 rows of 10 to 20 entries 217 / 380; 131,072 of 62 to 124
+// 1,821 / 3,930; 131,072 of 150 to 300 (236 MB) 6,000 / 5,780; 65,536 of 500 to
+// 1,000 (393 MB) 7,550 / 7,170; 131,072 of 500 to 1,000 (786 MB, HBM-bound
+// either way, and static shares end unevenly) 14,900 / 13,380.
 constexpr int kNsThreads = 1024, kNsWarps = kNsThreads / 32;
 constexpr int kNsMaxRows = 4096;     // rows a block may keep
 constexpr int kNsMaxNodes = 131072;  // above this a launch per sweep
@@ -161,7 +161,8 @@ __device__ __forceinline__ E ns_ld(const E *p, unsigned long long policy) {
 enum { NS_ALL = 0, NS_SOME = 1, NS_NONE = 2 };  // columns that a pass finds in shared memory
 
 constexpr int kNsL2Entries = 10000000;  // 80 MB, what L2 keeps of a set that is read over and over (65,536 rows of
-                                        // 500 to 1,000 entries: 7,760 us without the policies)
+                                        // 500 to 1,000 entries: 7,760 us without the policies, 7,360 with them when
+                                        // they came)
 
 struct NsArgs {
     int n, sweeps, refinements, smem;
@@ -191,8 +192,19 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         }
         sh_r[tid] = blk + tid == nb ? n : lo;
     }
+    if (tid == 0) sh_nch = 0;
     __syncthreads();
     const int r0 = sh_r[0], r1 = sh_r[1], e0 = rp[r0], ne = rp[r1] - e0;
+    // long rows: more than `chunk` entries streamed, more than klong kept
+    const bool wide = ne > 256ll * (r1 - r0);
+    int chunk = wide ? kNsLongWide : kNsLong;
+    auto count = [&]() {  // the chunks of all long rows
+        for (int r = r0 + tid; r < r1; r += kNsThreads) {
+            const int len = __ldg(rp + r + 1) - __ldg(rp + r);
+            if (len > chunk) atomicAdd(&sh_nch, (len - 1) / chunk + 1);
+        }
+    };
+    count();
     // the window: the smallest and largest column, as offsets from r0 modulo n
     int mn = 0x7fffffff, mx = -0x7fffffff;
     for (int e = tid; e < ne; e += kNsThreads) {
@@ -226,7 +238,7 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     // columns of v in shared memory: all of them; or, beside no entries, as many
     // as fit, around the block's own rows, where its entries are enough to pay
     // for the copy (100,000 rows of 20 to 40 entries, 20 thousand a block, 2,277 us
-    // without and 1,820 with it; of 30 to 60 3,317 and 2,383)
+    // without and 1,854 with it; of 30 to 60 3,317 and 2,424)
     int wv = W;
     if (!win4) {
         wv = ne > W / 8 ? min(W, (A.smem - 64) / 4) : 0;
@@ -248,21 +260,15 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         d += d < 0 ? n : 0;
         return d;
     };
-    const bool wide = ne > 256ll * (r1 - r0);
-    // long rows: more than `chunk` entries streamed, more than klong kept; the
-    // chunk that lets the block list all of its chunks
-    int chunk = wide ? kNsLongWide : kNsLong;
-    for (;; chunk *= 2) {
+    while (sh_nch > kNsChunks) {  // longer chunks, until the block can list all of them
+        chunk *= 2;
         __syncthreads();
         if (tid == 0) sh_nch = 0;
         __syncthreads();
-        for (int r = r0 + tid; r < r1; r += kNsThreads) {
-            const int len = __ldg(rp + r + 1) - __ldg(rp + r);
-            if (len > chunk) atomicAdd(&sh_nch, (len - 1) / chunk + 1);
-        }
+        count();
         __syncthreads();
-        if (sh_nch <= kNsChunks) break;
     }
+    int nch = sh_nch;
     const int klong = max(chunk, kNsLongKept);
     int kept = 0;  // rows [r0, r0 + kept), the long ones among them left out
     if (capq > 0) {
@@ -308,26 +314,22 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
     }
     // the list of the long rows' chunks (no more than were counted: klong >= chunk)
     auto longest = [&](int row) { return row < r0 + kept ? klong : chunk; };
-    if (tid == 0) sh_nch = 0;
-    __syncthreads();
-    for (int r = r0 + tid; r < r1; r += kNsThreads) {
-        const int p = __ldg(rp + r), len = __ldg(rp + r + 1) - p;
-        if (len <= longest(r)) continue;
-        const int nc = (len - 1) / chunk + 1, c0 = atomicAdd(&sh_nch, nc);
-        for (int c = 0; c < nc; ++c) {
-            sh_crow[c0 + c] = r;
-            sh_cst[c0 + c] = p + c * chunk;
+    if (nch > 0) {
+        __syncthreads();
+        if (tid == 0) sh_nch = 0;
+        __syncthreads();
+        for (int r = r0 + tid; r < r1; r += kNsThreads) {
+            const int p = __ldg(rp + r), len = __ldg(rp + r + 1) - p;
+            if (len <= longest(r)) continue;
+            const int nc = (len - 1) / chunk + 1, c0 = atomicAdd(&sh_nch, nc);
+            for (int c = 0; c < nc; ++c) {
+                sh_crow[c0 + c] = r;
+                sh_cst[c0 + c] = p + c * chunk;
+            }
         }
+        __syncthreads();
+        nch = sh_nch;
     }
-    __syncthreads();
-    const int nch = sh_nch;
-    // Entries streamed beyond what L2 holds for all blocks leave it first, so
-    // that they do not push the others out.
-    unsigned long long near_by, pass_by;
-    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(near_by));
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
-    const int streamed = r0 + kept < r1 ? __ldg(rp + r0 + kept) : e0 + ne;  // the first streamed entry
-    const int near_end = e0 + ne - streamed <= kNsL2Entries / nb * 11 / 10 ? 0x7fffffff : streamed + kNsL2Entries / nb;
     unsigned gen = 0;
     auto barrier = [&]() -> bool {
         ++gen;
@@ -348,163 +350,187 @@ __global__ void __launch_bounds__(kNsThreads, 1) k_na_solve(const __grid_constan
         __syncthreads();
         return sh_ok != 0;
     };
-    // Every row's sum over its entries of val times the gathered vector (from
-    // the kept entries; else from L2, with the window's `width` columns in
-    // shared memory and the others in global memory),
-    // handed to out(row, sum) in one lane of the row's L lanes.  The rows that
-    // are not kept go first: their loads take longest.  Long rows are skipped
-    // (long_rows).
-    auto rows = [&](auto lanes_c, auto mode_c, auto zero, const auto *vec, const auto *window, int width, auto out) {
-        constexpr int L = decltype(lanes_c)::value, MODE = decltype(mode_c)::value;
-        using V = decltype(zero);
-        const int sl = lane & (L - 1), first = tid / 32 * (32 / L) + lane / L, lanes = kNsThreads / L;
-        auto get = [&](int c) {
-            if constexpr (MODE == NS_NONE) return vec[c];
-            const int d = local(c);
-            if constexpr (MODE == NS_ALL) return window[d];
-            return d < width ? window[d] : vec[c];
-        };
-        auto sum = [&](V acc, int row, bool on) {
-            __syncwarp();
+    // Entries streamed beyond what L2 holds for all blocks leave it first, so
+    // that they do not push the others out.
+    unsigned long long near_by, pass_by;
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(near_by));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pass_by));
+    const int streamed = wide && r0 + kept < r1 ? __ldg(rp + r0 + kept) : e0 + ne;  // the first streamed entry
+    const int near_end = e0 + ne - streamed <= kNsL2Entries / nb * 11 / 10 ? 0x7fffffff : streamed + kNsL2Entries / nb;
+    // The refinements.  Blocks with a whole window, no long rows and 8 lanes to a
+    // row have code of their own: the tests and the registers of the others cost
+    // their sweeps 2 to 3 %.
+    auto refine = [&](auto general_c) {
+        constexpr bool GENERAL = decltype(general_c)::value;
+        // Every row's sum over its entries of val times the gathered vector (from
+        // the kept entries; else from L2, with the window's `width` columns in
+        // shared memory and the others in global memory),
+        // handed to out(row, sum) in one lane of the row's L lanes.  The rows that
+        // are not kept go first: their loads take longest.  Long rows are skipped
+        // (long_rows).
+        auto rows = [&](auto lanes_c, auto mode_c, auto zero, const auto *vec, const auto *window, int width, auto out) {
+            constexpr int L = decltype(lanes_c)::value, MODE = decltype(mode_c)::value;
+            using V = decltype(zero);
+            const int sl = lane & (L - 1), first = tid / 32 * (32 / L) + lane / L, lanes = kNsThreads / L;
+            auto get = [&](int c) {
+                if constexpr (MODE == NS_NONE) return vec[c];
+                const int d = local(c);
+                if constexpr (MODE == NS_ALL) return window[d];
+                return d < width ? window[d] : vec[c];
+            };
+            auto sum = [&](V acc, int row, bool on) {
+                __syncwarp();
 #pragma unroll
-            for (int o = L / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (sl == 0 && on) out(row, acc);
-        };
-        const int k0 = MODE == NS_ALL ? kept : 0;
-        for (int b = r0 + k0; b < r1; b += lanes) {
-            const int row = b + first;
-            int p = 0, end = 0;
-            if (row < r1) {
-                p = __ldg(rp + row);
-                end = __ldg(rp + row + 1);
-            }
-            const bool on = row < r1 && end - p <= (MODE == NS_ALL ? chunk : longest(row));
-            if (!on) end = p;
-            V acc = zero;
-            constexpr int U = sizeof(V) == 4 ? 6 : 4;
-            // (a policy operand costs matrices that stay in L2 2 to 4 %: wide rows only)
-            const unsigned long long policy = p < near_end ? near_by : pass_by;
-            for (int e = (p & ~7) + sl; e < end; e += U * L) {  // the lanes' 8 or 32 entries in whole sectors
-                float v[U];
-                int c[U];
+                for (int o = L / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (sl == 0 && on) out(row, acc);
+            };
+            const int k0 = MODE == NS_ALL ? kept : 0;
+            for (int b = r0 + k0; b < r1; b += lanes) {
+                const int row = b + first;
+                const bool in_block = row < r1;
+                const int p = in_block ? __ldg(rp + row) : 0, row_end = in_block ? __ldg(rp + row + 1) : 0;
+                const bool is_long = GENERAL && nch > 0 && row_end - p > (MODE == NS_ALL ? chunk : longest(row));
+                const bool on = in_block && !is_long;
+                const int end = is_long ? p : row_end;
+                V acc = zero;
+                constexpr int U = sizeof(V) == 4 ? 6 : 4;
+                // (a policy operand costs matrices that stay in L2 2 to 4 %: wide rows only)
+                const unsigned long long policy = p < near_end ? near_by : pass_by;
+                const int start = sizeof(V) == 4 ? p & ~7 : p;  // sweeps: the lanes' 8 or 32 entries in whole sectors
+                for (int e = start + sl; e < end; e += U * L) {
+                    float v[U];
+                    int c[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const bool in = e + u * L < end && (u > 0 || e >= p);
-                    v[u] = in ? ns_ld<L == 32>(A.val + e + u * L, policy) : 0.f;
-                    c[u] = in ? ns_ld<L == 32>(A.col + e + u * L, policy) : -1;
+                    for (int u = 0; u < U; ++u) {
+                        const bool in = e + u * L < end && (u > 0 || e >= p);
+                        v[u] = in ? ns_ld<L == 32>(A.val + e + u * L, policy) : 0.f;
+                        c[u] = in ? ns_ld<L == 32>(A.col + e + u * L, policy) : -1;
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (c[u] >= 0) acc += (V)v[u] * get(c[u]);
                 }
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (c[u] >= 0) acc += (V)v[u] * get(c[u]);
+                sum(acc, row, on);
             }
-            sum(acc, row, on);
-        }
-        for (int b = 0; b < k0; b += lanes) {
-            const int r = b + first;
-            const unsigned s0 = r < k0 ? srow[r] : 0u, s1 = r < k0 ? srow[r + 1] : kNsIsLong;
-            const bool on = !(s1 & kNsIsLong);
-            const int q0 = s0 & (kNsIsLong - 1), q1 = on ? s1 : q0;
-            V acc = zero;
+            for (int b = 0; b < k0; b += lanes) {
+                const int r = b + first;
+                bool on = r < k0;
+                int q0 = on ? srow[r] : 0, q1 = on ? srow[r + 1] : 0;
+                if constexpr (GENERAL) {
+                    on = on && !(q1 & kNsIsLong);
+                    q0 &= kNsIsLong - 1;
+                    q1 = on ? q1 : q0;
+                }
+                V acc = zero;
 #pragma unroll 2
-            for (int q = q0 + sl; q < q1; q += L) {
-                const float4 v = sval[q];
-                const uint2 ix = sidx[q];
-                acc += (V)v.x * window[ix.x & 0xffffu];
-                acc += (V)v.y * window[ix.x >> 16];
-                acc += (V)v.z * window[ix.y & 0xffffu];
-                acc += (V)v.w * window[ix.y >> 16];
+                for (int q = q0 + sl; q < q1; q += L) {
+                    const float4 v = sval[q];
+                    const uint2 ix = sidx[q];
+                    acc += (V)v.x * window[ix.x & 0xffffu];
+                    acc += (V)v.y * window[ix.x >> 16];
+                    acc += (V)v.z * window[ix.y & 0xffffu];
+                    acc += (V)v.w * window[ix.y >> 16];
+                }
+                sum(acc, r0 + r, on);
             }
-            sum(acc, r0 + r, on);
-        }
-    };
-    auto long_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
-        using V = decltype(zero);
-        for (int c = w; c < nch; c += kNsWarps) {
-            const int p = sh_cst[c], re = __ldg(rp + sh_crow[c] + 1), end = re - p > chunk ? p + chunk : re;
-            V acc = zero;
-#pragma unroll 8
-            for (int e = p + lane; e < end; e += 32) {
-                const int k = __ldg(A.col + e), d = local(k);
-                acc += (V)__ldg(A.val + e) * (d < width ? window[d] : vec[k]);
-            }
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) sh_csum[c] = (double)acc;
-        }
-        __syncthreads();
-        for (int c = tid; c < nch; c += kNsThreads) {
-            const int row = sh_crow[c], p = __ldg(rp + row), len = __ldg(rp + row + 1) - p;
-            if (sh_cst[c] != p) continue;  // not the row's first
-            V t = zero;
-            for (int k = 0; k <= (len - 1) / chunk; ++k) t += (V)sh_csum[c + k];
-            out(row, t);
-        }
-        __syncthreads();  // sh_csum
-    };
-    auto all_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
-        if (nch > 0) long_rows(zero, vec, window, width, out);
-        auto go = [&](auto mode_c) {
-            if (wide) rows(std::integral_constant<int, 32>(), mode_c, zero, vec, window, width, out);
-            else rows(std::integral_constant<int, 8>(), mode_c, zero, vec, window, width, out);
         };
-        if (width == W) return go(std::integral_constant<int, NS_ALL>());
-        if constexpr (sizeof(zero) == 4)
-            if (width > 0) return go(std::integral_constant<int, NS_SOME>());
-        go(std::integral_constant<int, NS_NONE>());
+        auto long_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
+            using V = decltype(zero);
+            for (int c = w; c < nch; c += kNsWarps) {
+                const int p = sh_cst[c], re = __ldg(rp + sh_crow[c] + 1), end = re - p > chunk ? p + chunk : re;
+                V acc = zero;
+#pragma unroll 8
+                for (int e = p + lane; e < end; e += 32) {
+                    const int k = __ldg(A.col + e), d = local(k);
+                    acc += (V)__ldg(A.val + e) * (d < width ? window[d] : vec[k]);
+                }
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) sh_csum[c] = (double)acc;
+            }
+            __syncthreads();
+            for (int c = tid; c < nch; c += kNsThreads) {
+                const int row = sh_crow[c], p = __ldg(rp + row), len = __ldg(rp + row + 1) - p;
+                if (sh_cst[c] != p) continue;  // not the row's first
+                V t = zero;
+                for (int k = 0; k <= (len - 1) / chunk; ++k) t += (V)sh_csum[c + k];
+                out(row, t);
+            }
+            __syncthreads();  // sh_csum
+        };
+        auto all_rows = [&](auto zero, const auto *vec, const auto *window, int width, auto out) {
+            if constexpr (GENERAL) {
+                if (nch > 0) long_rows(zero, vec, window, width, out);
+                auto go = [&](auto mode_c) {
+                    if (wide) rows(std::integral_constant<int, 32>(), mode_c, zero, vec, window, width, out);
+                    else rows(std::integral_constant<int, 8>(), mode_c, zero, vec, window, width, out);
+                };
+                if (width == W) return go(std::integral_constant<int, NS_ALL>());
+                if constexpr (sizeof(zero) == 4)
+                    if (width > 0) return go(std::integral_constant<int, NS_SOME>());
+                go(std::integral_constant<int, NS_NONE>());
+            } else {
+                constexpr std::integral_constant<int, 8> lanes_c{};
+                if (sizeof(zero) == 4 || width == W) rows(lanes_c, std::integral_constant<int, NS_ALL>(), zero, vec, window, width, out);
+                else rows(lanes_c, std::integral_constant<int, NS_NONE>(), zero, vec, window, width, out);
+            }
+        };
+        bool ok = true;
+        for (int r = 0; ok && r < A.refinements; ++r) {
+            if (win4 && tid == 0) win[W] = 0.f;  // (where x's window lay meanwhile)
+            const float *cur = A.b;
+            for (int k = 0; ok && k < A.sweeps; ++k) {
+                float *nxt = (k & 1) ? A.d1 : A.d0;
+                if (wv > 0) {
+#pragma unroll 8
+                    for (int j = tid; j < wv; j += kNsThreads) {
+                        const int g = w0 + j;
+                        win[j] = __ldcg(cur + (g >= n ? g - n : g));
+                    }
+                    __syncthreads();
+                }
+                all_rows(0.f, cur, win, wv, [&](int row, float v) { nxt[row] = A.b[row] + v; });
+                cur = nxt;
+                ok = barrier();
+            }
+            if (!ok) break;
+            for (int i = r0 + tid; i < r1; i += kNsThreads) A.x[i] += (double)cur[i];
+            ok = barrier();
+            if (!ok) break;
+            if (win8) {
+#pragma unroll 4
+                for (int j = tid; j < W; j += kNsThreads) {
+                    const int g = w0 + j;
+                    winx[j] = __ldcg(A.x + (g >= n ? g - n : g));
+                }
+                __syncthreads();
+            }
+            double loc = 0.0;
+            all_rows(0.0, A.x, winx, wx, [&](int row, double v) {
+                const double res = (double)A.s[row] - A.x[row] + v;
+                A.b[row] = (float)res;
+                loc += res * res;
+            });
+            if (r == A.refinements - 1 && A.resid2) {
+                for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+                if (lane == 0) sh_red[w] = loc;
+                __syncthreads();
+                if (tid == 0) {
+                    double t = 0.0;
+                    for (int q = 0; q < kNsWarps; ++q) t += sh_red[q];
+                    A.part[blk] = t;
+                }
+            }
+            if (r + 1 < A.refinements || A.resid2) ok = barrier();
+        }
+        return ok;
     };
-    bool ok = true;
     for (int i = r0 + tid; i < r1; i += kNsThreads) {
         A.x[i] = 0.0;
         A.b[i] = A.s[i];
     }
-    ok = barrier();
+    bool ok = barrier();
     if (win8 && tid == 0) winx[W] = 0.0;
-    for (int r = 0; ok && r < A.refinements; ++r) {
-        if (win4 && tid == 0) win[W] = 0.f;  // (where x's window lay meanwhile)
-        const float *cur = A.b;
-        for (int k = 0; ok && k < A.sweeps; ++k) {
-            float *nxt = (k & 1) ? A.d1 : A.d0;
-            if (wv > 0) {
-#pragma unroll 8
-                for (int j = tid; j < wv; j += kNsThreads) {
-                    const int g = w0 + j;
-                    win[j] = __ldcg(cur + (g >= n ? g - n : g));
-                }
-                __syncthreads();
-            }
-            all_rows(0.f, cur, win, wv, [&](int row, float v) { nxt[row] = A.b[row] + v; });
-            cur = nxt;
-            ok = barrier();
-        }
-        if (!ok) break;
-        for (int i = r0 + tid; i < r1; i += kNsThreads) A.x[i] += (double)cur[i];
-        ok = barrier();
-        if (!ok) break;
-        if (win8) {
-#pragma unroll 4
-            for (int j = tid; j < W; j += kNsThreads) {
-                const int g = w0 + j;
-                winx[j] = __ldcg(A.x + (g >= n ? g - n : g));
-            }
-            __syncthreads();
-        }
-        double loc = 0.0;
-        all_rows(0.0, A.x, winx, wx, [&](int row, double v) {
-            const double res = (double)A.s[row] - A.x[row] + v;
-            A.b[row] = (float)res;
-            loc += res * res;
-        });
-        if (r == A.refinements - 1 && A.resid2) {
-            for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
-            if (lane == 0) sh_red[w] = loc;
-            __syncthreads();
-            if (tid == 0) {
-                double t = 0.0;
-                for (int q = 0; q < kNsWarps; ++q) t += sh_red[q];
-                A.part[blk] = t;
-            }
-        }
-        if (r + 1 < A.refinements || A.resid2) ok = barrier();
-    }
+    if (ok) ok = wv == W && nch == 0 && !wide ? refine(std::false_type()) : refine(std::true_type());
     if (!ok) {  // a barrier gave up (the launch is cooperative, so none should): no half result
         for (int i = r0 + tid; i < r1; i += kNsThreads) A.x[i] = __longlong_as_double(0x7ff8000000000000ll);
     }
