@@ -12,7 +12,7 @@
 // mapping changes from pass to pass (both dies then keep copies).
 //
 // Why BiCGStab.  It takes two products per step and no spectrum estimate: on
-// the plume 36 products in 2 refinements against 38 in 3 (4 sweeps and 30
+// the plume 32 products in 2 refinements against 38 in 3 (4 sweeps and 30
 // Chebyshev steps), on scenes where the interval was missed and GMRES took
 // over 50 against 62 with 10 Arnoldi steps' host round trips.  Each block
 // keeps r and p on its rows and on every node its rows gather from (its tile,
@@ -24,8 +24,8 @@
 // (4 for the values, 4 for the gathers; 3.6 us for 7 groups), then the
 // exchange.  Measured on the plume, per step of two products: 6.4 and 6.6 us
 // of products, 1.5 and 2.0 us of barriers, 1.5 and 2.7 us of vector updates.
-// Whole solve 444 us (plume), 400 us (random 45 x 37 x 29: 1160 us with passes
-// and GMRES), 115 us (plume 16^3), about 1.1 ms (96 x 96 x 32, 150 MB of values
+// Whole solve 373 us (plume), 395 us (random 45 x 37 x 29: 1160 us with passes
+// and GMRES), 120 us (plume 16^3), 1.2 ms (96 x 96 x 32, 150 MB of values
 // of which L2 keeps 80).  FP64 is kept off the common path of FP32
 // scenes (an FP64 warp operation takes 16 issue slots of the SM): dot products
 // are FP32 pairs, 48 bits, and the outer loop's scalars are one thread's.
