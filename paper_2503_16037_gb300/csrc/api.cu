@@ -998,6 +998,7 @@ tursca_status persist_launch(tursca_scene *sc, const SolveIO<T> &io, double rtol
     J.part = sc->ps_part;
     J.bar = (unsigned *)sc->ps_ctl;
     J.status = sc->status;
+    static_assert(64 + sizeof(tk::PsInfo) <= 256, "ps_ctl");
     J.info = (tk::PsInfo *)(sc->ps_ctl + 64);
     J.rtol = rtol;
     J.max_iter = max_iter;

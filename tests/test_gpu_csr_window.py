@@ -64,7 +64,7 @@ def test_wide_windows(name):
 
 def test_gathers_from_anywhere_cost_no_more_than_a_launch_per_sweep():
     """100,000 rows in one launch against 131,073 rows with as many entries,
-    which take a launch per sweep: at most 1.3 times (1.5 with every gather in
+    which take a launch per sweep: at most 1.3 times (1.7 with every gather in
     global memory)."""
     def ms(n, k):
         s = system(n, k, 0)
